@@ -2222,7 +2222,11 @@ struct GraphArgs {
 };
 
 constexpr int GS_WARPS = 4;
-constexpr int GS_N = 128;  // W (<= efs <= 96) plus 32 new keys, sorted together
+constexpr int GS_MAX_EFS = 96;    // result-set capacity: three keys per lane
+constexpr int GS_INSERT_MAX = 8;  // new keys of an expansion inserted one by one (more: sorted and merged)
+// Shared bytes per CTA that bound the list length this search accepts (a
+// visited bit per member and a fixed allowance per warp).
+static size_t gs_smem_bound(int vwords) { return (size_t)GS_WARPS * (2048 + (size_t)vwords * 4); }
 
 // 32 distances of one block for the lane group of the whole warp (G = 32):
 // lane l receives vector l's sum.
@@ -2242,28 +2246,44 @@ __device__ __forceinline__ uint32_t block_sums32(const uint4* __restrict__ cp, c
     return out[0];
 }
 
+// Ascending sort of a bitonic sequence of one key per lane.
+__device__ __forceinline__ uint64_t warp_merge_key(uint64_t v, int lane) {
+#pragma unroll
+    for (int j = 16; j > 0; j >>= 1) {
+        const uint64_t o = __shfl_xor_sync(0xffffffffu, v, j);
+        v = ((lane & j) == 0) == (o < v) ? o : v;
+    }
+    return v;
+}
+
 // One warp per (query, distant list): best-first search of the list's graph
-// with result set W of capacity efs (Sec. 4.4).  W is kept sorted in shared
-// memory with, per entry, its list position and whether it was expanded; an
-// expansion takes the smallest unexpanded entry, computes its 32
-// neighbours' keys with one LUT16 block, marks them visited, and keeps the
-// efs smallest of W and the unvisited neighbours.  The search ends when every
-// entry of W is expanded (equivalently: the best candidate is worse than
-// W's worst once W is full).  Then, with theta the query's threshold: at
-// least tau keys of W below theta -> the list is scanned fully later;
-// otherwise W's keys at or below theta join the candidates.
-template <int SMAX>
+// with result set W of capacity efs (Sec. 4.4).  An expansion takes W's
+// smallest unexpanded entry, computes its 32 neighbours' keys with one LUT16
+// block, marks them visited, and keeps the efs smallest of W and the unvisited
+// neighbours.  The search ends when every entry of W is expanded
+// (equivalently: the best candidate is worse than W's worst once W is full).
+// Then, with theta the query's threshold: at least tau keys of W below theta
+// -> the list is scanned fully later; otherwise W's keys at or below theta
+// join the candidates.
+//
+// W lives in registers, sorted: entry 32 i + lane in W[i].  An entry is one
+// word, distance word << 32 | list position << 1 | expanded: a list's members
+// stand in ascending id, so positions order ties as ids do, and the expanded
+// bit of unique positions changes no order (an empty entry, all ones, reads as
+// expanded).  Ids are looked up once, for the final W.  Only new keys below
+// W's worst can enter: a few of them are inserted one by one (a compare and a
+// shift by one lane), more are sorted across the warp and merged.
+// The kernel is bound by instruction issue: about 450 issue slots per
+// expansion, a third of them the block's lookups.  Sorting W and the new keys
+// together in shared memory took about 4500 (100k x 64, M 32, 2000 queries, 10
+// distant lists each, efs 64: 6.2 ms against 0.51 ms now).
+template <int SMAX, int NR>
 __global__ void __launch_bounds__(GS_WARPS * 32) k_graph_search(ScanArgs A, ScanOut O, GraphArgs Gr,
                                                                 const uint32_t* __restrict__ pairs,
                                                                 const int64_t* __restrict__ npairs) {
-    extern __shared__ __align__(16) uint8_t gsm[];
+    extern __shared__ uint32_t gvis[];  // a visited bit per member, vwords per warp
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const size_t per_warp = (size_t)GS_N * 16 + (size_t)Gr.vwords * 4;
-    uint8_t* base_w = gsm + warp * per_warp;
-    uint64_t* wk = reinterpret_cast<uint64_t*>(base_w);             // keys
-    int32_t* wp = reinterpret_cast<int32_t*>(base_w + GS_N * 8);    // list positions
-    uint32_t* wf = reinterpret_cast<uint32_t*>(base_w + GS_N * 12); // expanded flags
-    uint32_t* vis = reinterpret_cast<uint32_t*>(base_w + GS_N * 16);
+    uint32_t* vis = gvis + (size_t)warp * Gr.vwords;
     const int M = A.M;
     const int64_t n_items = *npairs;
     for (int64_t it = (int64_t)blockIdx.x * GS_WARPS + warp; it < n_items; it += (int64_t)gridDim.x * GS_WARPS) {
@@ -2283,90 +2303,110 @@ __global__ void __launch_bounds__(GS_WARPS * 32) k_graph_search(ScanArgs A, Scan
         const int32_t bias = A.bias[e];
         const uint64_t th = O.thr[q];
         const int64_t slot0 = A.boff[p] * 32;
+        auto entry_of = [&](uint32_t sum, int pos) -> uint64_t {
+            return ((uint64_t)((uint32_t)(bias + (int32_t)sum) ^ 0x80000000u) << 32) | ((uint32_t)pos << 1);
+        };
         for (int w = lane; w < (np_ + 31) / 32; w += 32) vis[w] = 0u;
         __syncwarp();
+        uint64_t W[NR];
+#pragma unroll
+        for (int i = 0; i < NR; ++i) W[i] = KEY_NONE;
         // entry: its block's 32 sums, keep the entry's
         {
             const int64_t gb = A.boff[p] + (ep >> 5);
             const uint32_t sum = block_sums32<SMAX>(reinterpret_cast<const uint4*>(A.codes + gb * M * 16), t, M, lane);
-            if (lane == (ep & 31)) {
-                wk[0] = make_key(bias + (int32_t)sum, A.ids[slot0 + ep]);
-                wp[0] = ep;
-                wf[0] = 0;
+            const uint64_t k = __shfl_sync(0xffffffffu, entry_of(sum, ep), ep & 31);
+            if (lane == 0) {
+                W[0] = k;
                 vis[ep >> 5] = 1u << (ep & 31);
             }
             __syncwarp();
         }
-        int wn = 1;
         for (int guard = 0; guard <= np_; ++guard) {
-            // smallest unexpanded entry of the sorted W
-            int ui = -1;
-            for (int c = 0; c < wn && ui < 0; c += 32) {
-                const bool un = (c + lane < wn) && wf[c + lane] == 0;
-                const unsigned b = __ballot_sync(0xffffffffu, un);
-                if (b) ui = c + __ffs(b) - 1;
+            // smallest unexpanded entry of W
+            int src = -1;
+            uint32_t up = 0;
+#pragma unroll
+            for (int i = 0; i < NR; ++i) {
+                const uint32_t m = __ballot_sync(0xffffffffu, (W[i] & 1ull) == 0ull);
+                if (src < 0 && m) {
+                    src = __ffs(m) - 1;
+                    up = __shfl_sync(0xffffffffu, (uint32_t)W[i], src) >> 1;
+                    if (lane == src) W[i] |= 1ull;
+                }
             }
-            if (ui < 0) break;
-            const int upos = wp[ui];
-            __syncwarp();
-            if (lane == 0) wf[ui] = 1;
+            if (src < 0) break;
             // expand: the 32 neighbours' keys in one block
-            const int64_t su = slot0 + upos;
+            const int64_t su = slot0 + up;
+            const int pe = Gr.nbr_pos[su * 32 + lane];
             const uint32_t sum =
                 block_sums32<SMAX>(reinterpret_cast<const uint4*>(Gr.nbr_codes + su * M * 16), t, M, lane);
-            const int pe = Gr.nbr_pos[su * 32 + lane];
             uint64_t kn = KEY_NONE;
             if (pe >= 0) {
                 const uint32_t bit = 1u << (pe & 31);
                 const uint32_t old = atomicOr(&vis[pe >> 5], bit);
-                if (!(old & bit)) kn = make_key(bias + (int32_t)sum, A.ids[slot0 + pe]);
+                if (!(old & bit)) kn = entry_of(sum, pe);
             }
-            wk[wn + lane] = kn;
-            wp[wn + lane] = pe;
-            wf[wn + lane] = 0;
-            // sort W and the new keys together; keep the efs smallest
-            const int N = wn + 32;
-            const int S = N <= 64 ? 64 : GS_N;
-            for (int i = N + lane; i < S; i += 32) wk[i] = KEY_NONE;
-            __syncwarp();
-            for (int k2 = 2; k2 <= S; k2 <<= 1)
-                for (int j = k2 >> 1; j > 0; j >>= 1) {
-                    for (int i = lane; i < S; i += 32) {
-                        const int ixj = i ^ j;
-                        if (ixj > i) {
-                            const uint64_t a = wk[i], b2 = wk[ixj];
-                            const bool up = (i & k2) == 0;
-                            if ((a > b2) == up) {
-                                wk[i] = b2;
-                                wk[ixj] = a;
-                                const int32_t tp = wp[i];
-                                wp[i] = wp[ixj];
-                                wp[ixj] = tp;
-                                const uint32_t tf = wf[i];
-                                wf[i] = wf[ixj];
-                                wf[ixj] = tf;
-                            }
-                        }
+            // only keys below W's last entry (all ones until W is full) can enter
+            uint64_t worst = KEY_NONE;
+#pragma unroll
+            for (int i = 0; i < NR; ++i)
+                if ((Gr.efs - 1) >> 5 == i) worst = __shfl_sync(0xffffffffu, W[i], (Gr.efs - 1) & 31);
+            if (kn >= worst) kn = KEY_NONE;
+            uint32_t m = __ballot_sync(0xffffffffu, kn != KEY_NONE);
+            if (!m) continue;
+            if (__popc(m) <= GS_INSERT_MAX) {
+                while (m) {
+                    const uint64_t k = __shfl_sync(0xffffffffu, kn, __ffs(m) - 1);
+                    m &= m - 1u;
+                    // entries above k move up by one place, k takes the first of theirs
+#pragma unroll
+                    for (int i = NR - 1; i >= 0; --i) {
+                        uint64_t prev = __shfl_up_sync(0xffffffffu, W[i], 1);
+                        const uint64_t below = i > 0 ? __shfl_sync(0xffffffffu, W[i > 0 ? i - 1 : 0], 31) : 0ull;
+                        if (lane == 0) prev = below;
+                        if (W[i] > k) W[i] = prev > k ? prev : k;
                     }
-                    __syncwarp();
                 }
-            int valid = 0;
-            for (int c = 0; c < S; c += 32) valid += __popc(__ballot_sync(0xffffffffu, c + lane < S && wk[c + lane] != KEY_NONE));
-            wn = min(valid, Gr.efs);
+            } else {
+                // from the top 32 entries down: of W[i] and the new keys, the 32
+                // largest are final (those past the last register drop out), the
+                // 32 smallest go on against W[i - 1]
+                uint64_t N = warp_sort_key(kn, lane);
+#pragma unroll
+                for (int i = NR - 1; i >= 0; --i) {
+                    const uint64_t r = __shfl_sync(0xffffffffu, N, 31 - lane);
+                    const uint64_t lo = r < W[i] ? r : W[i], hi = r < W[i] ? W[i] : r;
+                    if (i + 1 < NR) W[i + 1 < NR ? i + 1 : 0] = warp_merge_key(hi, lane);
+                    N = warp_merge_key(lo, lane);
+                }
+                W[0] = N;
+            }
+#pragma unroll
+            for (int i = 0; i < NR; ++i)
+                if (32 * i + lane >= Gr.efs) W[i] = KEY_NONE;
         }
         // decide: full scan later, or W's keys join the candidates
         int good = 0;
-        for (int c = 0; c < wn; c += 32) good += __popc(__ballot_sync(0xffffffffu, c + lane < wn && wk[c + lane] < th));
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            // the entry as a candidate key: its id in place of its position
+            if (W[i] != KEY_NONE)
+                W[i] = (W[i] & 0xffffffff00000000ull) | (uint32_t)A.ids[slot0 + ((uint32_t)W[i] >> 1)];
+            good += __popc(__ballot_sync(0xffffffffu, W[i] < th && W[i] != KEY_NONE));
+        }
         if (good >= Gr.tau) {
             if (lane == 0) Gr.full_pairs[atomicAdd(reinterpret_cast<unsigned long long*>(Gr.nfull), 1ull)] = e;
         } else {
-            for (int c = 0; c < wn; c += 32) {
-                const bool keep = c + lane < wn && wk[c + lane] <= th;
+#pragma unroll
+            for (int i = 0; i < NR; ++i) {
+                const bool keep = W[i] != KEY_NONE && W[i] <= th;
                 const unsigned b = __ballot_sync(0xffffffffu, keep);
+                if (!b) continue;
                 int base = 0;
-                if (lane == 0 && b) base = atomicAdd(&O.cnt[q], __popc(b));
+                if (lane == 0) base = atomicAdd(&O.cnt[q], __popc(b));
                 base = __shfl_sync(0xffffffffu, base, 0) + __popc(b & ((1u << lane) - 1u));
-                if (keep && base < O.cap) O.cand[q * O.cap + base] = wk[c + lane];
+                if (keep && base < O.cap) O.cand[q * O.cap + base] = W[i];
             }
         }
         __syncwarp();
@@ -3440,6 +3480,35 @@ static int ensure_band(ksc_index* ix, cudaStream_t st) {
     return KSC_OK;
 }
 
+template <int SMAX, int NR>
+static int launch_graph_search_t(const ScanArgs& A, const ScanOut& O, const GraphArgs& Gr, const uint32_t* pairs,
+                                 const int64_t* npairs, cudaStream_t st) {
+    const size_t smem = sizeof(uint32_t) * GS_WARPS * (size_t)Gr.vwords;
+    auto kern = k_graph_search<SMAX, NR>;
+    KSC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int per_sm = 0;
+    KSC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, GS_WARPS * 32, smem));
+    kern<<<num_sms() * (per_sm > 0 ? per_sm : 1), GS_WARPS * 32, smem, st>>>(A, O, Gr, pairs, npairs);
+    KSC_LAUNCH_CHECK();
+    return KSC_OK;
+}
+
+// The graph search with as many subspaces and result entries per lane as M
+// and efs need.
+static int launch_graph_search(const ScanArgs& A, const ScanOut& O, const GraphArgs& Gr, const uint32_t* pairs,
+                               const int64_t* npairs, cudaStream_t st) {
+    const int sg = (A.M + 31) / 32, nr = (Gr.efs + 31) / 32;
+#define KSC_GS(SM)                                                                            \
+    (nr <= 1 ? launch_graph_search_t<SM, 1>(A, O, Gr, pairs, npairs, st)                      \
+             : (nr == 2 ? launch_graph_search_t<SM, 2>(A, O, Gr, pairs, npairs, st)           \
+                        : launch_graph_search_t<SM, 3>(A, O, Gr, pairs, npairs, st)))
+    if (sg <= 1) return KSC_GS(1);
+    if (sg <= 2) return KSC_GS(2);
+    if (sg <= 4) return KSC_GS(4);
+    return KSC_GS(8);
+#undef KSC_GS
+}
+
 // Cluster-major work list of the (query, rank) pairs of one part of the probe
 // ranks (the unfiltered first part or the rest).
 struct WorkList {
@@ -3603,23 +3672,11 @@ static int search_from_probes(ksc_index* ix, const float* Q, const Plan& pl, con
         int64_t* nfull = (int64_t*)ix->ws_full.p;
         uint32_t* full = (uint32_t*)(nfull + 2);
         KSC_CUDA(cudaMemsetAsync(nfull, 0, sizeof(int64_t), st));
-        const int vwords = (((ix->max_list + 31) / 32) + 1) & ~1;  // even: keeps every warp's keys 8-byte aligned
+        const int vwords = (((ix->max_list + 31) / 32) + 1) & ~1;
         GraphArgs Gr{ix->nbr_pos, ix->nbr_codes, ix->entry_pos, pl.efs, pl.tau, vwords, full, nfull};
-        const size_t smem = (size_t)GS_WARPS * ((size_t)GS_N * 16 + (size_t)vwords * 4);
-        KSC_CHECK_ARG(smem <= 200 * 1024, "lists too large for the hybrid search (%d members)", ix->max_list);
-        const int Sg = (M + 31) / 32;
-        const int grid = num_sms() * 8;
-        const ScanOut Og{thr, cnt, cand, pl.cap};
-#define KSC_GS(SM)                                                                                        \
-    do {                                                                                                  \
-        KSC_CUDA(cudaFuncSetAttribute(k_graph_search<SM>, cudaFuncAttributeMaxDynamicSharedMemorySize,     \
-                                      (int)smem));                                                        \
-        k_graph_search<SM><<<grid, GS_WARPS * 32, smem, st>>>(A, Og, Gr, wb.pairs, wb.pair_off + L);      \
-    } while (0)
-        if (Sg <= 2) KSC_GS(2);
-        else if (Sg <= 4) KSC_GS(4);
-        else KSC_GS(8);
-#undef KSC_GS
+        KSC_CHECK_ARG(gs_smem_bound(vwords) <= 200 * 1024, "lists too large for the hybrid search (%d members)",
+                      ix->max_list);
+        KSC_TRY(launch_graph_search(A, ScanOut{thr, cnt, cand, pl.cap}, Gr, wb.pairs, wb.pair_off + L, st));
         KSC_LAUNCH_CHECK();
         // work list of the marked lists, then their scan
         KSC_CUDA(cudaMemsetAsync(wb.cnt, 0, sizeof(int32_t) * L, st));
@@ -3796,7 +3853,7 @@ static int make_plan(ksc_index* ix, int64_t nq, int k, int Pmax, int Rmax, const
     pl.efs = (opts && opts->efs > 0) ? opts->efs : 64;
     pl.tau = (opts && opts->tau >= 0 && opts->hybrid) ? opts->tau : 8;
     if (pl.hybrid) {
-        KSC_CHECK_ARG(pl.efs <= 96, "efs must be <= 96");
+        KSC_CHECK_ARG(pl.efs <= GS_MAX_EFS, "efs must be <= %d", GS_MAX_EFS);
         if (!ix->nbr_codes) {
             set_error("the hybrid search needs an index built or imported with graphs");
             return KSC_ESTATE;
