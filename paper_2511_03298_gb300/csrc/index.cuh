@@ -119,8 +119,16 @@ int mlp_features(const float* scores, int64_t nq, int ld, int spherical, float* 
 int mlp_infer_scores(const float* w, const float* scores, int ld, int spherical, int64_t B,
                      const ksc_adaptive_params& prm, int32_t* nprobe, int32_t* rerank, cudaStream_t st);
 int mlp_hits(const float* dists, int64_t nq, int k, const float* kth, int ip, int32_t* hits, cudaStream_t st);
-int mlp_adam(float* w, const float* g, float* m, float* v, int t, float lr, cudaStream_t st);
-int mlp_adam_n(float* w, const float* g, float* m, float* v, int n, int t, float lr, cudaStream_t st);
+// One training step (forward, backward, Adam step t) of the predictor on the
+// samples idx[0..nb) of feats / Y, nb <= batch; act: mlp_train_act(batch)
+// floats of scratch; adds the step's mean loss to *loss.  prune_*: the same of
+// the pruning classifier.
+size_t mlp_train_act(int64_t batch);
+size_t prune_train_act(int64_t batch);
+int mlp_train_step(float* w, float* m, float* v, const float* feats, const float* Y, const int64_t* idx, int64_t nb,
+                   int64_t batch, float* act, float* loss, int t, float lr, cudaStream_t st);
+int prune_train_step(float* w, float* m, float* v, const float* feats, const float* Y, const int64_t* idx, int64_t nb,
+                     int64_t batch, float* act, float* loss, int t, float lr, cudaStream_t st);
 int prune_mlp_grad(const float* w, const float* x, const float* y, int64_t B, float* grad, float* loss,
                    cudaStream_t st);
 // Predictive cluster pruning (prune.cu): per-list statistics; features /

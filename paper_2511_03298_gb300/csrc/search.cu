@@ -4391,7 +4391,7 @@ int ksc_train_predictor(ksc_index* ix, const float* Qtrain_dev, int64_t nt, cons
     float* Y = nullptr;
     int32_t* probes = nullptr;
     int32_t* lab_dev = nullptr;
-    float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr, *xb = nullptr, *yb = nullptr, *lossd = nullptr;
+    float *w = nullptr, *m = nullptr, *v = nullptr, *act = nullptr, *lossd = nullptr;
     int64_t* idx = nullptr;
     std::vector<int32_t> lab_n(nt), lab_r(nt);
     int rc = KSC_OK;
@@ -4449,11 +4449,9 @@ int ksc_train_predictor(ksc_index* ix, const float* Qtrain_dev, int64_t nt, cons
             off += rows[l] * fan[l] + rows[l];
         }
         T_CUDA(cudaMalloc(&w, sizeof(float) * KSC_MLP_NPARAMS));
-        T_CUDA(cudaMalloc(&g, sizeof(float) * KSC_MLP_NPARAMS));
         T_CUDA(cudaMalloc(&m, sizeof(float) * KSC_MLP_NPARAMS));
         T_CUDA(cudaMalloc(&v, sizeof(float) * KSC_MLP_NPARAMS));
-        T_CUDA(cudaMalloc(&xb, sizeof(float) * batch * KSC_MLP_FEATURES));
-        T_CUDA(cudaMalloc(&yb, sizeof(float) * batch * 2));
+        T_CUDA(cudaMalloc(&act, sizeof(float) * mlp_train_act(batch)));
         T_CUDA(cudaMalloc(&idx, sizeof(int64_t) * nt));
         T_CUDA(cudaMalloc(&lossd, sizeof(float) * steps));
         T_CUDA(cudaMemcpy(w, wh.data(), sizeof(float) * KSC_MLP_NPARAMS, cudaMemcpyHostToDevice));
@@ -4466,13 +4464,10 @@ int ksc_train_predictor(ksc_index* ix, const float* Qtrain_dev, int64_t nt, cons
             for (int64_t i = 0; i < nt; ++i) perm[i] = i;
             for (int64_t i = nt - 1; i > 0; --i) std::swap(perm[i], perm[(int64_t)(mix64(seed) % (uint64_t)(i + 1))]);
             T_CUDA(cudaMemcpyAsync(idx, perm.data(), sizeof(int64_t) * nt, cudaMemcpyHostToDevice, st));
+            T_CUDA(cudaMemsetAsync(lossd, 0, sizeof(float) * steps, st));
             for (int s_ = 0; s_ < steps; ++s_) {
                 const int64_t b0 = (int64_t)s_ * batch, nb = std::min<int64_t>(batch, nt - b0);
-                k_gather_rows<<<(unsigned)((nb * KSC_MLP_FEATURES + 255) / 256), 256, 0, st>>>(feats, idx + b0, nb,
-                                                                                             KSC_MLP_FEATURES, xb);
-                k_gather_rows<<<(unsigned)((nb * 2 + 255) / 256), 256, 0, st>>>(Y, idx + b0, nb, 2, yb);
-                if ((rc = mlp_grad(w, xb, yb, nb, g, lossd + s_, st))) break;
-                if ((rc = mlp_adam(w, g, m, v, ++t, lr, st))) break;
+                if ((rc = mlp_train_step(w, m, v, feats, Y, idx + b0, nb, batch, act, lossd + s_, ++t, lr, st))) break;
             }
             T_CUDA(cudaStreamSynchronize(st));  // perm is reused by the next epoch
         }
@@ -4494,8 +4489,8 @@ int ksc_train_predictor(ksc_index* ix, const float* Qtrain_dev, int64_t nt, cons
                                                 0.3f, 0.5f, 0};
     } while (0);
 #undef T_CUDA
-    cudaFree(feats); cudaFree(Y); cudaFree(probes); cudaFree(lab_dev); cudaFree(w); cudaFree(g); cudaFree(m);
-    cudaFree(v); cudaFree(xb); cudaFree(yb); cudaFree(idx); cudaFree(lossd);
+    cudaFree(feats); cudaFree(Y); cudaFree(probes); cudaFree(lab_dev); cudaFree(w); cudaFree(m); cudaFree(v); cudaFree(act);
+    cudaFree(idx); cudaFree(lossd);
     return rc;
 }
 
@@ -4856,7 +4851,7 @@ int ksc_train_pruner(ksc_index* ix, const float* Qtrain_dev, int64_t nt, const f
     const int64_t chunk = 8192, rows = nt * P;
     const int NF = KSC_PRUNE_FEATURES, NP = KSC_PRUNE_NPARAMS;
     float *feats = nullptr, *lab = nullptr, *Y = nullptr, *dists = nullptr, *model = nullptr;
-    float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr, *xb = nullptr, *yb = nullptr, *lossd = nullptr;
+    float *w = nullptr, *m = nullptr, *v = nullptr, *act = nullptr, *lossd = nullptr;
     int32_t* probes = nullptr;
     int64_t *ids = nullptr, *idx = nullptr;
     int rc = KSC_OK;
@@ -4900,11 +4895,9 @@ int ksc_train_pruner(ksc_index* ix, const float* Qtrain_dev, int64_t nt, const f
             off += nrow[l] * fan[l] + nrow[l];
         }
         T_CUDA(cudaMalloc(&w, sizeof(float) * NP));
-        T_CUDA(cudaMalloc(&g, sizeof(float) * NP));
         T_CUDA(cudaMalloc(&m, sizeof(float) * NP));
         T_CUDA(cudaMalloc(&v, sizeof(float) * NP));
-        T_CUDA(cudaMalloc(&xb, sizeof(float) * batch * NF));
-        T_CUDA(cudaMalloc(&yb, sizeof(float) * batch * 2));
+        T_CUDA(cudaMalloc(&act, sizeof(float) * prune_train_act(batch)));
         T_CUDA(cudaMalloc(&idx, sizeof(int64_t) * rows));
         T_CUDA(cudaMalloc(&lossd, sizeof(float) * steps));
         T_CUDA(cudaMemcpy(w, wh.data(), sizeof(float) * NP, cudaMemcpyHostToDevice));
@@ -4917,12 +4910,10 @@ int ksc_train_pruner(ksc_index* ix, const float* Qtrain_dev, int64_t nt, const f
             for (int64_t i = 0; i < rows; ++i) perm[i] = i;
             for (int64_t i = rows - 1; i > 0; --i) std::swap(perm[i], perm[(int64_t)(mix64(seed) % (uint64_t)(i + 1))]);
             T_CUDA(cudaMemcpyAsync(idx, perm.data(), sizeof(int64_t) * rows, cudaMemcpyHostToDevice, st));
+            T_CUDA(cudaMemsetAsync(lossd, 0, sizeof(float) * steps, st));
             for (int s_ = 0; s_ < steps; ++s_) {
                 const int64_t b0 = (int64_t)s_ * batch, nb = std::min<int64_t>(batch, rows - b0);
-                k_gather_rows<<<(unsigned)((nb * NF + 255) / 256), 256, 0, st>>>(feats, idx + b0, nb, NF, xb);
-                k_gather_rows<<<(unsigned)((nb * 2 + 255) / 256), 256, 0, st>>>(Y, idx + b0, nb, 2, yb);
-                if ((rc = prune_mlp_grad(w, xb, yb, nb, g, lossd + s_, st))) break;
-                if ((rc = mlp_adam_n(w, g, m, v, NP, ++t, lr, st))) break;
+                if ((rc = prune_train_step(w, m, v, feats, Y, idx + b0, nb, batch, act, lossd + s_, ++t, lr, st))) break;
             }
             T_CUDA(cudaStreamSynchronize(st));  // perm is reused by the next epoch
         }
@@ -4940,7 +4931,7 @@ int ksc_train_pruner(ksc_index* ix, const float* Qtrain_dev, int64_t nt, const f
         model = nullptr;
         bump_workspace_generation();
     } while (0);
-    void* tmp[] = {feats, lab, Y, dists, model, w, g, m, v, xb, yb, lossd, probes, ids, idx};
+    void* tmp[] = {feats, lab, Y, dists, model, w, m, v, act, lossd, probes, ids, idx};
     for (void* p : tmp)
         if (p) cudaFree(p);
     return rc;
