@@ -212,6 +212,183 @@ __global__ void k_residual(const float* __restrict__ X, const int64_t* __restric
     }
 }
 
+// ------------------------------------------------------------------ PQ, sub-vectors of a fixed width
+// A thread keeps one subspace (j = thread % M) and its 16 codewords in
+// registers and walks rows: a warp reads consecutive sub-vectors of a row, and
+// an item costs 16 DS differences and FMAs and 16 compares.  (The kernels for
+// any width below read the codebook and the row through L1 for every codeword:
+// 517 us per 65,536 x 64 items of width 2 against 52 us here with the sums.)  Same
+// operations and order for every (row, codeword), ties to the lower codeword.
+// RG = 256 / M row groups share a CTA.
+template <int DS>
+struct PqRow {
+    float v[DS];
+};
+template <int DS>
+__device__ __forceinline__ PqRow<DS> pq_load(const float* __restrict__ p) {
+    PqRow<DS> r;
+    if constexpr (DS == 2) {
+        const float2 x = __ldg(reinterpret_cast<const float2*>(p));
+        r.v[0] = x.x;
+        r.v[1] = x.y;
+    } else if constexpr (DS % 4 == 0) {
+#pragma unroll
+        for (int t = 0; t < DS; t += 4) {
+            const float4 x = __ldg(reinterpret_cast<const float4*>(p + t));
+            r.v[t] = x.x;
+            r.v[t + 1] = x.y;
+            r.v[t + 2] = x.z;
+            r.v[t + 3] = x.w;
+        }
+    } else {
+#pragma unroll
+        for (int t = 0; t < DS; ++t) r.v[t] = __ldg(p + t);
+    }
+    return r;
+}
+
+// (double)x.  This chip converts on its FP64 pipe (two lanes a clock and SM), so
+// a normal number's bits are widened with integer operations instead.
+__device__ __forceinline__ double widen_f32(float x) {
+    const uint32_t u = __float_as_uint(x), e = u & 0x7f800000u;
+    if (e == 0u || e == 0x7f800000u) return (double)x;  // zero, subnormal, infinity, NaN
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+
+template <int DS>
+__device__ __forceinline__ int pq_nearest(const PqRow<DS>& r, const float (&w)[PQ_K][DS]) {
+    float best = INFINITY;
+    int bi = 0;
+#pragma unroll
+    for (int c = 0; c < PQ_K; ++c) {
+        float s = 0.f;
+#pragma unroll
+        for (int t = 0; t < DS; ++t) {
+            const float df = r.v[t] - w[c][t];
+            s = fmaf(df, df, s);
+        }
+        if (s < best) {
+            best = s;
+            bi = c;
+        }
+    }
+    return bi;
+}
+
+template <int DS>
+__device__ __forceinline__ void pq_codewords(const float* __restrict__ cb, int j, float (&w)[PQ_K][DS]) {
+#pragma unroll
+    for (int c = 0; c < PQ_K; ++c)
+#pragma unroll
+        for (int t = 0; t < DS; ++t) w[c][t] = __ldg(cb + ((int64_t)j * PQ_K + c) * DS + t);
+}
+
+// Codes [np x M] of the rows of X, residuals to the mean of their list.
+template <int DS>
+__global__ void __launch_bounds__(256) k_pq_encode_w(const float* __restrict__ X, const int32_t* __restrict__ assign,
+                                                     const float* __restrict__ c_mean, int64_t np, int M,
+                                                     const float* __restrict__ cb, uint8_t* __restrict__ codes) {
+    const int RG = 256 / M, rg = threadIdx.x / M, j = threadIdx.x - rg * M;
+    if (rg >= RG) return;
+    const int d = M * DS;
+    float w[PQ_K][DS];
+    pq_codewords<DS>(cb, j, w);
+    for (int64_t r = (int64_t)blockIdx.x * RG + rg; r < np; r += (int64_t)gridDim.x * RG) {
+        PqRow<DS> x = pq_load<DS>(X + r * d + j * DS);
+        const PqRow<DS> c = pq_load<DS>(c_mean + (int64_t)assign[r] * d + j * DS);
+#pragma unroll
+        for (int t = 0; t < DS; ++t) x.v[t] = __fsub_rn(x.v[t], c.v[t]);
+        codes[r * M + j] = (uint8_t)pq_nearest<DS>(x, w);
+    }
+}
+
+// One k-means step on residual rows R [np x d]: every row's codewords, and the
+// FP64 sums and counts of every codeword's rows.  A thread adds to its own
+// sums (its subspace and row group: no atomics) in shared memory, laid out
+// [codeword][t][subspace] so that a warp's updates fall in distinct banks
+// whatever the codewords; each CTA leaves its sums in part [grid][16 DS M] and
+// counts in pcnt [grid][16 M] (k_pq_finish_w adds them up in CTA order: the
+// result does not depend on the scheduling).  Adding every element to 16 d
+// global sums took 222 us per 65,536 x 128 elements in atomics.
+template <int DS>
+__global__ void __launch_bounds__(256) k_pq_step(const float* __restrict__ R, int64_t np, int M, int RG,
+                                                 const float* __restrict__ cb, double* __restrict__ part,
+                                                 uint32_t* __restrict__ pcnt) {
+    extern __shared__ double pq_sm[];  // RG x 16 DS M sums, then RG x 16 M counts
+    const int E = PQ_K * DS * M, EC = PQ_K * M;
+    uint32_t* cnt = reinterpret_cast<uint32_t*>(pq_sm + (size_t)RG * E);
+    for (int e = threadIdx.x; e < RG * E; e += 256) pq_sm[e] = 0.0;
+    for (int e = threadIdx.x; e < RG * EC; e += 256) cnt[e] = 0u;
+    __syncthreads();
+    const int rg = threadIdx.x / M, j = threadIdx.x - rg * M;
+    const int d = M * DS;
+    if (rg < RG) {
+        float w[PQ_K][DS];
+        pq_codewords<DS>(cb, j, w);
+        double* ms = pq_sm + (size_t)rg * E + j;
+        uint32_t* mc = cnt + (size_t)rg * EC + j;
+        const int64_t stride = (int64_t)gridDim.x * RG;
+        for (int64_t r = (int64_t)blockIdx.x * RG + rg; r < np; r += 4 * stride) {
+            PqRow<DS> x[4];  // four rows in flight
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (r + u * stride < np) x[u] = pq_load<DS>(R + (r + u * stride) * d + j * DS);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (r + u * stride >= np) break;
+                const int c = pq_nearest<DS>(x[u], w);
+                mc[c * M] += 1u;
+#pragma unroll
+                for (int t = 0; t < DS; ++t) ms[(c * DS + t) * M] += widen_f32(x[u].v[t]);
+            }
+        }
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < E; e += 256) {
+        double v = 0.0;
+        for (int g = 0; g < RG; ++g) v += pq_sm[(size_t)g * E + e];
+        part[(size_t)blockIdx.x * E + e] = v;
+    }
+    for (int e = threadIdx.x; e < EC; e += 256) {
+        uint32_t v = 0;
+        for (int g = 0; g < RG; ++g) v += cnt[(size_t)g * EC + e];
+        pcnt[(size_t)blockIdx.x * EC + e] = v;
+    }
+}
+
+// New codewords (one without rows keeps its value): 32 elements per CTA, 32
+// slices of the partial sums each, so that a slice is about ten loads deep.
+__global__ void __launch_bounds__(1024) k_pq_finish_w(const double* __restrict__ part,
+                                                      const uint32_t* __restrict__ pcnt, int nparts, int M, int DS,
+                                                      float* __restrict__ cb) {
+    __shared__ double ss[32][32];
+    __shared__ uint32_t sc[32][32];
+    const int E = PQ_K * DS * M, EC = PQ_K * M;
+    const int l = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int e = blockIdx.x * 32 + l;  // (c DS + t) M + j
+    const int ct = e / M, j = e - ct * M, c = ct / DS, t = ct - c * DS;
+    const int per = (nparts + 31) / 32, p0 = g * per, p1 = min(nparts, p0 + per);
+    double s = 0.0;
+    uint32_t n = 0;
+    if (e < E) {
+#pragma unroll 12
+        for (int p = p0; p < p1; ++p) {
+            s += part[(size_t)p * E + e];
+            n += pcnt[(size_t)p * EC + c * M + j];
+        }
+    }
+    ss[g][l] = s;
+    sc[g][l] = n;
+    __syncthreads();
+    if (g == 0 && e < E) {
+        for (int i = 1; i < 32; ++i) {
+            s += ss[i][l];
+            n += sc[i][l];
+        }
+        if (n > 0) cb[((int64_t)j * PQ_K + c) * DS + t] = (float)(s / (double)n);
+    }
+}
+
 // PQ: nearest of the 16 codewords of subspace j for residual rows (one
 // thread per (row, j)); rows either given as residuals R or computed from X.
 __global__ void k_pq_encode(const float* __restrict__ R, const float* __restrict__ X,
@@ -423,6 +600,73 @@ static void host_perm(int64_t n, uint64_t seed, std::vector<int64_t>& p) {
         p[i] = p[j];
         p[j] = t;
     }
+}
+
+// Row groups per CTA of k_pq_step and its shared bytes (at most 100 KB with
+// more than one group, so that two CTAs fit an SM).
+static size_t pq_step_smem(int M, int DS, int RG) { return (size_t)RG * M * PQ_K * (8 * DS + 4); }
+static int pq_step_groups(int M, int DS) {
+    int rg = 256 / M;
+    while (rg > 1 && pq_step_smem(M, DS, rg) > 100 * 1024) --rg;
+    return rg;
+}
+
+// k-means of the PQ codebooks cb [M x 16 x DS] on residual rows R [np x d],
+// one kernel pair per iteration.
+template <int DS>
+static int pq_train_w(const float* R, int64_t np, int M, int iters, float* cb, cudaStream_t st) {
+    const int RG = pq_step_groups(M, DS), E = PQ_K * DS * M, EC = PQ_K * M;
+    const size_t smem = pq_step_smem(M, DS, RG);
+    KSC_CUDA(cudaFuncSetAttribute(k_pq_step<DS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int per_sm = 0;
+    KSC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pq_step<DS>, 256, smem));
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((np + 4 * RG - 1) / (4 * RG),
+                                                                 (int64_t)num_sms() * (per_sm > 0 ? per_sm : 1)));
+    double* part = nullptr;
+    uint32_t* pcnt = nullptr;
+    KSC_CUDA(cudaMalloc(&part, sizeof(double) * (size_t)grid * E));
+    cudaError_t e = cudaMalloc(&pcnt, sizeof(uint32_t) * (size_t)grid * EC);
+    if (e == cudaSuccess) {
+        for (int it = 0; it < iters; ++it) {
+            k_pq_step<DS><<<grid, 256, smem, st>>>(R, np, M, RG, cb, part, pcnt);
+            k_pq_finish_w<<<(E + 31) / 32, 1024, 0, st>>>(part, pcnt, grid, M, DS, cb);
+        }
+        e = cudaGetLastError();
+    }
+    cudaFree(part);  // (waits for the kernels)
+    cudaFree(pcnt);
+    KSC_CUDA(e);
+    return KSC_OK;
+}
+
+// The widths that the register kernels serve (a row's sub-vectors then start
+// on the loads' alignment: DS floats, d a multiple of DS); other widths take
+// the kernels for any width.
+static bool pq_width_w(int dsub) { return dsub == 1 || dsub == 2 || dsub == 3 || dsub == 4 || dsub == 8; }
+
+static int pq_train(const float* R, int64_t np, int M, int dsub, int iters, float* cb, cudaStream_t st) {
+    switch (dsub) {
+        case 1: return pq_train_w<1>(R, np, M, iters, cb, st);
+        case 2: return pq_train_w<2>(R, np, M, iters, cb, st);
+        case 3: return pq_train_w<3>(R, np, M, iters, cb, st);
+        case 4: return pq_train_w<4>(R, np, M, iters, cb, st);
+        default: return pq_train_w<8>(R, np, M, iters, cb, st);
+    }
+}
+
+static int pq_encode(const float* X, const int32_t* assign, const float* c_mean, int64_t n, int M, int dsub,
+                     const float* cb, uint8_t* codes, cudaStream_t st) {
+    const int RG = 256 / M;
+    const int grid = (int)std::min<int64_t>((n + 4 * RG - 1) / (4 * RG), (int64_t)num_sms() * 8);
+    switch (dsub) {
+        case 1: k_pq_encode_w<1><<<grid, 256, 0, st>>>(X, assign, c_mean, n, M, cb, codes); break;
+        case 2: k_pq_encode_w<2><<<grid, 256, 0, st>>>(X, assign, c_mean, n, M, cb, codes); break;
+        case 3: k_pq_encode_w<3><<<grid, 256, 0, st>>>(X, assign, c_mean, n, M, cb, codes); break;
+        case 4: k_pq_encode_w<4><<<grid, 256, 0, st>>>(X, assign, c_mean, n, M, cb, codes); break;
+        default: k_pq_encode_w<8><<<grid, 256, 0, st>>>(X, assign, c_mean, n, M, cb, codes); break;
+    }
+    KSC_LAUNCH_CHECK();
+    return KSC_OK;
 }
 
 // Lloyd on rows `sample` of X (device), init = first L sample rows.
@@ -776,13 +1020,17 @@ int ksc_build_index(const float* X_dev, int64_t n, int32_t d, int32_t nlist, int
         B_CUDA(cudaMalloc(&Rs, sizeof(float) * npq * d));
         k_residual<<<grid_for(npq * d), 256, 0, st>>>(ix->X, perm_dev, npq, d, ix->assign, ix->c_mean, Rs);
         B_CUDA(cudaMalloc(&ix->codebook, sizeof(float) * M * PQ_K * ix->dsub));
-        B_CUDA(cudaMalloc(&pcodes, (size_t)npq * M));
-        cudaFree(sums); sums = nullptr;
-        cudaFree(cnt); cnt = nullptr;
-        B_CUDA(cudaMalloc(&sums, sizeof(double) * M * PQ_K * ix->dsub));
-        B_CUDA(cudaMalloc(&cnt, sizeof(unsigned long long) * M * PQ_K));
+        const bool wide = pq_width_w(ix->dsub);
+        if (!wide) {
+            B_CUDA(cudaMalloc(&pcodes, (size_t)npq * M));
+            cudaFree(sums); sums = nullptr;
+            cudaFree(cnt); cnt = nullptr;
+            B_CUDA(cudaMalloc(&sums, sizeof(double) * M * PQ_K * ix->dsub));
+            B_CUDA(cudaMalloc(&cnt, sizeof(unsigned long long) * M * PQ_K));
+        }
         k_pq_init<<<grid_for((int64_t)M * PQ_K * ix->dsub), 256, 0, st>>>(Rs, d, M, ix->dsub, ix->codebook);
-        for (int it = 0; it < iters; ++it) {
+        if (wide && (rc = pq_train(Rs, npq, M, ix->dsub, iters, ix->codebook, st))) break;
+        for (int it = 0; it < iters && !wide; ++it) {
             k_pq_encode<<<grid_for(npq * M), 256, 0, st>>>(Rs, nullptr, nullptr, nullptr, npq, d, M, ix->dsub,
                                                            ix->codebook, pcodes);
             B_CUDA(cudaMemsetAsync(sums, 0, sizeof(double) * M * PQ_K * ix->dsub, st));
@@ -794,8 +1042,10 @@ int ksc_build_index(const float* X_dev, int64_t n, int32_t d, int32_t nlist, int
         if (rc) break;
         // 5. encode every vector and pack the lists into blocks
         B_CUDA(cudaMalloc(&codes_dev, (size_t)n * M));
-        k_pq_encode<<<grid_for(n * M), 256, 0, st>>>(nullptr, ix->X, ix->assign, ix->c_mean, n, d, M, ix->dsub,
-                                                     ix->codebook, codes_dev);
+        if (wide) rc = pq_encode(ix->X, ix->assign, ix->c_mean, n, M, ix->dsub, ix->codebook, codes_dev, st);
+        else k_pq_encode<<<grid_for(n * M), 256, 0, st>>>(nullptr, ix->X, ix->assign, ix->c_mean, n, d, M, ix->dsub,
+                                                          ix->codebook, codes_dev);
+        if (rc) break;
         B_CUDA(cudaGetLastError());
         B_CUDA(cudaMemcpyAsync(assign_host.data(), ix->assign, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, st));
         B_CUDA(cudaStreamSynchronize(st));
