@@ -94,18 +94,24 @@ __global__ void k_normalise_rows(float* __restrict__ C, int L, int d) {
     }
 }
 
-// Nearest centroid of every row: score = ||c||^2 - 2<x,c> (L2) or -<x,c>
-// (spherical); ties -> lower centroid id.  64 rows x 64 centroids per tile,
+// Nearest centroid of every row (or of the listed rows): score = ||c||^2 -
+// 2<x,c> (L2) or -<x,c> (spherical); ties -> lower centroid id.  The rule of
+// every assignment; where the data fit FP16 operands, assign_tc.cu decides
+// most rows and this kernel the ones it lists.  64 rows x 64 centroids per tile,
 // 256 threads, 4 x 4 outputs per thread, dims staged 32 at a time.
 constexpr int AS_T = 64, AS_K = 32;
 __global__ void __launch_bounds__(256) k_assign(const float* __restrict__ X, int64_t np, int d,
                                                 const float* __restrict__ Cc, const float* __restrict__ cn,
                                                 int L, int spherical, int32_t* __restrict__ assign,
-                                                float* __restrict__ best_out) {
+                                                const int32_t* __restrict__ rows,
+                                                const int32_t* __restrict__ nrows, int above) {
     __shared__ float xs[AS_K][AS_T + 4];
     __shared__ float cs[AS_K][AS_T + 4];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const int64_t row0 = (int64_t)blockIdx.x * AS_T;
+    // every row, or (rows != NULL) the nrows[0] rows listed if those are more than `above`
+    if (nrows) np = *nrows > above ? min(np, (int64_t)*nrows) : 0;
+    if (row0 >= np) return;
     float best[4];
     int bid[4];
 #pragma unroll
@@ -121,7 +127,7 @@ __global__ void __launch_bounds__(256) k_assign(const float* __restrict__ X, int
                 int r = e / AS_K, kk = e % AS_K;
                 int64_t gr = row0 + r;
                 int gk = k0 + kk;
-                xs[kk][r] = (gr < np && gk < d) ? X[gr * d + gk] : 0.f;
+                xs[kk][r] = (gr < np && gk < d) ? X[(rows ? rows[gr] : gr) * d + gk] : 0.f;
                 int gc = c0 + r;
                 cs[kk][r] = (gc < L && gk < d) ? Cc[(int64_t)gc * d + gk] : 0.f;
             }
@@ -167,10 +173,7 @@ __global__ void __launch_bounds__(256) k_assign(const float* __restrict__ X, int
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             int64_t r = row0 + ty * 4 + i;
-            if (r < np) {
-                assign[r] = bid[i];
-                if (best_out) best_out[r] = best[i];
-            }
+            if (r < np) assign[rows ? rows[r] : r] = bid[i];
         }
     }
 }
@@ -669,9 +672,23 @@ static int pq_encode(const float* X, const int32_t* assign, const float* c_mean,
     return KSC_OK;
 }
 
-// Lloyd on rows `sample` of X (device), init = first L sample rows.
+// The assignment of T's rows to its centroids: tensor cores, then the FP32
+// kernel for the rows left over.
+static int assign_rows(AssignTc& T, int32_t* assign, cudaStream_t st) {
+    KSC_TRY(T.run(assign, st));
+    k_assign<<<(unsigned)((T.nrows + AS_T - 1) / AS_T), 256, 0, st>>>(T.X, T.nrows, T.d, T.C, T.cn, T.L, T.spherical,
+                                                                      assign, T.redo, T.small, T.redo_rows());
+    KSC_LAUNCH_CHECK();
+    return KSC_OK;
+}
+
+// Rows per pass of the final assignment (bounds the FP16 copy).
+constexpr int64_t ASSIGN_CHUNK = 1 << 20;
+
+// Lloyd on rows `sample` of X (device), init = first L sample rows.  T: the
+// tensor-core assignment, or null (FP32 cores throughout).
 static int lloyd(const float* X, const int64_t* sample_dev, int64_t ns, int d, int L, int iters, float* C,
-                 cudaStream_t st) {
+                 AssignTc* T, float xmax, cudaStream_t st) {
     float* Xs = nullptr;
     float* cn = nullptr;
     int32_t* a = nullptr;
@@ -689,12 +706,28 @@ static int lloyd(const float* X, const int64_t* sample_dev, int64_t ns, int d, i
     LL_CUDA(cudaMalloc(&cnt, sizeof(unsigned long long) * L));
     k_gather_rows<<<grid_for(ns * d), 256, 0, st>>>(X, sample_dev, ns, d, Xs);
     LL_CUDA(cudaMemcpyAsync(C, Xs, sizeof(float) * L * d, cudaMemcpyDeviceToDevice, st));
-    for (int it = 0; it < iters; ++it) {
-        k_row_sqnorm<<<(L + 255) / 256, 256, 0, st>>>(C, L, d, cn);
-        k_assign<<<(unsigned)((ns + AS_T - 1) / AS_T), 256, 0, st>>>(Xs, ns, d, C, cn, L, 0, a, nullptr);
-        LL_CUDA(cudaMemsetAsync(sums, 0, sizeof(double) * L * d, st));
-        LL_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * L, st));
+    LL_CUDA(cudaMemsetAsync(sums, 0, sizeof(double) * L * d, st));
+    LL_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * L, st));
+    if (T) rc = T->set_rows(Xs, ns, st);
+    for (int it = 0; it < iters && rc == KSC_OK; ++it) {
+        if (T) {
+            // the means of the previous round are taken as the operands are made
+            rc = T->set_centroids(C, it ? sums : nullptr, it ? cnt : nullptr, false, xmax, st);
+            if (rc == KSC_OK) rc = assign_rows(*T, a, st);
+            if (rc) break;
+        } else {
+            if (it) {
+                k_centroid_finish<<<grid_for((int64_t)L * d), 256, 0, st>>>(sums, cnt, C, L, d, C);
+                LL_CUDA(cudaMemsetAsync(sums, 0, sizeof(double) * L * d, st));
+                LL_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long) * L, st));
+            }
+            k_row_sqnorm<<<(L + 255) / 256, 256, 0, st>>>(C, L, d, cn);
+            k_assign<<<(unsigned)((ns + AS_T - 1) / AS_T), 256, 0, st>>>(Xs, ns, d, C, cn, L, 0, a, nullptr, nullptr, 0);
+        }
         k_centroid_accum<<<grid_for(ns * d), 256, 0, st>>>(Xs, nullptr, ns, d, a, sums, cnt);
+        LL_CUDA(cudaGetLastError());
+    }
+    if (rc == KSC_OK) {
         k_centroid_finish<<<grid_for((int64_t)L * d), 256, 0, st>>>(sums, cnt, C, L, d, C);
         LL_CUDA(cudaGetLastError());
     }
@@ -989,6 +1022,7 @@ int ksc_build_index(const float* X_dev, int64_t n, int32_t d, int32_t nlist, int
     uint8_t* pcodes = nullptr;
     int rc = KSC_OK;
     std::vector<int32_t> assign_host(n);
+    AssignTc T;
     do {
 #define B_CUDA(call) { cudaError_t e_ = (call); if (e_ != cudaSuccess) { set_error("%s: %s", #call, cudaGetErrorString(e_)); rc = e_ == cudaErrorMemoryAllocation ? KSC_ENOMEM : KSC_ECUDA; break; } }
         B_CUDA(cudaMalloc(&ix->X, sizeof(float) * n * d));
@@ -999,14 +1033,28 @@ int ksc_build_index(const float* X_dev, int64_t n, int32_t d, int32_t nlist, int
         B_CUDA(cudaMalloc(&ix->c_mean, sizeof(float) * nlist * d));
         B_CUDA(cudaMalloc(&ix->c_rank_sq, sizeof(float) * nlist));
         // 1. coarse quantiser
-        if ((rc = lloyd(ix->X, perm_dev, ns, d, nlist, iters, ix->c_mean, st))) break;
+        float xmax = 0.f;
+        if ((rc = max_abs(ix->X, n * d, &xmax, st))) break;
+        const bool tc = assign_tc_supported(xmax);
+        if (tc && (rc = T.init(std::max(ns, std::min(n, ASSIGN_CHUNK)), d, nlist, xmax, st))) break;
+        if ((rc = lloyd(ix->X, perm_dev, ns, d, nlist, iters, ix->c_mean, tc ? &T : nullptr, xmax, st))) break;
         B_CUDA(cudaMemcpyAsync(ix->c_rank, ix->c_mean, sizeof(float) * nlist * d, cudaMemcpyDeviceToDevice, st));
         if (spherical) k_normalise_rows<<<(nlist + 255) / 256, 256, 0, st>>>(ix->c_rank, nlist, d);
         k_row_sqnorm<<<(nlist + 255) / 256, 256, 0, st>>>(ix->c_rank, nlist, d, ix->c_rank_sq);
         // 2. list of every vector by the ranking score
         B_CUDA(cudaMalloc(&ix->assign, sizeof(int32_t) * n));
-        k_assign<<<(unsigned)((n + AS_T - 1) / AS_T), 256, 0, st>>>(ix->X, n, d, ix->c_rank, ix->c_rank_sq, nlist,
-                                                                    spherical, ix->assign, nullptr);
+        if (tc) {
+            rc = T.set_centroids(ix->c_rank, nullptr, nullptr, spherical, spherical ? 1.f : xmax, st);
+            for (int64_t r0 = 0; r0 < n && rc == KSC_OK; r0 += ASSIGN_CHUNK) {
+                if ((rc = T.set_rows(ix->X + r0 * d, std::min(n - r0, ASSIGN_CHUNK), st))) break;
+                if (r0) B_CUDA(cudaMemsetAsync(T.small, 0, sizeof(int32_t) * 2, st));
+                rc = assign_rows(T, ix->assign + r0, st);
+            }
+            if (rc) break;
+        } else {
+            k_assign<<<(unsigned)((n + AS_T - 1) / AS_T), 256, 0, st>>>(ix->X, n, d, ix->c_rank, ix->c_rank_sq, nlist,
+                                                                        spherical, ix->assign, nullptr, nullptr, 0);
+        }
         // 3. mean centroids of the lists (Sec. 4.6.1)
         B_CUDA(cudaMalloc(&sums, sizeof(double) * (size_t)nlist * d));
         B_CUDA(cudaMalloc(&cnt, sizeof(unsigned long long) * nlist));
@@ -1049,6 +1097,7 @@ int ksc_build_index(const float* X_dev, int64_t n, int32_t d, int32_t nlist, int
         B_CUDA(cudaGetLastError());
         B_CUDA(cudaMemcpyAsync(assign_host.data(), ix->assign, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, st));
         B_CUDA(cudaStreamSynchronize(st));
+        if (tc && (rc = T.check(st))) break;
         if ((rc = pack_lists(ix, codes_dev, assign_host.data(), st))) break;
         if ((rc = finish_common(ix, st))) break;
         if (opts && opts->build_graph) {

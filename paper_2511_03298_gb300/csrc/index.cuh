@@ -107,6 +107,33 @@ int rank_scores_tc(ksc_index* ix, const float* Q, int64_t nq, float* scores, flo
 int rank_scores_tc8(ksc_index* ix, const float* Q, int64_t nq, float* scores, float* err, cudaStream_t st);
 // Per-query error bound of the list scores (tensor-core or FP32 path).
 int score_err(ksc_index* ix, const float* Q, int64_t nq, bool tensor_cores, float* err, cudaStream_t st);
+// Nearest-centroid assignment with tensor-core scores (assign_tc.cu): the
+// operands and scratch of assignments of up to `rows` rows to L centroids.
+// set_rows, set_centroids, run; more than redo_rows() rows left on
+// redo[0..small[0]) are the FP32 tile kernel's (index.cu).
+struct AssignTc {
+    int64_t rows = 0, nrows = 0;
+    int d = 0, L = 0, Kp = 0, Lpad = 0, spherical = 0;
+    float xscale = 1.f, cscale = 1.f;
+    const float *X = nullptr, *C = nullptr;
+    void *x16 = nullptr, *c16 = nullptr;
+    float *xnorm = nullptr, *cn = nullptr, *base = nullptr;
+    int32_t *redo = nullptr, *small = nullptr;
+    int init(int64_t rows, int d, int L, float xmax, cudaStream_t st);
+    int set_rows(const float* X, int64_t n, cudaStream_t st);
+    // sums / cnt (optional): C becomes their means and they are cleared
+    int set_centroids(float* C, double* sums, unsigned long long* cnt, bool spherical, float cmax_abs,
+                      cudaStream_t st);
+    int run(int32_t* assign, cudaStream_t st);
+    static int redo_rows();
+    int check(cudaStream_t st);
+    void free();
+    ~AssignTc() { free(); }
+};
+// Whether rows of largest magnitude xmax (NaN or infinity: not finite) fit the
+// FP16 operands' bound, and that magnitude.
+bool assign_tc_supported(float xmax);
+int max_abs(const float* X, int64_t m, float* out, cudaStream_t st);
 // Gather of rows src[idx[r]] (width d floats) into dst (index.cu).
 __global__ void k_gather_rows(const float* __restrict__ X, const int64_t* __restrict__ idx, int64_t cnt, int d,
                               float* __restrict__ out);
