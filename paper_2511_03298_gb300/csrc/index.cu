@@ -8,6 +8,7 @@
 #include <atomic>
 #include <cstdarg>
 #include <algorithm>
+#include <functional>
 #include <cstdio>
 #include <cstring>
 #include <vector>
@@ -517,7 +518,7 @@ int free_index_memory(ksc_index* ix) {
         // a view: its own workspace, status, counters and events, and what it
         // allocated lazily itself (not the same pointer as its source's)
         const ksc_index* s = ix->parent;
-        void* own[] = {ix->status, ix->stats, ix->c_rank_bf16 != s->c_rank_bf16 ? ix->c_rank_bf16 : nullptr,
+        void* own[] = {ix->status, ix->c_rank_bf16 != s->c_rank_bf16 ? ix->c_rank_bf16 : nullptr,
                        ix->c_rank_f8 != s->c_rank_f8 ? ix->c_rank_f8 : nullptr,
                        ix->c_rank_f8_scale != s->c_rank_f8_scale ? ix->c_rank_f8_scale : nullptr,
                        ix->X_bf16 != s->X_bf16 ? ix->X_bf16 : nullptr, ix->X_fp8 != s->X_fp8 ? ix->X_fp8 : nullptr,
@@ -532,7 +533,7 @@ int free_index_memory(ksc_index* ix) {
         return KSC_OK;
     }
     void* ptrs[] = {ix->X, ix->c_rank, ix->c_rank_sq, ix->c_mean, ix->codebook, ix->list_boff, ix->list_n,
-                    ix->blk_ids, ix->blk_codes, ix->assign, ix->graph, ix->entry, ix->status, ix->stats,
+                    ix->blk_ids, ix->blk_codes, ix->assign, ix->graph, ix->entry, ix->status,
                     ix->c_rank_bf16, ix->mlp_w, ix->blk_list, ix->nbr_pos, ix->nbr_codes, ix->entry_pos,
                     ix->X_bf16, ix->X_fp8, ix->X_scale, ix->pr_stats, ix->pr_vecs, ix->pr_model, ix->dims,
                     ix->X_rr, ix->c_rank_f8, ix->c_rank_f8_scale, ix->gids, ix->X_band, ix->X_u8};
@@ -565,6 +566,10 @@ int pack_lists(ksc_index* ix, const uint8_t* codes_dev, const int32_t* assign_ho
     }
     ix->max_list = (int32_t)maxl;
     ix->nblocks = ix->h_boff[L];
+    ix->h_top_blocks.assign(L + 1, 0);
+    for (int c = 0; c < L; ++c) ix->h_top_blocks[c + 1] = ix->h_boff[c + 1] - ix->h_boff[c];
+    std::sort(ix->h_top_blocks.begin() + 1, ix->h_top_blocks.end(), std::greater<int64_t>());
+    for (int c = 0; c < L; ++c) ix->h_top_blocks[c + 1] += ix->h_top_blocks[c];
     std::vector<int32_t> ids((size_t)ix->nblocks * BLOCK_VECS, -1);
     std::vector<int64_t> fill(L);
     for (int c = 0; c < L; ++c) fill[c] = ix->h_boff[c] * BLOCK_VECS;
@@ -767,10 +772,9 @@ static int finish_common(ksc_index* ix, cudaStream_t st) {
     if (!ix->c_rank_sq) KSC_CUDA(cudaMalloc(&ix->c_rank_sq, sizeof(float) * ix->L));
     k_row_sqnorm<<<(ix->L + 255) / 256, 256, 0, st>>>(ix->c_rank, ix->L, ix->d, ix->c_rank_sq);
     KSC_LAUNCH_CHECK();
-    KSC_CUDA(cudaMalloc(&ix->status, sizeof(int32_t) * 4));
-    KSC_CUDA(cudaMemsetAsync(ix->status, 0, sizeof(int32_t) * 4, st));
-    KSC_CUDA(cudaMalloc(&ix->stats, sizeof(unsigned long long) * 4));
-    KSC_CUDA(cudaMemsetAsync(ix->stats, 0, sizeof(unsigned long long) * 4, st));
+    KSC_CUDA(cudaMalloc(&ix->status, STATUS_BYTES));
+    ix->stats = (unsigned long long*)(ix->status + STATUS_STATS);
+    KSC_CUDA(cudaMemsetAsync(ix->status, 0, STATUS_BYTES, st));
     KSC_CUDA(cudaStreamSynchronize(st));
     return KSC_OK;
 }
@@ -1148,10 +1152,11 @@ extern "C" int ksc_index_view(ksc_index* ix, ksc_index** out) {
     v->launches = 0;
     v->status = nullptr;
     v->stats = nullptr;
-    cudaError_t e = cudaMalloc(&v->status, sizeof(int32_t) * 4);
-    if (e == cudaSuccess) e = cudaMalloc(&v->stats, sizeof(unsigned long long) * 4);
-    if (e == cudaSuccess) e = cudaMemset(v->status, 0, sizeof(int32_t) * 4);
-    if (e == cudaSuccess) e = cudaMemset(v->stats, 0, sizeof(unsigned long long) * 4);
+    cudaError_t e = cudaMalloc(&v->status, STATUS_BYTES);
+    if (e == cudaSuccess) {
+        v->stats = (unsigned long long*)(v->status + STATUS_STATS);
+        e = cudaMemset(v->status, 0, STATUS_BYTES);
+    }
     if (e != cudaSuccess) {
         ksc::set_error("ksc_index_view: %s", cudaGetErrorString(e));
         ksc_index_free(v);

@@ -14,6 +14,9 @@
 constexpr int BLOCK_VECS = 32;
 constexpr int PQ_K = 16;
 
+// Layout of a handle's counters allocation (32-bit words).
+constexpr int STATUS_NREC = 2, STATUS_STATS = 4, STATUS_BYTES = 48;
+
 struct ksc_index {
     int64_t n = 0;
     int32_t d = 0, L = 0, M = 0, dsub = 0, metric = KSC_L2, spherical = 0;
@@ -42,11 +45,14 @@ struct ksc_index {
     void* X_u8 = nullptr;          // [n x d] U8 rows when every coordinate is an integer in [0, 255] (exact)
     int x_u8_state = 0;            // 0 not checked, 1 X_u8 holds the rows exactly, -1 they do not fit bytes
     float2* X_band = nullptr;      // [n] per re-rank row: bounds of its norm and of its BF16 rounding error's norm (made on first use)
-    int32_t* status = nullptr;     // device status word
+    // device status word, then [STATUS_NREC] the small-batch search's two item
+    // counts, then [STATUS_STATS] the counters (stats: in the same allocation)
+    int32_t* status = nullptr;
     unsigned long long* stats = nullptr;  // [4] counters of the last search
     // host mirrors
     std::vector<int64_t> h_boff;   // [L + 1]
     std::vector<int32_t> h_n;      // [L]
+    std::vector<int64_t> h_top_blocks;  // [L + 1] blocks of the p longest lists
     // tensor-core ranking: BF16 copy of c_rank [L x Kp], its TMA map, max ||c||
     void* c_rank_bf16 = nullptr;
     alignas(64) unsigned char map_c[128] = {};

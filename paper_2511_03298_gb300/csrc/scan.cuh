@@ -97,6 +97,11 @@ struct ScanOut {
     int32_t* cnt;
     uint64_t* cand;
     int cap;
+    // items given one by one (small batches): (pair e, first block, end block,
+    // list), their number, and each pair's place in the unfiltered store
+    const int4* recs = nullptr;
+    const int32_t* nrec = nullptr;
+    const int32_t* noff = nullptr;
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -139,6 +144,85 @@ __device__ __forceinline__ ScanItem locate_item(const ScanArgs& A, const int64_t
     r.g0 = pair_off[lo] + grp * QG;
     r.npairs = pair_off[lo + 1] - r.g0;
     return r;
+}
+
+__device__ __forceinline__ int nibble_of(const uint8_t* __restrict__ blk, int M, int j, int v) {
+    uint8_t byte = blk[j * 16 + (v >> 1)];
+    return (v & 1) ? (byte >> 4) : (byte & 15);
+}
+
+__device__ __forceinline__ int32_t scalar_dist(const uint8_t* __restrict__ lutp, int32_t b,
+                                               const uint8_t* __restrict__ blk, int M, int v) {
+    int32_t D = b;
+    for (int j = 0; j < M; ++j) D += lutp[j * 16 + nibble_of(blk, M, j, v)];
+    return D;
+}
+
+// A query whose candidate store overflowed, redone exactly by one CTA: every
+// key of every probed list is recomputed (scalar lookups) inside the radix
+// select.  The min(R, keys) smallest, sorted, into out; their number.  buf:
+// sel_cap keys (may be out), s_pref: one more than the query's probes.
+__device__ __forceinline__ int redo_select(const ScanArgs& A, int64_t q, int R, uint64_t* out, uint64_t* buf, int sel_cap,
+                                           uint32_t* hist, int32_t* s_pref) {
+    const int P = nprobe_of(A, q);
+    __syncthreads();  // s_pref of the previous query is no longer read
+    if (threadIdx.x == 0) {
+        int acc = 0;
+        for (int r = 0; r < P; ++r) {
+            s_pref[r] = acc;
+            const int p = A.probes[q * A.Pmax + r];
+            acc += (p >= 0 && p < A.L) ? A.list_n[p] : 0;
+        }
+        s_pref[P] = acc;
+    }
+    __syncthreads();
+    const int N = s_pref[P];
+    auto load = [&](int i) -> uint64_t {
+        int lo = 0, hi = P - 1;
+        while (lo < hi) {
+            int mid = (lo + hi + 1) >> 1;
+            if (s_pref[mid] <= i) lo = mid; else hi = mid - 1;
+        }
+        const int64_t item = q * A.Pmax + lo;
+        const int p = A.probes[item];
+        const int m = i - s_pref[lo];
+        const int64_t blk = A.boff[p] + (m >> 5);
+        const int v = m & 31;
+        int32_t D = scalar_dist(A.lut + item * A.M * PQ_K, A.bias[item], A.codes + blk * A.M * 16, A.M, v);
+        return make_key(D, A.ids[blk * 32 + v]);
+    };
+    const int K = min(R, N);
+    block_select_smallest(load, N, K, out, buf, sel_cap, hist);
+    return K;
+}
+
+// The exact FP32 score of list centroid c for the query qs (shared memory), by
+// one warp.
+__device__ __forceinline__ float exact_list_score(const float* __restrict__ qs, const float* __restrict__ c, int d,
+                                                  int spherical, int lane) {
+    float acc = 0.f;
+    if ((d & 3) == 0) {
+        for (int t = lane * 4; t < d; t += 128) {
+            float4 cv = __ldg(reinterpret_cast<const float4*>(c + t));
+            float4 qv = *reinterpret_cast<const float4*>(qs + t);
+            if (spherical) {
+                acc = fmaf(qv.x, cv.x, acc); acc = fmaf(qv.y, cv.y, acc);
+                acc = fmaf(qv.z, cv.z, acc); acc = fmaf(qv.w, cv.w, acc);
+            } else {
+                float e0 = qv.x - cv.x, e1 = qv.y - cv.y, e2 = qv.z - cv.z, e3 = qv.w - cv.w;
+                acc = fmaf(e0, e0, acc); acc = fmaf(e1, e1, acc); acc = fmaf(e2, e2, acc); acc = fmaf(e3, e3, acc);
+            }
+        }
+    } else {
+        for (int t = lane; t < d; t += 32) {
+            float cv = __ldg(c + t);
+            if (spherical) acc = fmaf(qs[t], cv, acc);
+            else { float e = qs[t] - cv; acc = fmaf(e, e, acc); }
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    return spherical ? -acc : acc;
 }
 
 // The tensor-core scan (scan_tc.cu): queries per item for M subspaces (0: not

@@ -19,8 +19,11 @@
 #include <cuda_fp8.h>
 
 #include "index.cuh"
+#include "lut.cuh"
 #include "mlp.cuh"
+#include "rerank.cuh"
 #include "scan.cuh"
+#include "small.cuh"
 
 namespace ksc {
 
@@ -102,33 +105,6 @@ __global__ void __launch_bounds__(256) k_list_scores(const float* __restrict__ Q
 constexpr int RS_CAP = 4096;     // largest re-score buffer
 constexpr int FEAT_K = 32;       // list distances of the predictor's features
 constexpr int RS_SMEM_L = 8192;  // score rows up to this length are staged in shared memory
-__device__ __forceinline__ float exact_list_score(const float* __restrict__ qs, const float* __restrict__ c, int d,
-                                                  int spherical, int lane) {
-    float acc = 0.f;
-    if ((d & 3) == 0) {
-        for (int t = lane * 4; t < d; t += 128) {
-            float4 cv = __ldg(reinterpret_cast<const float4*>(c + t));
-            float4 qv = *reinterpret_cast<const float4*>(qs + t);
-            if (spherical) {
-                acc = fmaf(qv.x, cv.x, acc); acc = fmaf(qv.y, cv.y, acc);
-                acc = fmaf(qv.z, cv.z, acc); acc = fmaf(qv.w, cv.w, acc);
-            } else {
-                float e0 = qv.x - cv.x, e1 = qv.y - cv.y, e2 = qv.z - cv.z, e3 = qv.w - cv.w;
-                acc = fmaf(e0, e0, acc); acc = fmaf(e1, e1, acc); acc = fmaf(e2, e2, acc); acc = fmaf(e3, e3, acc);
-            }
-        }
-    } else {
-        for (int t = lane; t < d; t += 32) {
-            float cv = __ldg(c + t);
-            if (spherical) acc = fmaf(qs[t], cv, acc);
-            else { float e = qs[t] - cv; acc = fmaf(e, e, acc); }
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    return spherical ? -acc : acc;
-}
-
 template <int NT>
 __global__ void __launch_bounds__(NT) k_rank_select(const float* __restrict__ scores, const float* __restrict__ err,
                                                      const float* __restrict__ Q, const float* __restrict__ Cc,
@@ -787,151 +763,7 @@ __global__ void __launch_bounds__(256) k_feat_scores(const float* __restrict__ s
     out[q * FEAT_K + lane] = unordered_f32(v) + qq;
 }
 
-// ------------------------------------------------------------------ a2: quantised LUTs
-// FP32 rule of the table entries, every op separately rounded:
-//   L2: u_t = q_t - c_t, acc += (u_t - C_jit)^2 over t ascending
-//   IP: u_t = q_t,       acc += u_t C_jit,                        T = -acc
-// The row operand u (the dsub values of subspace j) is formed once per row;
-// each entry is then the same sequence of rounded ops as written above.
-
-struct LutArgs {
-    const float* Q;
-    int64_t nq;
-    int d, M, dsub, ip, Pmax;
-    const int32_t* probes;
-    const int32_t* nprobe_q;
-    int Pfix;
-    const float* c_mean;
-    const float* cb;
-    int L;
-    // optional compact work: pairs e = q * Pmax + r, two ranges (NULL: every
-    // (q, r < P_q))
-    const uint32_t* pairs0;
-    const int64_t* npairs0;
-    const uint32_t* pairs1;
-    const int64_t* npairs1;
-};
-
-// Item i of the LUT pass: its (query, rank) flat index, or -1 if it does no work.
-__device__ __forceinline__ int64_t lut_item(const LutArgs& A, int64_t i, int64_t n0) {
-    if (A.pairs0) return i < n0 ? (int64_t)A.pairs0[i] : (int64_t)A.pairs1[i - n0];
-    return i;
-}
-
-__device__ __forceinline__ int64_t lut_items(const LutArgs& A, int64_t* n0) {
-    if (A.pairs0) {
-        *n0 = *A.npairs0;
-        return *n0 + *A.npairs1;
-    }
-    *n0 = 0;
-    return A.nq * A.Pmax;
-}
-
-__device__ __forceinline__ int probes_of(const LutArgs& A, int64_t q) {
-    int P = A.nprobe_q ? A.nprobe_q[q] : A.Pfix;
-    return P < 1 ? 1 : (P > A.Pmax ? A.Pmax : P);
-}
-
-// Codebook row stride in shared memory.  dsub = 2: 34 floats (codewords
-// 8-byte aligned; a half-warp reading 16 consecutive rows with 8-byte loads
-// covers all 32 banks once); else 16 dsub + 1 (odd: 32 consecutive rows fall
-// in distinct banks).
-__host__ __device__ __forceinline__ int cb_ld(int dsub) { return dsub == 2 ? 34 : PQ_K * dsub + 1; }
-
-__device__ __forceinline__ void stage_codebook(const LutArgs& A, float* cbs) {
-    const int ld = cb_ld(A.dsub), rowlen = PQ_K * A.dsub;
-    for (int e = threadIdx.x; e < A.M * rowlen; e += blockDim.x) {
-        const int j = e / rowlen;
-        cbs[j * ld + (e - j * rowlen)] = A.cb[e];
-    }
-    __syncthreads();
-}
-
-// The 16 FP32 entries of one subspace: qj, cj = the query's and the list
-// centroid's values of the subspace, cw = its codebook row in shared memory.
-// DS = dsub when fixed at compile time (2: 8-byte loads; qj and cj 8-byte
-// aligned), 0 = read from dsub.
-template <int DS>
-__device__ __forceinline__ void row_table(int dsub, int ip, const float* __restrict__ qj,
-                                          const float* __restrict__ cj, const float* cw, float (&T)[PQ_K]) {
-    if constexpr (DS == 2) {
-        const float2 qv = *reinterpret_cast<const float2*>(qj);
-        float u0 = qv.x, u1 = qv.y;
-        if (!ip) {
-            const float2 cv = *reinterpret_cast<const float2*>(cj);
-            u0 = __fsub_rn(u0, cv.x);
-            u1 = __fsub_rn(u1, cv.y);
-        }
-#pragma unroll
-        for (int i = 0; i < PQ_K; ++i) {
-            const float2 c = *reinterpret_cast<const float2*>(cw + 2 * i);
-            float acc = 0.f;
-            if (ip) {
-                acc = __fadd_rn(acc, __fmul_rn(u0, c.x));
-                acc = __fadd_rn(acc, __fmul_rn(u1, c.y));
-                T[i] = -acc;
-            } else {
-                // 0 + e0^2 is e0^2 exactly (a square is +0 or more), so the sum
-                // from 0 needs one addition; both differences and both squares
-                // as packed pairs
-                const float2 e = f2_sub(make_float2(u0, u1), c);
-                const float2 e2 = f2_mul(e, e);
-                T[i] = __fadd_rn(e2.x, e2.y);
-            }
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < PQ_K; ++i) T[i] = 0.f;
-        for (int t = 0; t < dsub; ++t) {
-            const float u = ip ? qj[t] : __fsub_rn(qj[t], cj[t]);
-#pragma unroll
-            for (int i = 0; i < PQ_K; ++i) {
-                const float c = cw[i * dsub + t];
-                if (ip) {
-                    T[i] = __fadd_rn(T[i], __fmul_rn(u, c));
-                } else {
-                    const float e = __fsub_rn(u, c);
-                    T[i] = __fadd_rn(T[i], __fmul_rn(e, e));
-                }
-            }
-        }
-        if (ip) {
-#pragma unroll
-            for (int i = 0; i < PQ_K; ++i) T[i] = -T[i];
-        }
-    }
-}
-
-// u8 entry min(255, floor((T - m) a + 1/2)) of four table entries, packed.
-// T >= m, so the argument of floor is positive (or NaN, which converts to 0
-// either way) and a conversion rounding down gives floor directly.
-__device__ __forceinline__ uint32_t quant4(const float* T, float mn, float a) {
-    uint32_t v[4];
-#pragma unroll
-    for (int i = 0; i < 4; i += 2) {  // (T - m) a + 1/2 of two entries as packed pairs
-        const float2 x = f2_add(f2_mul(f2_sub(make_float2(T[i], T[i + 1]), make_float2(mn, mn)), make_float2(a, a)),
-                                make_float2(0.5f, 0.5f));
-        v[i] = min(__float2uint_rd(x.x), 255u);
-        v[i + 1] = min(__float2uint_rd(x.y), 255u);
-    }
-    return __byte_perm(__byte_perm(v[0], v[1], 0x0040), __byte_perm(v[2], v[3], 0x0040), 0x5410);
-}
-
-// Integer bias floor(S a + 1/2) of one (query, list), S = sum_j m_j in
-// ascending j (+ -<q, c_p> first for IP), clamped to +-2^30.
-__device__ __forceinline__ int32_t lut_bias(const LutArgs& A, const float* __restrict__ qv, const float* __restrict__ cp,
-                                            const float* mins, float a) {
-    float S = 0.f;
-    if (A.ip) {
-        float dot = 0.f;
-        for (int t = 0; t < A.d; ++t) dot = __fadd_rn(dot, __fmul_rn(qv[t], cp[t]));
-        S = -dot;
-    }
-    for (int j = 0; j < A.M; ++j) S = __fadd_rn(S, mins[j]);
-    float bf = floorf(__fadd_rn(__fmul_rn(S, a), 0.5f));
-    bf = fminf(fmaxf(bf, -1073741824.f), 1073741823.f);
-    return (int32_t)bf;
-}
+// ------------------------------------------------------------------ a2: quantised LUTs (rule: lut.cuh)
 
 // Two-pass tables when a query's tables do not fit one CTA's shared memory
 // (many probes): a warp per item (query, probe rank), lane l computing the
@@ -1162,19 +994,6 @@ static size_t lut_fused_smem(int M, int dsub, int d, int Pb, int Pm) {
 static bool lut_ds2(const LutArgs& A) { return A.dsub == 2 && (reinterpret_cast<uintptr_t>(A.Q) & 7) == 0; }
 
 static int launch_luts(const LutArgs& A, uint32_t* rb, uint8_t* lut, int32_t* bias, float* scale, cudaStream_t st);
-
-// ------------------------------------------------------------------ code access
-__device__ __forceinline__ int nibble_of(const uint8_t* __restrict__ blk, int M, int j, int v) {
-    uint8_t byte = blk[j * 16 + (v >> 1)];
-    return (v & 1) ? (byte >> 4) : (byte & 15);
-}
-
-__device__ __forceinline__ int32_t scalar_dist(const uint8_t* __restrict__ lutp, int32_t b,
-                                               const uint8_t* __restrict__ blk, int M, int v) {
-    int32_t D = b;
-    for (int j = 0; j < M; ++j) D += lutp[j * 16 + nibble_of(blk, M, j, v)];
-    return D;
-}
 
 // ------------------------------------------------------------------ candidate-key selection
 // The need smallest keys of distance word h among keys[0..N) (the others
@@ -1759,7 +1578,7 @@ struct ChunkCursor {
     int c;  // chunk index within the item
 };
 
-template <int G, int SMAX, bool DIRECT, bool FULL>
+template <int G, int SMAX, bool DIRECT, bool FULL, bool REC>
 __global__ void __launch_bounds__(SCAN_WARPS * 32, (SMAX <= 2 ? 3 : (SMAX <= 8 ? 2 : 1))) k_scan(ScanArgs A, ScanOut O, const int64_t* __restrict__ pair_off,
                                                           const int64_t* __restrict__ item_off,
                                                           const uint32_t* __restrict__ pairs, int L, int TB,
@@ -1784,7 +1603,17 @@ __global__ void __launch_bounds__(SCAN_WARPS * 32, (SMAX <= 2 ? 3 : (SMAX <= 8 ?
     const int S = (M + G - 1) / G;
     const int blk_bytes = M * 16;
     const int cb = CHUNK / blk_bytes;  // blocks per chunk (>= 1)
-    const int64_t total = item_off[L];
+    // REC: items given one by one (a small batch: one pair each), else located
+    // in the cluster-major work list
+    const int64_t total = REC ? (int64_t)*O.nrec : item_off[L];
+    auto locate = [&](int64_t i) -> ScanItem {
+        if constexpr (REC) {
+            const int4 r = __ldg(O.recs + i);
+            return ScanItem{r.w, r.y, r.z, (int64_t)r.x, 1};
+        } else {
+            return locate_item(A, pair_off, item_off, L, TB, QG, i);
+        }
+    };
     const int64_t stride = (int64_t)gridDim.x * SCAN_WARPS;
     uint8_t* mybuf = bufs + (size_t)warp * 2 * CHUNK;
     uint4* sel = reinterpret_cast<uint4*>(bufs + (size_t)SCAN_WARPS * 2 * CHUNK) + (size_t)warp * 4 * M;
@@ -1810,7 +1639,7 @@ __global__ void __launch_bounds__(SCAN_WARPS * 32, (SMAX <= 2 ? 3 : (SMAX <= 8 ?
     };
     int64_t it = (int64_t)blockIdx.x * SCAN_WARPS + warp;
     if (it >= total) return;
-    ScanItem x = locate_item(A, pair_off, item_off, L, TB, QG, it), nx = x;
+    ScanItem x = locate(it), nx = x;
     if (lane == 0) issue(x, 0, 0);
     uint32_t phase[2] = {0u, 0u};
     int b = 0;
@@ -1834,9 +1663,9 @@ __global__ void __launch_bounds__(SCAN_WARPS * 32, (SMAX <= 2 ? 3 : (SMAX <= 8 ?
         uint32_t thI = 0;
         int64_t noff = 0;
         if (active) {
-            const uint32_t e = pairs[x.g0 + pi];
+            const uint32_t e = REC ? (uint32_t)x.g0 : pairs[x.g0 + pi];
             q = e / A.Pmax;
-            if (direct) noff = near_offset(A, q, (int)(e - q * A.Pmax));
+            if (direct) noff = REC ? (int64_t)O.noff[e] : near_offset(A, q, (int)(e - q * A.Pmax));
             const uint4* lp = reinterpret_cast<const uint4*>(A.lut + (int64_t)e * M * PQ_K);
 #pragma unroll
             for (int u = 0; u < SMAX; ++u) {
@@ -1884,7 +1713,7 @@ __global__ void __launch_bounds__(SCAN_WARPS * 32, (SMAX <= 2 ? 3 : (SMAX <= 8 ?
         const int64_t next_it = it + stride;
         for (int c = 0; c < nch; ++c) {
             // prefetch the chunk after this one into the other buffer
-            if (c + 1 == nch && next_it < total) nx = locate_item(A, pair_off, item_off, L, TB, QG, next_it);
+            if (c + 1 == nch && next_it < total) nx = locate(next_it);
             if (lane == 0) {
                 if (c + 1 < nch) issue(x, c + 1, b ^ 1);
                 else if (next_it < total) issue(nx, 0, b ^ 1);
@@ -2548,9 +2377,7 @@ __global__ void __launch_bounds__(NT) k_select_cta(ScanArgs A, int Rmax, const i
     if (threadIdx.x == 0 && ncand) ncand[q] = K;
 }
 
-// Queries whose candidate store overflowed, redone exactly: every key of every
-// probed list is recomputed (scalar lookups) inside the radix select.  A
-// persistent grid walks the redo list (usually empty).
+// The queries on the redo list.  A persistent grid walks it (usually empty).
 __global__ void __launch_bounds__(256) k_select_redo(ScanArgs A, int Rmax, int sel_cap, uint64_t* __restrict__ topr,
                                                      int32_t* __restrict__ ncand, const int32_t* __restrict__ redo) {
     extern __shared__ uint64_t sbuf[];  // sel_cap keys
@@ -2561,169 +2388,29 @@ __global__ void __launch_bounds__(256) k_select_redo(ScanArgs A, int Rmax, int s
         const int64_t q = redo[1 + r0];
         const int R = rerank_of(A.rerank_q, A.Rfix, A.Rmin, Rmax, q);
         uint64_t* out = topr + q * Rmax;
-        const int P = nprobe_of(A, q);
-        __syncthreads();  // s_pref of the previous query is no longer read
-        if (threadIdx.x == 0) {
-            int acc = 0;
-            for (int r = 0; r < P; ++r) {
-                s_pref[r] = acc;
-                const int p = A.probes[q * A.Pmax + r];
-                acc += (p >= 0 && p < A.L) ? A.list_n[p] : 0;
-            }
-            s_pref[P] = acc;
-        }
-        __syncthreads();
-        const int N = s_pref[P];
-        auto load = [&](int i) -> uint64_t {
-            int lo = 0, hi = P - 1;
-            while (lo < hi) {
-                int mid = (lo + hi + 1) >> 1;
-                if (s_pref[mid] <= i) lo = mid; else hi = mid - 1;
-            }
-            const int64_t item = q * A.Pmax + lo;
-            const int p = A.probes[item];
-            const int m = i - s_pref[lo];
-            const int64_t blk = A.boff[p] + (m >> 5);
-            const int v = m & 31;
-            int32_t D = scalar_dist(A.lut + item * A.M * PQ_K, A.bias[item], A.codes + blk * A.M * 16, A.M, v);
-            return make_key(D, A.ids[blk * 32 + v]);
-        };
-        const int K = min(R, N);
-        block_select_smallest(load, N, K, out, sbuf, sel_cap, hist);
+        const int K = redo_select(A, q, R, out, sbuf, sel_cap, hist, s_pref);
         for (int i = K + threadIdx.x; i < Rmax; i += blockDim.x) out[i] = KEY_NONE;
         if (threadIdx.x == 0 && ncand) ncand[q] = K;
     }
 }
 
 // ------------------------------------------------------------------ a6: rerank
-// Exact distance of each candidate (warp per candidate, 16-byte loads when d
-// is a multiple of 4): L2 = sum (q_t - x_t)^2, IP = -<q, x>; the k best by
-// (distance, id).  Output: L2 distance ascending / IP similarity descending.
+// A CTA per query (rerank.cuh): the candidates' exact distances, the k best.
 template <int NT>
 __global__ void __launch_bounds__(NT) k_rerank(const float* __restrict__ Q, const float* __restrict__ X, int d,
                                                 int ip, const uint64_t* __restrict__ topr, int Rmax,
                                                 const int32_t* __restrict__ rerank_q, int Rfix, int k,
                                                 int64_t* __restrict__ out_ids, float* __restrict__ out_d) {
-    extern __shared__ uint64_t keys[];
+    extern __shared__ uint64_t keys[];  // Rmax keys, then KSC_MAX_K for the selection of more than RR_RANK_R
     __shared__ __align__(16) float qs[KSC_MAX_DIM];
     const int64_t q = blockIdx.x;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int R = rerank_of(rerank_q, Rfix, k, Rmax, q);
     for (int t = threadIdx.x; t < d; t += blockDim.x) qs[t] = Q[q * d + t];
     // the candidate keys staged in shared memory (each row load then waits
-    // for a shared load); each slot is later replaced by its FP32 key by
-    // the one warp that read it
+    // for a shared load)
     for (int c = threadIdx.x; c < R; c += blockDim.x) keys[c] = topr[q * Rmax + c];
     __syncthreads();
-    const uint64_t* cq = keys;
-    const bool vec4 = (d & 3) == 0;
-    if (vec4 && d <= 128) {
-        // one float4 per lane per row; four rows in flight per warp
-        const bool inl = lane * 4 < d;
-        const float4 qv = inl ? *reinterpret_cast<const float4*>(qs + lane * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int c0 = w * 4; c0 < R; c0 += nw * 4) {
-            float4 xv[4];
-            int32_t idv[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint64_t kk = c0 + u < R ? cq[c0 + u] : KEY_NONE;
-                idv[u] = kk != KEY_NONE ? (int32_t)(kk & 0xffffffffu) : -1;
-                xv[u] = (idv[u] >= 0 && inl) ? __ldg(reinterpret_cast<const float4*>(X + (int64_t)idv[u] * d) + lane)
-                                             : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                float s = 0.f;
-                if (ip) {
-                    s = qv.x * xv[u].x + qv.y * xv[u].y + qv.z * xv[u].z + qv.w * xv[u].w;
-                } else {
-                    const float e0 = qv.x - xv[u].x, e1 = qv.y - xv[u].y, e2 = qv.z - xv[u].z, e3 = qv.w - xv[u].w;
-                    s = fmaf(e0, e0, fmaf(e1, e1, fmaf(e2, e2, e3 * e3)));
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                __syncwarp();  // (every lane read the step's keys before they are replaced)
-                if (lane == 0 && c0 + u < R)
-                    keys[c0 + u] = idv[u] >= 0 ? (((uint64_t)ordered_f32(ip ? -s : s) << 32) | (uint32_t)idv[u])
-                                               : KEY_NONE;
-            }
-        }
-    } else
-    for (int c = w; c < R; c += nw) {
-        const uint64_t kk = cq[c];
-        uint64_t outk = KEY_NONE;
-        if (kk != KEY_NONE) {
-            const int32_t id = (int32_t)(kk & 0xffffffffu);
-            const float* x = X + (int64_t)id * d;
-            float s = 0.f;
-            if (vec4) {
-                for (int t = lane * 4; t < d; t += 128) {
-                    float4 xv = __ldg(reinterpret_cast<const float4*>(x + t));
-                    float4 qv = *reinterpret_cast<const float4*>(qs + t);
-                    if (ip) {
-                        s = fmaf(qv.x, xv.x, s); s = fmaf(qv.y, xv.y, s);
-                        s = fmaf(qv.z, xv.z, s); s = fmaf(qv.w, xv.w, s);
-                    } else {
-                        float e0 = qv.x - xv.x, e1 = qv.y - xv.y, e2 = qv.z - xv.z, e3 = qv.w - xv.w;
-                        s = fmaf(e0, e0, s); s = fmaf(e1, e1, s); s = fmaf(e2, e2, s); s = fmaf(e3, e3, s);
-                    }
-                }
-            } else {
-                for (int t = lane; t < d; t += 32) {
-                    float xv = __ldg(x + t);
-                    if (ip) s = fmaf(qs[t], xv, s);
-                    else { float e = qs[t] - xv; s = fmaf(e, e, s); }
-                }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            const float dist = ip ? -s : s;
-            outk = ((uint64_t)ordered_f32(dist) << 32) | (uint32_t)id;
-        }
-        __syncwarp();  // (every lane read the key before it is replaced)
-        if (lane == 0) keys[c] = outk;
-    }
-    __syncthreads();
-    if (k <= 32) {
-        // k rounds of a warp minimum over the R keys (each taken key is retired)
-        if (w == 0) {
-            uint64_t mine = KEY_NONE;  // lane r keeps the r-th smallest
-            for (int r = 0; r < k; ++r) {
-                uint64_t m = KEY_NONE;
-                int at = -1;
-                for (int i = lane; i < R; i += 32) {
-                    if (keys[i] < m) { m = keys[i]; at = i; }
-                }
-                uint64_t g = m;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    const uint64_t y = __shfl_xor_sync(0xffffffffu, g, o);
-                    g = y < g ? y : g;
-                }
-                if (g != KEY_NONE && m == g) keys[at] = KEY_NONE;  // keys are unique: one lane matches
-                __syncwarp();
-                if (lane == r) mine = g;
-            }
-            if (lane < k) keys[lane] = mine;
-        }
-        __syncthreads();
-    } else {
-        const int S = pow2_ceil(R < 2 ? 2 : R);
-        for (int i = R + threadIdx.x; i < S; i += blockDim.x) keys[i] = KEY_NONE;
-        __syncthreads();
-        block_bitonic_sort(keys, S);
-    }
-    for (int r = threadIdx.x; r < k; r += blockDim.x) {
-        const uint64_t kk = r < R ? keys[r] : KEY_NONE;
-        if (kk == KEY_NONE) {
-            out_ids[q * k + r] = -1;
-            out_d[q * k + r] = ip ? -INFINITY : INFINITY;
-        } else {
-            out_ids[q * k + r] = (int64_t)(kk & 0xffffffffu);
-            const float dist = unordered_f32((uint32_t)(kk >> 32));
-            out_d[q * k + r] = ip ? -dist : dist;
-        }
-    }
+    cta_rerank<NT>(keys, R, keys + Rmax, qs, X, d, ip, k, out_ids + q * k, out_d + q * k);
 }
 
 // One warp per query (8 per CTA) when k <= 32, R <= RW_MAXR, d <= 128 and
@@ -2756,55 +2443,6 @@ __global__ void __launch_bounds__(NT) k_rerank(const float* __restrict__ Q, cons
 // plain pass's.
 constexpr int RW_WARPS = 8;
 constexpr int RW_MAXR = 512;
-
-// Halving exchange of 8 rows' partial sums over the warp (9 shuffles):
-// afterwards every lane of quad `myrow` (lane bits 4, 3, 2) holds that row's
-// total, summed in the same tree for every row.
-__device__ __forceinline__ float exchange_rows8(float (&a)[8], int lane) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const bool up = lane & 16;
-        const float send = up ? a[i] : a[i + 4], keep = up ? a[i + 4] : a[i];
-        a[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const bool up = lane & 8;
-        const float send = up ? a[i] : a[i + 2], keep = up ? a[i + 2] : a[i];
-        a[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-    }
-    {
-        const bool up = lane & 4;
-        const float send = up ? a[0] : a[1], keep = up ? a[1] : a[0];
-        a[0] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-    }
-    a[0] += __shfl_xor_sync(0xffffffffu, a[0], 2);
-    a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
-    return a[0];
-}
-
-// FP32 partial sums of the 8 rows idv[] (-1: none) for this lane's 4
-// coordinates, summed across the warp: every lane of quad `myrow` ends with
-// that row's distance term (L2: the squared distance, IP: the dot product).
-__device__ __forceinline__ float rerank_rows8(const float4& qv, const float* __restrict__ X, int d, int ip, bool inl,
-                                              const int32_t (&idv)[8], int lane) {
-    float4 xv[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-        xv[u] = (idv[u] >= 0 && inl) ? __ldg(reinterpret_cast<const float4*>(X + (int64_t)idv[u] * d) + lane)
-                                     : make_float4(0.f, 0.f, 0.f, 0.f);
-    float a[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-        if (ip) {
-            a[u] = qv.x * xv[u].x + qv.y * xv[u].y + qv.z * xv[u].z + qv.w * xv[u].w;
-        } else {
-            const float e0 = qv.x - xv[u].x, e1 = qv.y - xv[u].y, e2 = qv.z - xv[u].z, e3 = qv.w - xv[u].w;
-            a[u] = fmaf(e0, e0, fmaf(e1, e1, fmaf(e2, e2, e3 * e3)));
-        }
-    }
-    return exchange_rows8(a, lane);
-}
 
 // The distance terms of 16 low-precision rows at once, 8 lanes per row:
 // lane l = 8 h + j takes rows 4 h .. 4 h + 3 of the step (idv[], -1: none)
@@ -3222,6 +2860,18 @@ static void mark(ksc_index* ix, int i, cudaStream_t st) {
     ix->ev_used[i] = true;
 }
 
+// Status word, item counts and counters of a search, cleared in one go (they
+// share an allocation: index.cuh).
+static int reset_counters(ksc_index* ix, cudaStream_t st) {
+    KSC_CUDA(cudaMemsetAsync(ix->status, 0, STATUS_BYTES, st));
+    return KSC_OK;
+}
+// The item counts alone (searches inside a training call keep the rest).
+static int reset_items(ksc_index* ix, cudaStream_t st) {
+    KSC_CUDA(cudaMemsetAsync(ix->status + STATUS_NREC, 0, 2 * sizeof(int32_t), st));
+    return KSC_OK;
+}
+
 static unsigned blocks_for(int64_t work, int threads) { return (unsigned)((work + threads - 1) / threads); }
 
 struct Plan {
@@ -3238,6 +2888,10 @@ struct Plan {
     int Pq_max;    // bound on the per-query nprobe (<= Pmax)
     bool tc;       // scan on the tensor cores (k_scan_tc)
     int nt;        // its queries per item
+    bool small;    // the small-batch kernels (small.cu) around the scan,
+    bool rank;     // which also rank the lists (no ranking has run)
+    bool all_near; // no filtered part: the store holds every key a query can probe
+    int64_t nrec;  // bound on the scan items of either part
 };
 
 static int choose_G(const ksc_index* ix, int64_t nq, int Pmax, int want) {
@@ -3264,8 +2918,10 @@ static int launch_scan(const ScanArgs& A, const ScanOut& O, const int64_t* pair_
                         (scan_shared_sel<G>() ? (size_t)SCAN_WARPS * A.M * 64 : 0);
     // M = G SMAX: every lane has SMAX subspaces, no per-subspace guards
     const bool full = A.M == G * SMAX;
-    auto kern = O.thr ? (full ? k_scan<G, SMAX, false, true> : k_scan<G, SMAX, false, false>)
-                      : (full ? k_scan<G, SMAX, true, true> : k_scan<G, SMAX, true, false>);
+    auto kern = O.thr ? (full ? k_scan<G, SMAX, false, true, false> : k_scan<G, SMAX, false, false, false>)
+                      : (full ? k_scan<G, SMAX, true, true, false> : k_scan<G, SMAX, true, false, false>);
+    if constexpr (G <= 16)
+        if (O.recs) kern = O.thr ? k_scan<G, SMAX, false, false, true> : k_scan<G, SMAX, true, false, true>;
     KSC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
     KSC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, SCAN_WARPS * 32, smem));
@@ -3551,6 +3207,229 @@ static int work_queries(ksc_index* ix, const float* Q, int64_t nq, cudaStream_t 
     return KSC_OK;
 }
 
+// 6. exact rerank of the selected keys topr (precision variant: a BF16 / FP8
+//    re-rank of the widened shortlist first, then FP32 of its best Rf), with
+//    the full queries and vectors (Alg. 2: q_init)
+static int rerank_stage(ksc_index* ix, const float* Qr, const Plan& pl, const uint64_t* topr, int64_t* ids,
+                        float* dists, cudaStream_t st) {
+    const int64_t nq = pl.nq;
+    mark(ix, 6, st);
+    const float* Xr = rr_X(ix);
+    const int dr = rr_d(ix);
+    const uint64_t* rr_keys = topr;
+    int rr_R = pl.Rmax;
+    const int32_t* rr_q = pl.rerank_q;
+    if (pl.prec > 0) {
+        KSC_TRY(ensure_lowp(ix, pl.prec, st));
+        KSC_TRY(ensure(ix->ws_topr2, sizeof(uint64_t) * nq * pl.Rf, st));
+        uint64_t* topr2 = (uint64_t*)ix->ws_topr2.p;
+        const size_t smem = sizeof(uint64_t) * pow2_ceil(pl.Rmax < 2 ? 2 : pl.Rmax);
+        KSC_CUDA(cudaFuncSetAttribute(k_rerank_lowp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        k_rerank_lowp<<<(unsigned)nq, 256, smem, st>>>(Qr, dr, ix->metric == KSC_IP, pl.prec,
+                                                       (const uint16_t*)ix->X_bf16, (const uint8_t*)ix->X_fp8,
+                                                       ix->X_scale, topr, pl.Rmax, pl.rerank_q, pl.Rfix, pl.k, pl.Rf,
+                                                       topr2);
+        KSC_LAUNCH_CHECK();
+        ix->launches++;
+        rr_keys = topr2;
+        rr_R = pl.Rf;
+        rr_q = nullptr;
+    }
+    if (pl.k <= 32 && rr_R <= RW_MAXR && dr <= 128 && (dr & 3) == 0 && warp_per_query(nq)) {
+        const bool band = pl.band && pl.prec == 0 && rr_R > pl.k;
+        if (band) KSC_TRY(ensure_band(ix, st));
+        const size_t smem = sizeof(uint64_t) * RW_WARPS * rr_R * (band ? 2 : 1) +
+                            (band ? sizeof(uint32_t) * RW_WARPS * (rr_R + 64) : 0);
+        auto kr = band && ix->x_u8_state == 1 ? k_rerank_w<true> : k_rerank_w<false>;
+        KSC_CUDA(cudaFuncSetAttribute(kr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        kr<<<(unsigned)((nq + RW_WARPS - 1) / RW_WARPS), RW_WARPS * 32, smem, st>>>(
+            Qr, Xr, dr, ix->metric == KSC_IP, rr_keys, rr_R, rr_q, rr_R, pl.k, nq, ids, dists,
+            band && ix->x_u8_state != 1 ? (const uint16_t*)ix->X_bf16 : nullptr,
+            band && ix->x_u8_state == 1 ? (const uint8_t*)ix->X_u8 : nullptr, band ? ix->X_band : nullptr);
+        ix->launches++;
+        KSC_LAUNCH_CHECK();
+    } else {
+        const size_t smem = rerank_smem(rr_R, pl.k);
+        // a CTA per query; 1024 threads (more rows in flight) when the batch is
+        // too small to fill the GPU with 256-thread CTAs
+        if (nq < 2 * (int64_t)num_sms()) {
+            KSC_CUDA(cudaFuncSetAttribute(k_rerank<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            k_rerank<1024><<<(unsigned)nq, 1024, smem, st>>>(Qr, Xr, dr, ix->metric == KSC_IP, rr_keys, rr_R, rr_q,
+                                                             rr_R, pl.k, ids, dists);
+        } else {
+            KSC_CUDA(cudaFuncSetAttribute(k_rerank<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            k_rerank<256><<<(unsigned)nq, 256, smem, st>>>(Qr, Xr, dr, ix->metric == KSC_IP, rr_keys, rr_R, rr_q,
+                                                           rr_R, pl.k, ids, dists);
+        }
+        ix->launches++;
+        KSC_LAUNCH_CHECK();
+    }
+    mark(ix, KSC_NUM_STAGES, st);
+    return KSC_OK;
+}
+
+// 5. the R best keys per query into topr (and, sorted, cand_out)
+static int select_stage(ksc_index* ix, const Plan& pl, const ScanArgs& A, const int32_t* cnt, const uint64_t* cand,
+                        uint64_t* topr, uint64_t* cand_out, int32_t* ncand_out, cudaStream_t st) {
+    const int64_t nq = pl.nq;
+    {
+        KSC_TRY(ensure(ix->ws_redo, sizeof(int32_t) * (nq + 1), st));
+        int32_t* redo = (int32_t*)ix->ws_redo.p;
+        KSC_CUDA(cudaMemsetAsync(redo, 0, sizeof(int32_t), st));
+        // candidates per query: the R kept by the threshold plus a few R more
+        if (4 * pl.Rmax <= SW_MAX_KEYS && warp_per_query(nq))
+            k_select<<<(unsigned)((nq + SW_WARPS - 1) / SW_WARPS), SW_WARPS * 32, 0, st>>>(
+                A, pl.Rmax, cnt, cand, pl.cap, topr, ncand_out, ix->status, ix->stats, redo);
+        else if (nq < 2 * (int64_t)num_sms())  // few queries: more threads per query
+            k_select_cta<1024><<<(unsigned)nq, 1024, 0, st>>>(A, pl.Rmax, cnt, cand, pl.cap, topr, ncand_out,
+                                                               ix->status, ix->stats, redo);
+        else
+            k_select_cta<256><<<(unsigned)nq, 256, 0, st>>>(A, pl.Rmax, cnt, cand, pl.cap, topr, ncand_out,
+                                                             ix->status, ix->stats, redo);
+        KSC_LAUNCH_CHECK();
+        // overflowed queries (usually none): radix select over recomputed keys,
+        // the R best plus their sort in a buffer of sel_cap keys
+        const int sel_cap = sel_keys(pl.Rmax);
+        const size_t smem = sel_cap * sizeof(uint64_t);
+        KSC_CUDA(cudaFuncSetAttribute(k_select_redo, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        k_select_redo<<<num_sms() * 2, 256, smem, st>>>(A, pl.Rmax, sel_cap, topr, ncand_out, redo);
+        KSC_LAUNCH_CHECK();
+        ix->launches += 2;
+    }
+    if (cand_out) {
+        const size_t csm = sizeof(uint64_t) * pow2_ceil(pl.Rmax < 2 ? 2 : pl.Rmax);
+        KSC_CUDA(cudaFuncSetAttribute(k_copy_cands, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm));
+        k_copy_cands<<<(unsigned)nq, 256, csm, st>>>(topr, pl.Rmax, cand_out);
+        ix->launches++;
+        KSC_LAUNCH_CHECK();
+    }
+    return KSC_OK;
+}
+
+// The search of a few queries (small.cu).
+static int search_small(ksc_index* ix, const float* Q, const Plan& pl, const int32_t* probes, int64_t* ids,
+                        float* dists, uint64_t* cand_out, int32_t* ncand_out, cudaStream_t st, const float* Qr) {
+    const int64_t nq = pl.nq;
+    const int M = ix->M;
+    KSC_TRY(ensure(ix->ws_lut, (size_t)nq * pl.Pmax * M * PQ_K, st));
+    KSC_TRY(ensure(ix->ws_bias, sizeof(int32_t) * nq * pl.Pmax, st));
+    KSC_TRY(ensure(ix->ws_scale, sizeof(float) * nq, st));
+    KSC_TRY(ensure(ix->ws_thr, sizeof(uint64_t) * nq, st));
+    KSC_TRY(ensure(ix->ws_cnt, sizeof(int32_t) * nq, st));
+    KSC_TRY(ensure(ix->ws_cand, sizeof(uint64_t) * nq * pl.cap, st));
+    KSC_TRY(ensure(ix->ws_topr, sizeof(uint64_t) * nq * pl.Rmax, st));
+    KSC_TRY(ensure(ix->ws_items, sizeof(int4) * 2 * pl.nrec + sizeof(int32_t) * nq * pl.Pmax, st));
+    int32_t* bias = (int32_t*)ix->ws_bias.p;
+    uint8_t* lut = (uint8_t*)ix->ws_lut.p;
+    int32_t* cnt = (int32_t*)ix->ws_cnt.p;
+    uint64_t* thr = (uint64_t*)ix->ws_thr.p;
+    uint64_t* cand = (uint64_t*)ix->ws_cand.p;
+    uint64_t* topr = (uint64_t*)ix->ws_topr.p;
+    int4* recs = (int4*)ix->ws_items.p;
+    int32_t* nrec = ix->status + STATUS_NREC;
+    ScanArgs A{M, pl.Pmax, nq, probes, pl.nprobe_q, pl.Pfix, pl.rerank_q, pl.Rfix, pl.k, lut, bias,
+               ix->list_boff, ix->list_n, ix->blk_codes, ix->blk_ids, ix->L};
+    SmallPrep S{};
+    S.T = LutArgs{Q, nq, ix->d, M, ix->dsub, ix->metric == KSC_IP, pl.Pmax, probes, pl.nprobe_q, pl.Pfix, ix->c_mean,
+                  ix->codebook, ix->L};
+    S.A = A;
+    S.c_rank = pl.rank ? ix->c_rank : nullptr;
+    S.spherical = ix->spherical;
+    S.probes_out = const_cast<int32_t*>(probes);  // written only when pl.rank: then the handle's own buffer
+    S.lut = lut;
+    S.bias = bias;
+    S.scale = (float*)ix->ws_scale.p;
+    S.cnt = cnt;
+    S.noff = (int32_t*)(recs + 2 * pl.nrec);
+    S.recsA = recs;
+    S.recsB = recs + pl.nrec;
+    S.nrec = nrec;
+    S.TBa = pl.TBa;
+    S.TB = pl.TB;
+    S.Rmax = pl.Rmax;
+    S.cap = pl.cap;
+    S.all_near = pl.all_near;
+    S.near_keys_per_r = NEAR_KEYS_PER_R;
+    S.near_share_div = NEAR_SHARE_DIV;
+    KSC_TRY(launch_small_prep(S, st));
+    ix->launches++;
+    for (int i = 1; i <= 3; ++i) mark(ix, i, st);
+    const WorkList none{};
+    KSC_TRY(run_scan(pl, M, A, ScanOut{nullptr, cnt, cand, pl.cap, S.recsA, nrec, S.noff}, none, ix->L, ix->status, st,
+                     nullptr, false));
+    ix->launches++;
+    if (!pl.all_near) {
+        k_threshold_cta<1024><<<(unsigned)nq, 1024, 0, st>>>(A, pl.Rmax, cnt, cand, pl.cap, topr, thr);
+        KSC_LAUNCH_CHECK();
+        ix->launches++;
+    }
+    mark(ix, 4, st);
+    if (!pl.all_near) {
+        KSC_TRY(run_scan(pl, M, A, ScanOut{thr, cnt, cand, pl.cap, S.recsB, nrec + 1, S.noff}, none, ix->L, ix->status,
+                         st, nullptr, false));
+        ix->launches++;
+    }
+    mark(ix, 5, st);
+    if (cand_out || pl.prec > 0 || !ids) {
+        KSC_TRY(select_stage(ix, pl, A, cnt, cand, topr, cand_out, ncand_out, st));
+        if (!ids && !dists) {  // candidates only
+            mark(ix, 6, st);
+            mark(ix, KSC_NUM_STAGES, st);
+            return KSC_OK;
+        }
+        return rerank_stage(ix, Qr, pl, topr, ids, dists, st);
+    }
+    KSC_TRY(launch_select_rerank(A, pl.Rmax, cnt, cand, pl.cap, pl.all_near ? 0 : sel_keys(pl.Rmax), Qr, rr_X(ix),
+                                 rr_d(ix), ix->metric == KSC_IP, pl.k, ids, dists, ix->status, ix->stats, st));
+    ix->launches++;
+    mark(ix, 6, st);
+    mark(ix, KSC_NUM_STAGES, st);
+    return KSC_OK;
+}
+
+// Whether the small-batch kernels serve this search (small.cu).  They give a
+// query a cluster and a CTA of its own, so they pay off while those fill the
+// GPU at most about twice (2 SMs' worth of queries: the general kernels then
+// share lists and tables between queries); the rest are limits of their
+// buffers.  distinct: no list occurs twice in a query's probes (a ranking);
+// can_rank: the lists are not ranked yet.
+//  - ranking: every list is scored exactly by the query's own cluster, L d
+//    floats from L2 per query: up to SMALL_RANK_BYTES over the batch (at 1024 x
+//    128, one query: RK_SMALL us in all against 20 us of the three ranking
+//    kernels; at 128 queries the reads equal the tensor cores' time).
+//  - all_near: if no query can probe more than SMALL_NEAR_KEYS keys, the store
+//    holds all of them and the threshold, the second scan and its items go.
+constexpr int64_t SMALL_RANK_BYTES = 64 << 20;
+constexpr int64_t SMALL_NEAR_KEYS = 32768;
+constexpr int64_t SMALL_MAX_RECS = 1 << 22;
+static void plan_small(const ksc_index* ix, Plan& pl, const ksc_search_opts* opts, bool distinct, bool can_rank) {
+    const int64_t nq = pl.nq, P = pl.Pmax;
+    if (nq == 0 || nq >= 2 * (int64_t)num_sms() || pl.hybrid || pl.tc || (pl.G != 8 && pl.G != 16) || P > SP_MAX_P ||
+        nq * P > 65536 || P * ix->max_list >= (1ll << 31))
+        return;
+    const int64_t maxb = (ix->max_list + 31) / 32;
+    const int64_t blocks = distinct ? ix->h_top_blocks[P] : P * maxb;
+    const int64_t keys = std::min(32 * blocks, P * (int64_t)ix->max_list);
+    const bool own_cap = opts && opts->cand_cap > 0;
+    const bool near = keys <= (own_cap ? std::min<int64_t>(pl.cap, SMALL_NEAR_KEYS) : SMALL_NEAR_KEYS);
+    int TB = pl.TB, TBa = pl.TBa;
+    if (!(opts && opts->tile_blocks > 0)) {
+        // a pair per item: about 8 items per warp of the scan, 4 to 32 blocks each
+        const double per = (double)nq * P * ix->nblocks / ix->L / (60.0 * num_sms());
+        TB = TBa = per < 4 ? 4 : (per > 32 ? 32 : (int)per);
+    }
+    const int64_t nrec = nq * (P + blocks / std::min(TB, TBa) + 1);
+    if (nrec > SMALL_MAX_RECS) return;
+    pl.small = true;
+    pl.all_near = near;
+    if (near && !own_cap) pl.cap = (int)std::max<int64_t>(pl.cap, keys);
+    pl.TB = TB;
+    pl.TBa = TBa;
+    pl.nrec = nrec;
+    pl.rank = can_rank && pl.rank_mode == RANK_TC16 && ix->L <= SP_RANK_L && P <= SP_RANK_P &&
+              nq * (int64_t)ix->L * ix->d * 4 <= SMALL_RANK_BYTES;
+}
+
 // Q: the queries in the index's (working) dimensions; Qr: the same queries
 // with all their dimensions for the re-rank (null: Q; they differ only under
 // component filtration).
@@ -3559,6 +3438,8 @@ static int search_from_probes(ksc_index* ix, const float* Q, const Plan& pl, con
                               const float* Qr = nullptr) {
     const int64_t nq = pl.nq;
     const int M = ix->M, L = ix->L;
+    if (!Qr) Qr = Q;
+    if (pl.small) return search_small(ix, Q, pl, probes, ids, dists, cand_out, ncand_out, st, Qr);
     // queries per work item: the unfiltered first part always runs the
     // byte-permute scan (few queries share a list there: too few columns for
     // the tensor cores); the rest the chosen scan
@@ -3692,98 +3573,12 @@ static int search_from_probes(ksc_index* ix, const float* Q, const Plan& pl, con
     ix->launches++;
     // 5. the R best keys per query
     mark(ix, 5, st);
-    {
-        KSC_TRY(ensure(ix->ws_redo, sizeof(int32_t) * (nq + 1), st));
-        int32_t* redo = (int32_t*)ix->ws_redo.p;
-        KSC_CUDA(cudaMemsetAsync(redo, 0, sizeof(int32_t), st));
-        // candidates per query: the R kept by the threshold plus a few R more
-        if (4 * pl.Rmax <= SW_MAX_KEYS && warp_per_query(nq))
-            k_select<<<(unsigned)((nq + SW_WARPS - 1) / SW_WARPS), SW_WARPS * 32, 0, st>>>(
-                A, pl.Rmax, cnt, cand, pl.cap, topr, ncand_out, ix->status, ix->stats, redo);
-        else if (nq < 2 * (int64_t)num_sms())  // few queries: more threads per query
-            k_select_cta<1024><<<(unsigned)nq, 1024, 0, st>>>(A, pl.Rmax, cnt, cand, pl.cap, topr, ncand_out,
-                                                               ix->status, ix->stats, redo);
-        else
-            k_select_cta<256><<<(unsigned)nq, 256, 0, st>>>(A, pl.Rmax, cnt, cand, pl.cap, topr, ncand_out,
-                                                             ix->status, ix->stats, redo);
-        KSC_LAUNCH_CHECK();
-        // overflowed queries (usually none): radix select over recomputed keys,
-        // the R best plus their sort in a buffer of sel_cap keys
-        const int sel_cap = sel_keys(pl.Rmax);
-        const size_t smem = sel_cap * sizeof(uint64_t);
-        KSC_CUDA(cudaFuncSetAttribute(k_select_redo, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_select_redo<<<num_sms() * 2, 256, smem, st>>>(A, pl.Rmax, sel_cap, topr, ncand_out, redo);
-        KSC_LAUNCH_CHECK();
-        ix->launches += 2;
-    }
-    if (cand_out) {
-        const size_t csm = sizeof(uint64_t) * pow2_ceil(pl.Rmax < 2 ? 2 : pl.Rmax);
-        KSC_CUDA(cudaFuncSetAttribute(k_copy_cands, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm));
-        k_copy_cands<<<(unsigned)nq, 256, csm, st>>>(topr, pl.Rmax, cand_out);
-        ix->launches++;
-        KSC_LAUNCH_CHECK();
-    }
+    KSC_TRY(select_stage(ix, pl, A, cnt, cand, topr, cand_out, ncand_out, st));
     if (!ids && !dists) {  // candidates only (a shard's first step): no re-rank
         mark(ix, KSC_NUM_STAGES, st);
         return KSC_OK;
     }
-    // 6. exact rerank (precision variant: a BF16 / FP8 re-rank of the widened
-    //    shortlist first, then FP32 of its best Rf), with the full queries and
-    //    vectors (Alg. 2: q_init)
-    mark(ix, 6, st);
-    if (!Qr) Qr = Q;
-    const float* Xr = rr_X(ix);
-    const int dr = rr_d(ix);
-    const uint64_t* rr_keys = topr;
-    int rr_R = pl.Rmax;
-    const int32_t* rr_q = pl.rerank_q;
-    if (pl.prec > 0) {
-        KSC_TRY(ensure_lowp(ix, pl.prec, st));
-        KSC_TRY(ensure(ix->ws_topr2, sizeof(uint64_t) * nq * pl.Rf, st));
-        uint64_t* topr2 = (uint64_t*)ix->ws_topr2.p;
-        const size_t smem = sizeof(uint64_t) * pow2_ceil(pl.Rmax < 2 ? 2 : pl.Rmax);
-        KSC_CUDA(cudaFuncSetAttribute(k_rerank_lowp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_rerank_lowp<<<(unsigned)nq, 256, smem, st>>>(Qr, dr, ix->metric == KSC_IP, pl.prec,
-                                                       (const uint16_t*)ix->X_bf16, (const uint8_t*)ix->X_fp8,
-                                                       ix->X_scale, topr, pl.Rmax, pl.rerank_q, pl.Rfix, pl.k, pl.Rf,
-                                                       topr2);
-        KSC_LAUNCH_CHECK();
-        ix->launches++;
-        rr_keys = topr2;
-        rr_R = pl.Rf;
-        rr_q = nullptr;
-    }
-    if (pl.k <= 32 && rr_R <= RW_MAXR && dr <= 128 && (dr & 3) == 0 && warp_per_query(nq)) {
-        const bool band = pl.band && pl.prec == 0 && rr_R > pl.k;
-        if (band) KSC_TRY(ensure_band(ix, st));
-        const size_t smem = sizeof(uint64_t) * RW_WARPS * rr_R * (band ? 2 : 1) +
-                            (band ? sizeof(uint32_t) * RW_WARPS * (rr_R + 64) : 0);
-        auto kr = band && ix->x_u8_state == 1 ? k_rerank_w<true> : k_rerank_w<false>;
-        KSC_CUDA(cudaFuncSetAttribute(kr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        kr<<<(unsigned)((nq + RW_WARPS - 1) / RW_WARPS), RW_WARPS * 32, smem, st>>>(
-            Qr, Xr, dr, ix->metric == KSC_IP, rr_keys, rr_R, rr_q, rr_R, pl.k, nq, ids, dists,
-            band && ix->x_u8_state != 1 ? (const uint16_t*)ix->X_bf16 : nullptr,
-            band && ix->x_u8_state == 1 ? (const uint8_t*)ix->X_u8 : nullptr, band ? ix->X_band : nullptr);
-        ix->launches++;
-        KSC_LAUNCH_CHECK();
-    } else {
-        const size_t smem = sizeof(uint64_t) * pow2_ceil(rr_R < 2 ? 2 : rr_R);
-        // a CTA per query; 1024 threads (more rows in flight) when the batch is
-        // too small to fill the GPU with 256-thread CTAs
-        if (nq < 2 * (int64_t)num_sms()) {
-            KSC_CUDA(cudaFuncSetAttribute(k_rerank<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            k_rerank<1024><<<(unsigned)nq, 1024, smem, st>>>(Qr, Xr, dr, ix->metric == KSC_IP, rr_keys, rr_R, rr_q,
-                                                             rr_R, pl.k, ids, dists);
-        } else {
-            KSC_CUDA(cudaFuncSetAttribute(k_rerank<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            k_rerank<256><<<(unsigned)nq, 256, smem, st>>>(Qr, Xr, dr, ix->metric == KSC_IP, rr_keys, rr_R, rr_q,
-                                                           rr_R, pl.k, ids, dists);
-        }
-        ix->launches++;
-        KSC_LAUNCH_CHECK();
-    }
-    mark(ix, KSC_NUM_STAGES, st);
-    return KSC_OK;
+    return rerank_stage(ix, Qr, pl, topr, ids, dists, st);
 }
 
 // Tile lengths of the scan's warp items for an expected P probes per query.
@@ -3837,6 +3632,8 @@ static int make_plan(ksc_index* ix, int64_t nq, int k, int Pmax, int Rmax, const
     pl.cap = std::max(cap, Rmax);
     pl.rank_mode = (opts && opts->rank_fp32) ? RANK_FP32 : ((opts && opts->rank_fp8) ? RANK_FP8 : RANK_TC16);
     pl.Pq_max = Pmax;
+    pl.small = pl.rank = pl.all_near = false;
+    pl.nrec = 0;
     pl.prec = opts ? opts->precision : 0;
     // the re-rank band: on by default for L2 (for inner products of
     // real-valued rows the BF16 band is wide against the gaps between the
@@ -3917,12 +3714,12 @@ int ksc_search_with_probes(ksc_index* ix, const float* Q_dev, int64_t nq, const 
     if (nq == 0) return KSC_OK;  // empty batch: pointers may be NULL
     KSC_CHECK_ARG(Q_dev && probes_dev && ids_dev && dists_dev, "null argument");
     cudaStream_t st = as_stream(stream);
-    KSC_CUDA(cudaMemsetAsync(ix->status, 0, sizeof(int32_t), st));
-    KSC_CUDA(cudaMemsetAsync(ix->stats, 0, sizeof(unsigned long long) * 4, st));
+    KSC_TRY(reset_counters(ix, st));
     ix->launches = 0;
     mark(ix, 0, st);
     const float* Qw;
     KSC_TRY(work_queries(ix, Q_dev, nq, st, &Qw));
+    plan_small(ix, pl, opts, false, false);
     return search_from_probes(ix, Qw, pl, probes_dev, ids_dev, dists_dev, cand_dev, ncand_dev, st, Q_dev);
 }
 
@@ -3938,15 +3735,15 @@ int search_keys(ksc_index* ix, const float* Q, int64_t nq, int nprobe, int reran
     KSC_TRY(make_plan(ix, nq, 1, nprobe, rerank, opts, pl));
     KSC_CHECK_ARG(!pl.hybrid && pl.prec == 0, "sharded search: plain scan and FP32 re-rank only");
     if (nq == 0) return KSC_OK;
-    KSC_CUDA(cudaMemsetAsync(ix->status, 0, sizeof(int32_t), st));
+    KSC_TRY(reset_counters(ix, st));
     KSC_TRY(ensure(ix->ws_probes, sizeof(int32_t) * nq * pl.Pmax, st));
     int32_t* probes = (int32_t*)ix->ws_probes.p;
-    KSC_CUDA(cudaMemsetAsync(ix->stats, 0, sizeof(unsigned long long) * 4, st));
     ix->launches = 0;
     mark(ix, 0, st);
     const float* Qw;
     KSC_TRY(work_queries(ix, Q, nq, st, &Qw));
-    KSC_TRY(rank_lists(ix, Qw, nq, nullptr, pl.Pmax, pl.Pmax, probes, nullptr, pl.rank_mode, st));
+    plan_small(ix, pl, opts, true, true);
+    if (!pl.rank) KSC_TRY(rank_lists(ix, Qw, nq, nullptr, pl.Pmax, pl.Pmax, probes, nullptr, pl.rank_mode, st));
     return search_from_probes(ix, Qw, pl, probes, nullptr, nullptr, keys, nullptr, st, Q);
 }
 
@@ -3963,7 +3760,7 @@ int rerank_keys(ksc_index* ix, const float* Q, int64_t nq, int k, const uint64_t
         k_rerank_w<false><<<(unsigned)((nq + RW_WARPS - 1) / RW_WARPS), RW_WARPS * 32, smem, st>>>(
             Q, Xr, dr, ip, keys, R, nullptr, R, k, nq, ids, dists, nullptr, nullptr, nullptr);
     } else {
-        const size_t smem = sizeof(uint64_t) * pow2_ceil(R < 2 ? 2 : R);
+        const size_t smem = rerank_smem(R, k);
         if (nq < 2 * (int64_t)num_sms()) {
             KSC_CUDA(cudaFuncSetAttribute(k_rerank<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             k_rerank<1024><<<(unsigned)nq, 1024, smem, st>>>(Q, Xr, dr, ip, keys, R, nullptr, R, k, ids, dists);
@@ -3988,15 +3785,15 @@ int ksc_search(ksc_index* ix, const float* Q_dev, int64_t nq, int32_t k, int32_t
     if (nq == 0) return KSC_OK;  // empty batch: pointers may be NULL
     KSC_CHECK_ARG(Q_dev && ids_dev && dists_dev, "null argument");
     cudaStream_t st = as_stream(stream);
-    KSC_CUDA(cudaMemsetAsync(ix->status, 0, sizeof(int32_t), st));
+    KSC_TRY(reset_counters(ix, st));
     KSC_TRY(ensure(ix->ws_probes, sizeof(int32_t) * nq * pl.Pmax, st));
     int32_t* probes = (int32_t*)ix->ws_probes.p;
-    KSC_CUDA(cudaMemsetAsync(ix->stats, 0, sizeof(unsigned long long) * 4, st));
     ix->launches = 0;
     mark(ix, 0, st);
     const float* Qw;
     KSC_TRY(work_queries(ix, Q_dev, nq, st, &Qw));
-    KSC_TRY(rank_lists(ix, Qw, nq, nullptr, pl.Pmax, pl.Pmax, probes, nullptr, pl.rank_mode, st));
+    plan_small(ix, pl, opts, true, true);
+    if (!pl.rank) KSC_TRY(rank_lists(ix, Qw, nq, nullptr, pl.Pmax, pl.Pmax, probes, nullptr, pl.rank_mode, st));
     return search_from_probes(ix, Qw, pl, probes, ids_dev, dists_dev, nullptr, nullptr, st, Q_dev);
 }
 
@@ -4012,15 +3809,15 @@ int ksc_search_varprobe(ksc_index* ix, const float* Q_dev, int64_t nq, int32_t k
     pl.nprobe_q = nprobe_dev;
     pl.rerank_q = rerank_dev;
     set_tiles(ix, pl, nq, 0.5 * pl.Pmax, opts);  // per-query nprobe: about half the largest on average
-    KSC_CUDA(cudaMemsetAsync(ix->status, 0, sizeof(int32_t), st));
+    KSC_TRY(reset_counters(ix, st));
     KSC_TRY(ensure(ix->ws_probes, sizeof(int32_t) * nq * pl.Pmax, st));
     int32_t* probes = (int32_t*)ix->ws_probes.p;
-    KSC_CUDA(cudaMemsetAsync(ix->stats, 0, sizeof(unsigned long long) * 4, st));
     ix->launches = 0;
     mark(ix, 0, st);
     const float* Qw;
     KSC_TRY(work_queries(ix, Q_dev, nq, st, &Qw));
-    KSC_TRY(rank_lists(ix, Qw, nq, nprobe_dev, pl.Pmax, pl.Pmax, probes, nullptr, pl.rank_mode, st));
+    plan_small(ix, pl, opts, true, true);
+    if (!pl.rank) KSC_TRY(rank_lists(ix, Qw, nq, nprobe_dev, pl.Pmax, pl.Pmax, probes, nullptr, pl.rank_mode, st));
     return search_from_probes(ix, Qw, pl, probes, ids_dev, dists_dev, nullptr, nullptr, st, Q_dev);
 }
 
@@ -4334,6 +4131,8 @@ static int label_queries(ksc_index* ix, const float* Q, const float* Qr, int64_t
             Plan pl;
             if ((rc = make_plan(ix, m, k, P, np ? gv : R_fixed, nullptr, pl))) break;
             if (np) pl.nprobe_q = npd;
+            plan_small(ix, pl, nullptr, true, false);
+            if ((rc = reset_items(ix, st))) break;
             if ((rc = search_from_probes(ix, Qs, pl, pc, ids, dists, nullptr, nullptr, st,
                                          qrc ? (part ? qrc : Qr) : Qs)))
                 break;
@@ -4558,8 +4357,7 @@ int ksc_search_adaptive(ksc_index* ix, const float* Q_dev, int64_t nq, int32_t k
     if (nq == 0) return KSC_OK;
     KSC_CHECK_ARG(Q_dev && ids_dev && dists_dev, "null argument");
     cudaStream_t st = as_stream(stream);
-    KSC_CUDA(cudaMemsetAsync(ix->status, 0, sizeof(int32_t), st));
-    KSC_CUDA(cudaMemsetAsync(ix->stats, 0, sizeof(unsigned long long) * 4, st));
+    KSC_TRY(reset_counters(ix, st));
     KSC_TRY(ensure(ix->ws_probes, sizeof(int32_t) * nq * Pr, st));
     KSC_TRY(ensure(ix->ws_nprobe, sizeof(int32_t) * nq, st));
     KSC_TRY(ensure(ix->ws_rerank, sizeof(int32_t) * nq, st));
@@ -4588,6 +4386,7 @@ int ksc_search_adaptive(ksc_index* ix, const float* Q_dev, int64_t nq, int32_t k
         pl.nprobe_q = pn;
     }
     set_tiles(ix, pl, nq, 0.5 * (prm.pmin + prm.pmax), opts);
+    plan_small(ix, pl, opts, true, false);
     KSC_TRY(search_from_probes(ix, Qw, pl, sprobes, ids_dev, dists_dev, nullptr, nullptr, st, Q_dev));
     if (nprobe_dev) KSC_CUDA(cudaMemcpyAsync(nprobe_dev, np_q, sizeof(int32_t) * nq, cudaMemcpyDeviceToDevice, st));
     if (rerank_dev) KSC_CUDA(cudaMemcpyAsync(rerank_dev, r_q, sizeof(int32_t) * nq, cudaMemcpyDeviceToDevice, st));
@@ -4861,14 +4660,13 @@ int ksc_search_pruned(ksc_index* ix, const float* Q_dev, int64_t nq, int32_t k, 
     if (nq == 0) return KSC_OK;  // empty batch: pointers may be NULL
     KSC_CHECK_ARG(Q_dev && ids_dev && dists_dev, "null argument");
     cudaStream_t st = as_stream(stream);
-    KSC_CUDA(cudaMemsetAsync(ix->status, 0, sizeof(int32_t), st));
+    KSC_TRY(reset_counters(ix, st));
     KSC_TRY(ensure(ix->ws_probes, sizeof(int32_t) * nq * pl.Pmax, st));
     KSC_TRY(ensure(ix->ws_pprobes, sizeof(int32_t) * nq * pl.Pmax, st));
     KSC_TRY(ensure(ix->ws_pn, sizeof(int32_t) * nq, st));
     int32_t* probes = (int32_t*)ix->ws_probes.p;
     int32_t* kept = (int32_t*)ix->ws_pprobes.p;
     int32_t* pn = (int32_t*)ix->ws_pn.p;
-    KSC_CUDA(cudaMemsetAsync(ix->stats, 0, sizeof(unsigned long long) * 4, st));
     ix->launches = 0;
     mark(ix, 0, st);
     const float* Qw;
@@ -4881,6 +4679,7 @@ int ksc_search_pruned(ksc_index* ix, const float* Q_dev, int64_t nq, int32_t k, 
     set_tiles(ix, pl, nq, 0.75 * pl.Pmax, opts);
     if (nprobe_out_dev)
         KSC_CUDA(cudaMemcpyAsync(nprobe_out_dev, pn, sizeof(int32_t) * nq, cudaMemcpyDeviceToDevice, st));
+    plan_small(ix, pl, opts, true, false);
     return search_from_probes(ix, Qw, pl, kept, ids_dev, dists_dev, nullptr, nullptr, st, Q_dev);
 }
 
