@@ -219,6 +219,46 @@ __device__ __forceinline__ uint64_t warp_sort_key(uint64_t v, int lane) {
 // loads per lane are in flight (the keys usually come from global memory).
 constexpr int TOPK_U = 8;
 
+// The least shift with width >> shift < 256.
+__device__ __forceinline__ int bin_shift(uint64_t width) {
+    return width < 256ull ? 0 : 56 - __clzll((long long)width);
+}
+
+// One warp: the bin that holds the need-th of the counts in hist[256] (lt: the
+// counts below it, inB: its own).  All 32 lanes get the result.
+__device__ __forceinline__ void find_bin(const uint32_t* hist, int need, int lane, int& B, int& lt, int& inB) {
+    uint32_t c[8], local = 0;
+    const uint4 h0 = *reinterpret_cast<const uint4*>(hist + 8 * lane), h1 = *reinterpret_cast<const uint4*>(hist + 8 * lane + 4);
+    c[0] = h0.x; c[1] = h0.y; c[2] = h0.z; c[3] = h0.w;
+    c[4] = h1.x; c[5] = h1.y; c[6] = h1.z; c[7] = h1.w;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) local += c[j];
+    uint32_t incl = local;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const uint32_t excl = incl - local;
+    int mb = -1, ml = 0, mi = 0;
+    if (excl < (uint32_t)need && (uint32_t)need <= incl) {
+        uint32_t acc = excl;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            if (mb < 0 && acc + c[j] >= (uint32_t)need) {
+                mb = 8 * lane + j;
+                ml = (int)acc;
+                mi = (int)c[j];
+            }
+            acc += c[j];
+        }
+    }
+    const int owner = __ffs(__ballot_sync(0xffffffffu, mb >= 0)) - 1;
+    B = __shfl_sync(0xffffffffu, mb, owner);
+    lt = __shfl_sync(0xffffffffu, ml, owner);
+    inB = __shfl_sync(0xffffffffu, mi, owner);
+}
+
 template <class Load, class Emit>
 __device__ uint64_t warp_topk(Load load, int N, int K, Emit emit, uint32_t* hist, uint64_t* bb) {
     const int lane = threadIdx.x & 31;
@@ -247,8 +287,7 @@ __device__ uint64_t warp_topk(Load load, int N, int K, Emit emit, uint32_t* hist
     }
     int out = 0, need = K;
     while (true) {
-        int shift = 0;
-        while (((hi - lo) >> shift) >= 256ull) ++shift;
+        const int shift = bin_shift(hi - lo);
         for (int b = lane; b < 256; b += 32) hist[b] = 0u;
         __syncwarp();
         for (int i0 = 0; i0 < N; i0 += 32 * TOPK_U) {
@@ -332,107 +371,134 @@ __device__ uint64_t warp_topk(Load load, int N, int K, Emit emit, uint32_t* hist
     }
 }
 
-// The same radix refinement by a whole CTA (blockDim.x a multiple of 32):
-// block-wide range, histogram and emission (positions from a shared counter,
-// so in no particular order), the bin search and the final sort of at most 32
-// keys by warp 0.  For queries with many keys.  All threads call; every
-// thread gets the K-th smallest.
-template <class Load, class Emit>
-__device__ uint64_t block_topk(Load load, int N, int K, Emit emit, uint32_t* hist, uint64_t* bb) {
-    __shared__ unsigned long long s_lo, s_hi, s_kth;
-    __shared__ int s_B, s_lt, s_inB, s_out, s_nb;
-    const int lane = threadIdx.x & 31;
+// The same radix refinement by a whole CTA (blockDim.x a multiple of 32).
+// Bound by its barriers and, with 32 warps, by the shuffles of whatever every
+// warp repeats: so the range comes from the keys' high words (two warp
+// reductions), one warp finds a pass's bin, the passes only count, and the
+// keys below the last bin are emitted in one sweep, places from a shared
+// counter, one request per warp (so in no particular order).
+// each(f) calls f(in, key) the same number of times in every thread of a warp,
+// `in` false for none: the keys of the thread.  hist: 256 words, 16-byte
+// aligned; bb: 32 keys.  The K smallest (0 < K < N) to emit(i, key); returns
+// the K-th to every thread.
+template <class Each, class Emit>
+__device__ __forceinline__ uint64_t block_topk_each(Each each, int K, Emit emit, uint32_t* hist, uint64_t* bb) {
+    __shared__ int s_out, s_nb, s_B, s_lt, s_inB;
+    __shared__ unsigned long long s_kth;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const uint32_t below = (1u << lane) - 1u;
+    uint32_t mn = 0xffffffffu, mx = 0u;
+    each([&](bool in, uint64_t k) {
+        if (in) {
+            mn = min(mn, (uint32_t)(k >> 32));
+            mx = max(mx, (uint32_t)(k >> 32));
+        }
+    });
+    mn = __reduce_min_sync(0xffffffffu, mn);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    __syncthreads();  // hist and bb are free
+    if (lane == 0) bb[w] = ((uint64_t)mx << 32) | mn;
+    for (int b = threadIdx.x; b < 256; b += blockDim.x) hist[b] = 0u;
     if (threadIdx.x == 0) {
-        s_lo = KEY_NONE;
-        s_hi = 0ull;
         s_out = 0;
+        s_nb = 0;
     }
     __syncthreads();
-    uint64_t lo = KEY_NONE, hi = 0ull;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        const uint64_t k = load(i);
-        lo = k < lo ? k : lo;
-        hi = k > hi ? k : hi;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const uint64_t a = __shfl_xor_sync(0xffffffffu, lo, o), b = __shfl_xor_sync(0xffffffffu, hi, o);
-        lo = a < lo ? a : lo;
-        hi = b > hi ? b : hi;
-    }
-    if (lane == 0) {
-        atomicMin(&s_lo, (unsigned long long)lo);
-        atomicMax(&s_hi, (unsigned long long)hi);
-    }
-    __syncthreads();
-    lo = s_lo;
-    hi = s_hi;
+    mn = __reduce_min_sync(0xffffffffu, lane < nw ? (uint32_t)bb[lane] : 0xffffffffu);
+    mx = __reduce_max_sync(0xffffffffu, lane < nw ? (uint32_t)(bb[lane] >> 32) : 0u);
+    // passes on the high words alone (32-bit compares) until the K-th key's bin
+    // is small, or a single high word: then on the whole keys
+    uint32_t lo32 = mn, width32 = mx - mn;
+    bool words = true;
+    uint64_t lo = 0ull, hi = 0ull;
     int need = K;
     while (true) {
-        int shift = 0;
-        while (((hi - lo) >> shift) >= 256ull) ++shift;
-        for (int b = threadIdx.x; b < 256; b += blockDim.x) hist[b] = 0u;
-        if (threadIdx.x == 0) s_nb = 0;
-        __syncthreads();
-        for (int i = threadIdx.x; i < N; i += blockDim.x) {
-            const uint64_t k = load(i);
-            if (k >= lo && k <= hi) atomicAdd(&hist[(uint32_t)((k - lo) >> shift)], 1u);
+        const int shift = words ? (width32 < 256u ? 0 : 24 - __clz((int)width32)) : bin_shift(hi - lo);
+        if (words) {
+            each([&](bool in, uint64_t k) {
+                const uint32_t o = (uint32_t)(k >> 32) - lo32;
+                if (in && o <= width32) atomicAdd(&hist[o >> shift], 1u);
+            });
+            lo = (uint64_t)lo32 << 32;
+            hi = ((uint64_t)(lo32 + width32) << 32) | 0xffffffffull;
+        } else {
+            each([&](bool in, uint64_t k) {
+                if (in && k >= lo && k <= hi) atomicAdd(&hist[(uint32_t)((k - lo) >> shift)], 1u);
+            });
         }
         __syncthreads();
-        if (threadIdx.x < 32) {
-            uint32_t c[8], local = 0;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                c[j] = hist[8 * lane + j];
-                local += c[j];
-            }
-            uint32_t incl = local;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
-            }
-            const uint32_t excl = incl - local;
-            if (excl < (uint32_t)need && (uint32_t)need <= incl) {
-                uint32_t acc = excl;
-                int B = -1;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    if (B < 0 && acc + c[j] >= (uint32_t)need) {
-                        B = 8 * lane + j;
-                        s_B = B;
-                        s_lt = (int)acc;
-                        s_inB = (int)c[j];
-                    }
-                    acc += c[j];
-                }
+        if (w == 0) {
+            int B, lt, inB;
+            find_bin(hist, need, lane, B, lt, inB);
+            if (lane == 0) {
+                s_B = B;
+                s_lt = lt;
+                s_inB = inB;
             }
         }
         __syncthreads();
-        const int B = s_B, lt = s_lt, inB = s_inB;
-        const uint64_t blo = lo + ((uint64_t)B << shift);
-        const uint64_t bhi = (hi - blo < (1ull << shift)) ? hi : blo + ((1ull << shift) - 1ull);
-        const bool last = inB <= 32;
-        for (int i = threadIdx.x; i < N; i += blockDim.x) {
-            const uint64_t k = load(i);
-            if (k >= lo && k < blo) emit(atomicAdd(&s_out, 1), k);
-            else if (last && k >= blo && k <= bhi) bb[atomicAdd(&s_nb, 1)] = k;
-        }
-        __syncthreads();
+        const int lt = s_lt, inB = s_inB;
+        const int sh = words ? shift + 32 : shift;  // (shift + 32 < 64: width32 is 32 bits)
+        const uint64_t blo = lo + ((uint64_t)s_B << sh);
+        const uint64_t bhi = (hi - blo < (1ull << sh)) ? hi : blo + ((1ull << sh) - 1ull);
         need -= lt;
-        if (last) {
-            if (threadIdx.x < 32) {
-                const uint64_t v = warp_sort_key(lane < inB ? bb[lane] : KEY_NONE, lane);
-                if (lane < need) emit(s_out + lane, v);
-                if (lane == need - 1) s_kth = v;
+        if (inB <= 32 || blo == bhi) {
+            each([&](bool in, uint64_t k) {
+                const bool e = in && k < blo;
+                const uint32_t m = __ballot_sync(0xffffffffu, e);
+                if (m) {
+                    int base = 0;
+                    if (lane == 0) base = atomicAdd(&s_out, __popc(m));
+                    base = __shfl_sync(0xffffffffu, base, 0);
+                    if (e) emit(base + __popc(m & below), k);
+                }
+                if (in && k >= blo && k <= bhi && inB <= 32) bb[atomicAdd(&s_nb, 1)] = k;
+            });
+            __syncthreads();
+            if (inB > 32) {  // (equal keys, more than a warp orders: any of them)
+                for (int i = threadIdx.x; i < need; i += blockDim.x) emit(s_out + i, blo);
+                __syncthreads();
+                return blo;
+            }
+            if (w == 0) {  // the bin's keys by counting the smaller (of equal ones: the earlier) ones
+                const uint64_t v = lane < inB ? bb[lane] : KEY_NONE;
+                int r = 0;
+                for (int j = 0; j < inB; ++j) r += bb[j] < v || (bb[j] == v && j < lane);
+                if (lane < inB && r < need) emit(s_out + r, v);
+                if (lane < inB && r == need - 1) s_kth = v;
             }
             __syncthreads();
             return s_kth;
         }
+        for (int b = threadIdx.x; b < 256; b += blockDim.x) hist[b] = 0u;
+        __syncthreads();
         lo = blo;
         hi = bhi;
-        __syncthreads();
+        if (words) {
+            lo32 = (uint32_t)(blo >> 32);
+            width32 = (uint32_t)(bhi >> 32) - lo32;
+            words = width32 > 0u;
+        }
     }
+}
+
+// The same for N keys given by load(i).
+template <class Load, class Emit>
+__device__ uint64_t block_topk(Load load, int N, int K, Emit emit, uint32_t* hist, uint64_t* bb) {
+    auto each = [&](auto f) {
+        for (int i0 = 0; i0 < N; i0 += 4 * blockDim.x) {  // four loads in flight per thread
+            uint64_t k[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int i = i0 + u * blockDim.x + threadIdx.x;
+                k[u] = i < N ? load(i) : KEY_NONE;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (i0 + u * (int)blockDim.x < N) f(i0 + u * (int)blockDim.x + (int)threadIdx.x < N, k[u]);
+        }
+    };
+    return block_topk_each(each, K, emit, hist, bb);
 }
 
 // ------------------------------------------------------------------ workspace

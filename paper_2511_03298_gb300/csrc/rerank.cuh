@@ -168,15 +168,21 @@ __device__ __forceinline__ void cta_rerank(uint64_t* keys, int R, uint64_t* kbuf
         }
     };
     if (R <= RR_RANK_R) {
-        for (int i = threadIdx.x; i < R; i += NT) {
-            const uint64_t v = keys[i];
+        // a group of `parts` lanes per key (a power of two, all NT threads in
+        // use), each counting every parts-th of the others
+        int parts = 1;
+        while (2 * parts * R <= NT && parts < 32) parts *= 2;
+        for (int i0 = 0; i0 < R; i0 += NT / parts) {
+            const int i = i0 + threadIdx.x / parts, o = threadIdx.x % parts;
+            const uint64_t v = i < R ? keys[i] : 0ull;
             int rank = 0;
 #pragma unroll 8
-            for (int j = 0; j < R; ++j) rank += keys[j] < v;
-            if (rank < k) put(rank, v);
+            for (int j = o; j < R; j += parts) rank += keys[j] < v;
+            for (int s = parts >> 1; s > 0; s >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, s);
+            if (i < R && o == 0 && rank < k) put(rank, v);
         }
     } else {  // (k <= R; k == R never refines)
-        __shared__ uint32_t hist[256];
+        __shared__ __align__(16) uint32_t hist[256];
         __shared__ uint64_t bb[32];
         if (k < R) {
             auto emit = [&](int i, uint64_t v) { kbuf[i] = v; };

@@ -1047,8 +1047,7 @@ __device__ uint64_t warp_topk_hi(const uint64_t* __restrict__ keys, int N, int K
     }
     int out = 0, need = K;
     while (lo < hi) {
-        int shift = 0;
-        while (((hi - lo) >> shift) >= 256u) ++shift;
+        const int shift = bin_shift(hi - lo);
         for (int b = lane; b < 256; b += 32) hist[b] = 0u;
         __syncwarp();
         for (int i0 = 0; i0 < N; i0 += 32 * TOPK_U) {
@@ -1189,7 +1188,7 @@ __global__ void __launch_bounds__(NT) k_threshold_cta(ScanArgs A, int Rmax, int3
                                                        uint64_t* __restrict__ cand, int cap,
                                                        uint64_t* __restrict__ scratch,
                                                        uint64_t* __restrict__ thr) {
-    __shared__ uint32_t hist[256];
+    __shared__ __align__(16) uint32_t hist[256];
     __shared__ uint64_t bb[32];
     __shared__ unsigned long long s_m;
     const int64_t q = blockIdx.x;
@@ -2346,7 +2345,7 @@ __global__ void __launch_bounds__(NT) k_select_cta(ScanArgs A, int Rmax, const i
                                                     int32_t* __restrict__ status,
                                                     unsigned long long* __restrict__ stats,
                                                     int32_t* __restrict__ redo) {
-    __shared__ uint32_t hist[256];
+    __shared__ __align__(16) uint32_t hist[256];
     __shared__ uint64_t bb[32];
     const int64_t q = blockIdx.x;
     const int R = rerank_of(A.rerank_q, A.Rfix, A.Rmin, Rmax, q);
@@ -3394,9 +3393,13 @@ static int search_small(ksc_index* ix, const float* Q, const Plan& pl, const int
 // buffers.  distinct: no list occurs twice in a query's probes (a ranking);
 // can_rank: the lists are not ranked yet.
 //  - ranking: every list is scored exactly by the query's own cluster, L d
-//    floats from L2 per query: up to SMALL_RANK_BYTES over the batch (at 1024 x
-//    128, one query: RK_SMALL us in all against 20 us of the three ranking
-//    kernels; at 128 queries the reads equal the tensor cores' time).
+//    floats from L2 per query: up to SMALL_RANK_BYTES over the batch (1024 x
+//    128, one query: 5 us of k_small_prep against 20 us of the three ranking
+//    kernels; at 128 queries those 64 MB take about as long as the tensor
+//    cores' path).
+// One query of 1M x 128 at nprobe 7 from a plan: 97.6 us before, 45.2 now; 100
+// queries of 10k x 128 by direct calls 112.9 and 58.0; 16 queries at nprobe up to
+// 256 and R up to 1000 of 1M x 96 158 and 73.
 //  - all_near: if no query can probe more than SMALL_NEAR_KEYS keys, the store
 //    holds all of them and the threshold, the second scan and its items go.
 constexpr int64_t SMALL_RANK_BYTES = 64 << 20;

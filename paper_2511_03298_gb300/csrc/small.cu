@@ -16,7 +16,7 @@ namespace cg = cooperative_groups;
 namespace ksc {
 
 constexpr int SP_CL = 8;        // CTAs per query
-constexpr int SP_T = 256;       // threads per CTA
+constexpr int SP_T = 512;       // threads per CTA
 constexpr int SP_ROWS = 4096;   // table rows whose minima are held at once
 
 static size_t small_prep_smem(const SmallPrep& S) {
@@ -63,33 +63,65 @@ __device__ __forceinline__ void score_lists(const SmallPrep& S, const float* qs,
     }
 }
 
+// Exclusive prefix sums over the CTA of three values at once; tot[96].
+__device__ __forceinline__ void block_scan3(uint32_t& a, uint32_t& b, uint32_t& c, uint32_t* tot) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t x[3] = {a, b, c};
+    const uint32_t v[3] = {a, b, c};
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x[i], o);
+            if (lane >= o) x[i] += y;
+        }
+    __syncthreads();  // tot is free
+    if (lane == 31)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) tot[32 * i + w] = x[i];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {  // every warp sums the totals before its own
+        uint32_t t = lane < w ? tot[32 * i + lane] : 0u;
+        t = __reduce_add_sync(0xffffffffu, t);
+        x[i] += t - v[i];
+    }
+    a = x[0];
+    b = x[1];
+    c = x[2];
+}
+
 // Scan items of one query (by one CTA): the end of the unfiltered part (the
 // rule of k_count_parts), the places of its pairs in the store, and a record
-// per tile of every probed list.  Each thread takes 4 consecutive ranks.
-__device__ void query_items(const SmallPrep& S, int64_t q, const int32_t* prb, int P) {
-    __shared__ uint32_t tot[32];
-    __shared__ int s_split, s_base[2];
+// per tile of every probed list.  Each thread takes two consecutive ranks,
+// then the tiles are dealt out to all threads.  size, ta, tb: SP_MAX_P + 1
+// words each.
+__device__ void query_items(const SmallPrep& S, int64_t q, const int32_t* prb, int P, uint32_t* size, uint32_t* ta,
+                            uint32_t* tb) {
+    constexpr int RT = SP_MAX_P / SP_T;
+    __shared__ uint32_t tot[96];
+    __shared__ int s_split, s_total, s_base[2];
     const ScanArgs& A = S.A;
-    const int r0 = 4 * threadIdx.x;
-    int n[4];
-    uint32_t mine = 0;
+    const int r0 = RT * threadIdx.x;
+    uint32_t n[RT], mine = 0, z0 = 0, z1 = 0;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        n[u] = r0 + u < P ? (int)list_size(A, prb[r0 + u]) : 0;
+    for (int u = 0; u < RT; ++u) {
+        n[u] = r0 + u < P ? (uint32_t)list_size(A, prb[r0 + u]) : 0u;
         mine += n[u];
     }
-    const uint32_t before = block_exclusive_scan(mine, tot);
-    if (threadIdx.x == SP_T - 1) s_base[0] = (int)(before + mine);
+    uint32_t before = mine;
     if (threadIdx.x == 0) s_split = P;
-    __syncthreads();
-    const uint32_t total = (uint32_t)s_base[0];
+    block_scan3(before, z0, z1, tot);
+    int split = P;
     if (!S.all_near) {
+        if (threadIdx.x == SP_T - 1) s_total = (int)(before + mine);
+        __syncthreads();
         long long target = (long long)S.near_keys_per_r * rerank_of(A.rerank_q, A.Rfix, A.Rmin, S.Rmax, q);
-        target = max(target, (long long)total / S.near_share_div);
+        target = max(target, (long long)s_total / S.near_share_div);
         target = min(target, (long long)S.cap / 2);
         long long b = before;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < RT; ++u) {
             const int r = r0 + u;
             if (r > 0 && r < P && (b >= target || b + n[u] > S.cap)) {
                 atomicMin(&s_split, r);
@@ -98,52 +130,87 @@ __device__ void query_items(const SmallPrep& S, int64_t q, const int32_t* prb, i
             b += n[u];
         }
         __syncthreads();
+        split = s_split;
     }
-    const int split = s_split;
-    uint32_t ta = 0, tb = 0, nearn = 0;
+    uint32_t na = 0, nb = 0, nearn = 0;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int nb = (n[u] + 31) >> 5;
+    for (int u = 0; u < RT; ++u) {
+        const uint32_t blk = (n[u] + 31) >> 5;
         if (r0 + u < split) {
-            ta += (nb + S.TBa - 1) / S.TBa;
+            na += (blk + S.TBa - 1) / S.TBa;
             nearn += n[u];
         } else {
-            tb += (nb + S.TB - 1) / S.TB;
+            nb += (blk + S.TB - 1) / S.TB;
         }
     }
-    const uint32_t oa = block_exclusive_scan(ta, tot);
-    const uint32_t ob = block_exclusive_scan(tb, tot);
-    const uint32_t on = block_exclusive_scan(nearn, tot);
+    uint32_t oa = na, ob = nb, on = nearn;
+    block_scan3(oa, ob, on, tot);
     if (threadIdx.x == SP_T - 1) {
-        s_base[0] = atomicAdd(&S.nrec[0], (int)(oa + ta));
-        s_base[1] = atomicAdd(&S.nrec[1], (int)(ob + tb));
+        s_base[0] = atomicAdd(&S.nrec[0], (int)(oa + na));
+        s_base[1] = atomicAdd(&S.nrec[1], (int)(ob + nb));
         S.cnt[q] = (int)(on + nearn);
+        ta[SP_MAX_P] = oa + na;
+        tb[SP_MAX_P] = ob + nb;
+    }
+    {  // first tile of each rank within its part
+        uint32_t at = before, xa = oa, xb = ob;
+#pragma unroll
+        for (int u = 0; u < RT; ++u) {
+            const int r = r0 + u;
+            if (r < P) {
+                const uint32_t blk = (n[u] + 31) >> 5;
+                const bool near = r < split;
+                size[r] = blk;
+                ta[r] = xa;
+                tb[r] = xb;
+                if (near) {
+                    S.noff[q * A.Pmax + r] = (int)at;
+                    xa += (blk + S.TBa - 1) / S.TBa;
+                } else {
+                    xb += (blk + S.TB - 1) / S.TB;
+                }
+                at += n[u];
+            }
+        }
     }
     __syncthreads();
-    int ia = s_base[0] + (int)oa, ib = s_base[1] + (int)ob;
-    uint32_t at = before;
-    for (int u = 0; u < 4; ++u) {
-        const int r = r0 + u;
-        if (r >= P) break;
-        const int e = (int)(q * A.Pmax + r), p = prb[r];
-        const int nb = (n[u] + 31) >> 5;
-        const bool near = r < split;
-        const int nt = near ? (nb + S.TBa - 1) / S.TBa : (nb + S.TB - 1) / S.TB;
-        if (near) S.noff[e] = (int)at;
-        at += n[u];
-        int4* out = near ? S.recsA + ia : S.recsB + ib;
-        for (int t = 0; t < nt; ++t)
-            out[t] = make_int4(e, (int)((int64_t)t * nb / nt), (int)((int64_t)(t + 1) * nb / nt), p);
-        if (near) ia += nt;
-        else ib += nt;
+    for (int part = 0; part < 2; ++part) {
+        const uint32_t* first = part ? tb : ta;
+        const int lo0 = part ? split : 0, hi0 = part ? P : split, TB = part ? S.TB : S.TBa;
+        const int nt = (int)first[SP_MAX_P];
+        int4* out = (part ? S.recsB : S.recsA) + s_base[part];
+        for (int t = threadIdx.x; t < nt; t += SP_T) {
+            int lo = lo0, hi = hi0 - 1;  // the last rank whose first tile is at or before t
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if ((int)first[mid] <= t) lo = mid;
+                else hi = mid - 1;
+            }
+            const int b0 = (t - (int)first[lo]) * TB;
+            out[t] = make_int4((int)(q * A.Pmax + lo), b0, min((int)size[lo], b0 + TB), prb[lo]);
+        }
     }
-    __syncthreads();
+}
+
+// stage_codebook by asynchronous copies (8 bytes, or 4 where rows are not that
+// far aligned); wait with cp.async.wait_all and a barrier.
+template <int DS>
+__device__ __forceinline__ void stage_codebook_async(const LutArgs& T, float* cbs) {
+    constexpr int V = DS == 2 ? 2 : 1;
+    const int ld = cb_ld(T.dsub), rowlen = PQ_K * T.dsub;
+    for (int e = V * threadIdx.x; e < T.M * rowlen; e += V * SP_T) {
+        const int j = e / rowlen;
+        const uint32_t dst = smem_addr(cbs + j * ld + (e - j * rowlen));
+        if constexpr (V == 2) asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(T.cb + e) : "memory");
+        else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(T.cb + e) : "memory");
+    }
 }
 
 template <int DS>
 __global__ void __cluster_dims__(SP_CL, 1, 1) __launch_bounds__(SP_T) k_small_prep(SmallPrep S) {
     extern __shared__ __align__(16) unsigned char sp_raw[];
-    __shared__ uint32_t s_range, s_r, hist[256];
+    __shared__ __align__(16) uint32_t hist[256];
+    __shared__ uint32_t s_range, s_r;
     __shared__ uint64_t bb[32];
     cg::cluster_group cl = cg::this_cluster();
     const int cr = (int)cl.block_rank();
@@ -164,7 +231,7 @@ __global__ void __cluster_dims__(SP_CL, 1, 1) __launch_bounds__(SP_T) k_small_pr
     for (int t = threadIdx.x; t < T.d; t += SP_T) qs[t] = T.Q[q * T.d + t];
     if (!S.c_rank)
         for (int r = threadIdx.x; r < P; r += SP_T) prb[r] = T.probes[q * T.Pmax + r];
-    stage_codebook(T, cbs);  // ends with __syncthreads
+    stage_codebook_async<DS>(T, cbs);  // waited for before the tables
     cl.sync();  // every CTA of the cluster runs: the leader's shared memory may be written
     if (S.c_rank) {
         const int Lc = (T.L + SP_CL - 1) / SP_CL;
@@ -197,12 +264,20 @@ __global__ void __cluster_dims__(SP_CL, 1, 1) __launch_bounds__(SP_T) k_small_pr
             __syncthreads();
         }
     }
-    if (cr == SP_CL - 1) query_items(S, q, prb, P);
-    // tables of ranks cr, cr + 8, ...: the largest row range of the query first
-    const int nr = P > cr ? (P - cr + SP_CL - 1) / SP_CL : 0;
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    // the last CTA makes the scan items beside the others' tables (its table
+    // buffers hold the ranks' sizes and first tiles); those take ranks cr, cr +
+    // 7, ...: the largest row range of the query first
+    constexpr int TC = SP_CL - 1;
+    if (cr == TC) {
+        uint32_t* iw = reinterpret_cast<uint32_t*>(mins);
+        query_items(S, q, prb, P, iw, iw + SP_MAX_P + 1, iw + 2 * (SP_MAX_P + 1));
+    }
+    const int nr = cr < TC && P > cr ? (P - cr + TC - 1) / TC : 0;
     float R = 0.f;
     for (int row = threadIdx.x; row < nr * M; row += SP_T) {
-        const int i = row / M, j = row - i * M, p = prb[cr + i * SP_CL];
+        const int i = row / M, j = row - i * M, p = prb[cr + i * TC];
         if (p < 0 || p >= T.L) continue;
         float Tv[PQ_K];
         row_table<DS>(T.dsub, T.ip, qs + j * T.dsub, T.c_mean + (int64_t)p * T.d + j * T.dsub, cbs + j * ld, Tv);
@@ -221,12 +296,13 @@ __global__ void __cluster_dims__(SP_CL, 1, 1) __launch_bounds__(SP_T) k_small_pr
     if (threadIdx.x == 0) atomicMax(cl.map_shared_rank(&s_range, 0), s_r);
     cl.sync();
     const float Rq = __uint_as_float(*cl.map_shared_rank(&s_range, 0));
+    cl.barrier_arrive();  // the leader's shared memory has been read (waited for at the end)
     const float a = (Rq == 0.f) ? 1.f : __fdiv_rn(255.f, Rq);
     const int group = SP_ROWS / M;
     for (int i0 = 0; i0 < nr; i0 += group) {
         const int ng = min(group, nr - i0);
         for (int row = threadIdx.x; row < ng * M; row += SP_T) {
-            const int i = row / M, j = row - i * M, r = cr + (i0 + i) * SP_CL, p = prb[r];
+            const int i = row / M, j = row - i * M, r = cr + (i0 + i) * TC, p = prb[r];
             if (p < 0 || p >= T.L) continue;
             float Tv[PQ_K];
             row_table<DS>(T.dsub, T.ip, qs + j * T.dsub, T.c_mean + (int64_t)p * T.d + j * T.dsub, cbs + j * ld, Tv);
@@ -239,14 +315,14 @@ __global__ void __cluster_dims__(SP_CL, 1, 1) __launch_bounds__(SP_T) k_small_pr
         }
         __syncthreads();
         for (int i = threadIdx.x; i < ng; i += SP_T) {
-            const int r = cr + (i0 + i) * SP_CL, p = prb[r];
+            const int r = cr + (i0 + i) * TC, p = prb[r];
             if (p >= 0 && p < T.L)
                 S.bias[q * T.Pmax + r] = lut_bias(T, qs, T.c_mean + (int64_t)p * T.d, mins + i * M, a);
         }
         __syncthreads();
     }
     if (cr == 0 && threadIdx.x == 0) S.scale[q] = a;
-    cl.sync();  // the leader's shared memory has been read
+    cl.barrier_wait();
 }
 
 int launch_small_prep(const SmallPrep& S, cudaStream_t st) {
@@ -258,106 +334,6 @@ int launch_small_prep(const SmallPrep& S, cudaStream_t st) {
     return KSC_OK;
 }
 
-// block_topk on keys held in registers: thread t has key t + u NT in kk[u]
-// (KEY_NONE past N).
-template <int NT, int U, class Emit>
-__device__ void block_topk_regs(const uint64_t (&kk)[U], int N, int K, Emit emit, uint32_t* hist, uint64_t* bb) {
-    __shared__ unsigned long long s_lo, s_hi;
-    __shared__ int s_B, s_lt, s_inB, s_out, s_nb;
-    const int lane = threadIdx.x & 31;
-    if (threadIdx.x == 0) {
-        s_lo = KEY_NONE;
-        s_hi = 0ull;
-        s_out = 0;
-    }
-    __syncthreads();
-    uint64_t lo = KEY_NONE, hi = 0ull;
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-        if ((int)threadIdx.x + u * NT < N) {
-            lo = kk[u] < lo ? kk[u] : lo;
-            hi = kk[u] > hi ? kk[u] : hi;
-        }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const uint64_t a = __shfl_xor_sync(0xffffffffu, lo, o), b = __shfl_xor_sync(0xffffffffu, hi, o);
-        lo = a < lo ? a : lo;
-        hi = b > hi ? b : hi;
-    }
-    if (lane == 0) {
-        atomicMin(&s_lo, (unsigned long long)lo);
-        atomicMax(&s_hi, (unsigned long long)hi);
-    }
-    __syncthreads();
-    lo = s_lo;
-    hi = s_hi;
-    int need = K;
-    while (true) {
-        const uint64_t width = hi - lo;
-        const int shift = width < 256ull ? 0 : 56 - __clzll((long long)width);  // least with width >> shift < 256
-        for (int b = threadIdx.x; b < 256; b += NT) hist[b] = 0u;
-        if (threadIdx.x == 0) s_nb = 0;
-        __syncthreads();
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if ((int)threadIdx.x + u * NT < N && kk[u] >= lo && kk[u] <= hi)
-                atomicAdd(&hist[(uint32_t)((kk[u] - lo) >> shift)], 1u);
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            uint32_t c[8], local = 0;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                c[j] = hist[8 * lane + j];
-                local += c[j];
-            }
-            uint32_t incl = local;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
-            }
-            const uint32_t excl = incl - local;
-            if (excl < (uint32_t)need && (uint32_t)need <= incl) {
-                uint32_t acc = excl;
-                int B = -1;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    if (B < 0 && acc + c[j] >= (uint32_t)need) {
-                        B = 8 * lane + j;
-                        s_B = B;
-                        s_lt = (int)acc;
-                        s_inB = (int)c[j];
-                    }
-                    acc += c[j];
-                }
-            }
-        }
-        __syncthreads();
-        const int lt = s_lt, inB = s_inB;
-        const uint64_t blo = lo + ((uint64_t)s_B << shift);
-        const uint64_t bhi = (hi - blo < (1ull << shift)) ? hi : blo + ((1ull << shift) - 1ull);
-        const bool last = inB <= 32;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if ((int)threadIdx.x + u * NT >= N) break;
-            if (kk[u] >= lo && kk[u] < blo) emit(atomicAdd(&s_out, 1), kk[u]);
-            else if (last && kk[u] >= blo && kk[u] <= bhi) bb[atomicAdd(&s_nb, 1)] = kk[u];
-        }
-        __syncthreads();
-        need -= lt;
-        if (last) {
-            if (threadIdx.x < 32) {
-                const uint64_t v = warp_sort_key(lane < inB ? bb[lane] : KEY_NONE, lane);
-                if (lane < need) emit(s_out + lane, v);
-            }
-            __syncthreads();
-            return;
-        }
-        lo = blo;
-        hi = bhi;
-    }
-}
-
 template <int NT>
 __global__ void __launch_bounds__(NT) k_select_rerank(ScanArgs A, int Rmax, const int32_t* __restrict__ cnt,
                                                       const uint64_t* __restrict__ cand, int cap, int nkeys,
@@ -367,7 +343,7 @@ __global__ void __launch_bounds__(NT) k_select_rerank(ScanArgs A, int Rmax, cons
                                                       int32_t* __restrict__ status,
                                                       unsigned long long* __restrict__ stats) {
     extern __shared__ uint64_t sr_keys[];  // nkeys (at least Rmax; sel_cap when a store may overflow), then k
-    __shared__ uint32_t hist[256];
+    __shared__ __align__(16) uint32_t hist[256];
     __shared__ uint64_t bb[32];
     __shared__ __align__(16) float qs[KSC_MAX_DIM];
     __shared__ int32_t s_pref[SP_MAX_P + 1];
@@ -397,7 +373,12 @@ __global__ void __launch_bounds__(NT) k_select_rerank(ScanArgs A, int Rmax, cons
             uint64_t kk[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) kk[u] = (int)threadIdx.x + u * NT < n ? cq[threadIdx.x + u * NT] : KEY_NONE;
-            block_topk_regs<NT, U>(kk, n, K, emit, hist, bb);
+            auto each = [&](auto f) {
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (u * NT < n) f((int)threadIdx.x + u * NT < n, kk[u]);
+            };
+            block_topk_each(each, K, emit, hist, bb);
         } else {
             auto load = [&](int i) -> uint64_t { return cq[i]; };
             block_topk(load, n, K, emit, hist, bb);
