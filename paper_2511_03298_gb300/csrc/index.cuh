@@ -107,7 +107,6 @@ int pack_lists(ksc_index* ix, const uint8_t* codes_dev, const int32_t* assign_ho
 int free_index_memory(ksc_index* ix);
 // Tensor-core list scores (rank_tc.cu): approximate scores [nq x L] and a
 // per-query bound err [nq] on their error.
-bool tc_rank_supported(const ksc_index* ix);
 int rank_scores_tc(ksc_index* ix, const float* Q, int64_t nq, float* scores, float* err, cudaStream_t st);
 // The same from e4m3 operands with per-row power-of-two scales (FP8 option).
 int rank_scores_tc8(ksc_index* ix, const float* Q, int64_t nq, float* scores, float* err, cudaStream_t st);

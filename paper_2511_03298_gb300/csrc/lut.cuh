@@ -53,9 +53,12 @@ __device__ __forceinline__ int probes_of(const LutArgs& A, int64_t q) {
 
 // Codebook row stride in shared memory.  dsub = 2: 34 floats (codewords
 // 8-byte aligned; a half-warp reading 16 consecutive rows with 8-byte loads
-// covers all 32 banks once); else 16 dsub + 1 (odd: 32 consecutive rows fall
-// in distinct banks).
-__host__ __device__ __forceinline__ int cb_ld(int dsub) { return dsub == 2 ? 34 : PQ_K * dsub + 1; }
+// covers all 32 banks once); dsub = 4: 68 (16-byte aligned; 8 consecutive rows
+// of a 16-byte load cover all banks once); else 16 dsub + 1 (odd: 32
+// consecutive rows fall in distinct banks).
+__host__ __device__ __forceinline__ int cb_ld(int dsub) {
+    return dsub == 2 ? 34 : (dsub == 4 ? 68 : PQ_K * dsub + 1);
+}
 
 __device__ __forceinline__ void stage_codebook(const LutArgs& A, float* cbs) {
     const int ld = cb_ld(A.dsub), rowlen = PQ_K * A.dsub;
@@ -68,8 +71,9 @@ __device__ __forceinline__ void stage_codebook(const LutArgs& A, float* cbs) {
 
 // The 16 FP32 entries of one subspace: qj, cj = the query's and the list
 // centroid's values of the subspace, cw = its codebook row in shared memory.
-// DS = dsub when fixed at compile time (2: 8-byte loads; qj and cj 8-byte
-// aligned), 0 = read from dsub.
+// DS = dsub when fixed at compile time (2: 8-byte loads, 4: 16-byte loads; qj
+// and cj aligned to that), 0 = read from dsub.  (60k x 784, M 196, 10,000
+// queries at nprobe 4: 419 us with width 4 read from dsub, 367 us fixed.)
 template <int DS>
 __device__ __forceinline__ void row_table(int dsub, int ip, const float* __restrict__ qj,
                                           const float* __restrict__ cj, const float* cw, float (&T)[PQ_K]) {
@@ -97,6 +101,33 @@ __device__ __forceinline__ void row_table(int dsub, int ip, const float* __restr
                 const float2 e2 = f2_mul(e, e);
                 T[i] = __fadd_rn(e2.x, e2.y);
             }
+        }
+    } else if constexpr (DS == 4) {
+        // 16-byte loads, differences, products and squares as packed pairs, the
+        // sums in ascending t (0 + the first term is the term)
+        const float4 qv = *reinterpret_cast<const float4*>(qj);
+        float2 u01 = make_float2(qv.x, qv.y), u23 = make_float2(qv.z, qv.w);
+        if (!ip) {
+            const float4 cv = *reinterpret_cast<const float4*>(cj);
+            u01 = f2_sub(u01, make_float2(cv.x, cv.y));
+            u23 = f2_sub(u23, make_float2(cv.z, cv.w));
+        }
+#pragma unroll
+        for (int i = 0; i < PQ_K; ++i) {
+            const float4 c = *reinterpret_cast<const float4*>(cw + 4 * i);
+            float2 e01, e23;
+            if (ip) {
+                e01 = f2_mul(u01, make_float2(c.x, c.y));
+                e23 = f2_mul(u23, make_float2(c.z, c.w));
+                e01.x = __fadd_rn(0.f, e01.x);
+            } else {
+                e01 = f2_sub(u01, make_float2(c.x, c.y));
+                e23 = f2_sub(u23, make_float2(c.z, c.w));
+                e01 = f2_mul(e01, e01);
+                e23 = f2_mul(e23, e23);
+            }
+            const float s = __fadd_rn(__fadd_rn(__fadd_rn(e01.x, e01.y), e23.x), e23.y);
+            T[i] = ip ? -s : s;
         }
     } else {
 #pragma unroll

@@ -33,8 +33,10 @@
 namespace ksc {
 
 // scores[q][c] for one 128 x 256 tile.  KB = number of K boxes of 128 bytes
-// per row (64 16-bit or 128 8-bit elements).  F8: e4m3 operands whose rows
-// carry the power-of-two scales qs [nq] and cs [L].
+// per row (64 16-bit or 128 8-bit elements); up to RG_STAGES boxes are in
+// shared memory, a box's place is loaded again once its MMAs are done.  F8:
+// e4m3 operands whose rows carry the power-of-two scales qs [nq] and cs [L].
+constexpr int RG_STAGES = 4;
 template <bool F8>
 __global__ void __launch_bounds__(128, 1) k_rank_gemm_tc(const __grid_constant__ CUtensorMap mapA,
                                                          const __grid_constant__ CUtensorMap mapB, int KB, int64_t nq,
@@ -44,15 +46,18 @@ __global__ void __launch_bounds__(128, 1) k_rank_gemm_tc(const __grid_constant__
                                                          int32_t* __restrict__ status) {
     constexpr int BOX_K = F8 ? 128 : TC_KB;  // elements per 128-byte box row
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bars[2];
+    __shared__ __align__(8) uint64_t bars[2 * RG_STAGES + 1];
     __shared__ uint32_t tmem_base;
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    const uint32_t sA = smem_u32(smem), sB = sA + KB * (TC_M * 128);
-    const uint32_t bar_tma = smem_u32(&bars[0]), bar_mma = smem_u32(&bars[1]);
+    const int NS = KB < RG_STAGES ? KB : RG_STAGES;
+    const uint32_t sA = smem_u32(smem), sB = sA + NS * (TC_M * 128);
+    auto full = [&](int i) { return smem_u32(&bars[i]); };               // stage i's copies have landed
+    auto used = [&](int i) { return smem_u32(&bars[RG_STAGES + i]); };   // stage i's MMAs are done
+    const uint32_t bar_mma = smem_u32(&bars[2 * RG_STAGES]);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m0 = blockIdx.y * TC_M, n0 = blockIdx.x * TC_N;
     if (threadIdx.x == 0) {
-        mbar_init(bar_tma, 1);
+        for (int i = 0; i < 2 * RG_STAGES; ++i) mbar_init(full(i), 1);
         mbar_init(bar_mma, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -67,28 +72,42 @@ __global__ void __launch_bounds__(128, 1) k_rank_gemm_tc(const __grid_constant__
     const uint32_t tmem = tmem_base;
     bool ok = true;
     if (threadIdx.x == 0) {
-        mbar_expect_tx(bar_tma, (uint32_t)KB * (TC_M + TC_N) * 128);
-        for (int kb = 0; kb < KB; ++kb) {
-            tma_load_2d(sA + kb * (TC_M * 128), &mapA, bar_tma, kb * BOX_K, m0);
-            tma_load_2d(sB + kb * (TC_N * 128), &mapB, bar_tma, kb * BOX_K, n0);
-        }
-        ok = mbar_wait(bar_tma, 0, TC_WAIT_LIMIT);
-        if (ok) {
+        auto load = [&](int kb) {
+            const int i = kb % NS;
+            mbar_expect_tx(full(i), (TC_M + TC_N) * 128);
+            tma_load_2d(sA + i * (TC_M * 128), &mapA, full(i), kb * BOX_K, m0);
+            tma_load_2d(sB + i * (TC_N * 128), &mapB, full(i), kb * BOX_K, n0);
+        };
+        for (int kb = 0; kb < NS; ++kb) load(kb);
+        const uint32_t idesc = idesc_f16kind(fmt, TC_M, TC_N);
+        int loaded = NS, kb = 0;
+        for (; kb < KB; ++kb) {
+            const int i = kb % NS;
+            ok = mbar_wait(full(i), (kb / NS) & 1, TC_WAIT_LIMIT);
+            if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t idesc = idesc_f16kind(fmt, TC_M, TC_N);
             // four MMAs per 128-byte box: K = 16 16-bit or 32 8-bit elements = 32 bytes each
-            for (int kb = 0; kb < KB; ++kb)
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const uint64_t a = smem_desc(sA + kb * (TC_M * 128) + k * 32);
-                    const uint64_t b = smem_desc(sB + kb * (TC_N * 128) + k * 32);
-                    if (F8) tc_mma_f8(tmem, a, b, idesc, (kb | k) != 0);
-                    else tc_mma(tmem, a, b, idesc, (kb | k) != 0);
-                }
+            for (int k = 0; k < 4; ++k) {
+                const uint64_t a = smem_desc(sA + i * (TC_M * 128) + k * 32);
+                const uint64_t b = smem_desc(sB + i * (TC_N * 128) + k * 32);
+                if (F8) tc_mma_f8(tmem, a, b, idesc, (kb | k) != 0);
+                else tc_mma(tmem, a, b, idesc, (kb | k) != 0);
+            }
+            tc_commit(used(i));
+            if (kb > 0 && loaded < KB) {  // the stage before this one again, once its MMAs have read it
+                ok = mbar_wait(used((kb - 1) % NS), ((kb - 1) / NS) & 1, TC_WAIT_LIMIT);
+                if (!ok) break;
+                load(loaded++);
+            }
+        }
+        if (ok) {
             tc_commit(bar_mma);
-        } else {
-            atomicOr(status, 2);  // the operand copy never completed: wait (bounded) once more
-            mbar_wait(bar_tma, 0, TC_WAIT_LIMIT);
+        } else {  // a copy or MMA never completed: what is in flight is waited for (bounded) once more
+            atomicOr(status, 2);
+            for (int l = kb; l < loaded; ++l) mbar_wait(full(l % NS), (l / NS) & 1, TC_WAIT_LIMIT);
+            tc_commit(bar_mma);
+            mbar_wait(bar_mma, 0, TC_WAIT_LIMIT);
         }
     }
     __syncthreads();
@@ -279,8 +298,6 @@ __global__ void k_q8_err(const float* __restrict__ Q, int64_t nq, int d, int Kp,
     err[q] = (spherical ? e : 2.f * e) + r;
 }
 
-bool tc_rank_supported(const ksc_index* ix) { return ix->d <= 256; }
-
 // Approximate scores [nq x L] with the tensor cores plus the per-query error
 // bound err [nq]; the caller re-scores exactly what the bound cannot exclude.
 static int err_params(ksc_index* ix, bool tensor_cores, float* rel, float* qmax, cudaStream_t st);
@@ -310,7 +327,7 @@ int rank_scores_tc(ksc_index* ix, const float* Q, int64_t nq, float* scores, flo
     KSC_LAUNCH_CHECK();
     CUtensorMap mapA;
     KSC_TRY(make_map(&mapA, qb, nq, Kp, TC_M, ix->tc_fp16));
-    const size_t smem = (size_t)KB * (TC_M + TC_N) * 128 + 1024;
+    const size_t smem = (size_t)std::min(KB, RG_STAGES) * (TC_M + TC_N) * 128 + 1024;
     KSC_CUDA(cudaFuncSetAttribute(k_rank_gemm_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     dim3 grid((ix->L + TC_N - 1) / TC_N, (unsigned)((nq + TC_M - 1) / TC_M));
     k_rank_gemm_tc<false><<<grid, 128, smem, st>>>(mapA, *reinterpret_cast<const CUtensorMap*>(ix->map_c), KB, nq,
@@ -362,7 +379,7 @@ int rank_scores_tc8(ksc_index* ix, const float* Q, int64_t nq, float* scores, fl
     KSC_LAUNCH_CHECK();
     CUtensorMap mapA;
     KSC_TRY(make_map(&mapA, q8, nq, Kp, TC_M, false, 1));
-    const size_t smem = (size_t)KB * (TC_M + TC_N) * 128 + 1024;
+    const size_t smem = (size_t)std::min(KB, RG_STAGES) * (TC_M + TC_N) * 128 + 1024;
     KSC_CUDA(cudaFuncSetAttribute(k_rank_gemm_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     dim3 grid((ix->L + TC_N - 1) / TC_N, (unsigned)((nq + TC_M - 1) / TC_M));
     k_rank_gemm_tc<true><<<grid, 128, smem, st>>>(mapA, *reinterpret_cast<const CUtensorMap*>(ix->map_c8), KB, nq,

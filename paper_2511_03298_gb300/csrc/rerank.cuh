@@ -181,9 +181,10 @@ __device__ __forceinline__ void cta_rerank(uint64_t* keys, int R, uint64_t* kbuf
             for (int s = parts >> 1; s > 0; s >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, s);
             if (i < R && o == 0 && rank < k) put(rank, v);
         }
-    } else {  // (k <= R; k == R never refines)
+    } else {
         __shared__ __align__(16) uint32_t hist[256];
         __shared__ uint64_t bb[32];
+        const int kr = k < R ? k : R;  // (all of them: no refinement)
         if (k < R) {
             auto emit = [&](int i, uint64_t v) { kbuf[i] = v; };
             auto load = [&](int i) -> uint64_t { return keys[i]; };
@@ -192,11 +193,11 @@ __device__ __forceinline__ void cta_rerank(uint64_t* keys, int R, uint64_t* kbuf
             for (int i = threadIdx.x; i < R; i += NT) kbuf[i] = keys[i];
         }
         __syncthreads();
-        for (int i = threadIdx.x; i < k; i += NT) {
+        for (int i = threadIdx.x; i < kr; i += NT) {
             const uint64_t v = kbuf[i];
             int rank = 0;
 #pragma unroll 8
-            for (int j = 0; j < k; ++j) rank += kbuf[j] < v;
+            for (int j = 0; j < kr; ++j) rank += kbuf[j] < v;
             put(rank, v);
         }
     }

@@ -22,6 +22,7 @@
 #include "lut.cuh"
 #include "mlp.cuh"
 #include "rerank.cuh"
+#include "rerank_low.cuh"
 #include "scan.cuh"
 #include "small.cuh"
 
@@ -774,7 +775,7 @@ constexpr int LUT_WARPS = 8;
 
 template <int DS>
 __global__ void __launch_bounds__(LUT_WARPS * 32) k_lut_range(LutArgs A, uint32_t* __restrict__ range_bits) {
-    extern __shared__ float cbs[];
+    extern __shared__ __align__(16) float cbs[];
     stage_codebook(A, cbs);
     const int ld = cb_ld(A.dsub);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -809,7 +810,7 @@ template <int DS>
 __global__ void __launch_bounds__(LUT_WARPS * 32) k_lut_quant(LutArgs A, const uint32_t* __restrict__ range_bits,
                                                               uint8_t* __restrict__ lut, int32_t* __restrict__ bias,
                                                               float* __restrict__ scale) {
-    extern __shared__ float cbs[];
+    extern __shared__ __align__(16) float cbs[];
     __shared__ float s_min[LUT_WARPS][KSC_MAX_M];
     stage_codebook(A, cbs);
     const int ld = cb_ld(A.dsub);
@@ -990,8 +991,15 @@ static size_t lut_fused_smem(int M, int dsub, int d, int Pb, int Pm) {
            sizeof(int32_t) * 2 * (size_t)Pm;
 }
 
-// 8-byte row loads need dsub = 2 and an 8-byte aligned query matrix.
-static bool lut_ds2(const LutArgs& A) { return A.dsub == 2 && (reinterpret_cast<uintptr_t>(A.Q) & 7) == 0; }
+// The fixed row width of the tables (0: any): vector loads of the rows need
+// the query matrix aligned to them (d is a multiple of dsub; the fused kernel
+// reads the query from shared memory).
+static int lut_width(const LutArgs& A, bool from_shared) {
+    const uintptr_t q = from_shared ? 0 : reinterpret_cast<uintptr_t>(A.Q);
+    if (A.dsub == 2 && (q & 7) == 0) return 2;
+    if (A.dsub == 4 && (q & 15) == 0) return 4;
+    return 0;
+}
 
 static int launch_luts(const LutArgs& A, uint32_t* rb, uint8_t* lut, int32_t* bias, float* scale, cudaStream_t st);
 
@@ -2732,10 +2740,14 @@ __global__ void k_band_rows(const float* __restrict__ X, const uint16_t* __restr
 // byte holds it exactly; -0 counts as 0).
 __global__ void k_bytes_exact(const float* __restrict__ X, int64_t m, int32_t* __restrict__ ok) {
     bool all = true;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    for (int round = 0; i < m && all; i += (int64_t)gridDim.x * blockDim.x, ++round) {
+        // (real-valued rows end the check at once, in every CTA)
+        if ((round & 15) == 15 && *reinterpret_cast<const volatile int32_t*>(ok) == 0) break;
         const float v = X[i];
         all &= v >= 0.f && v <= 255.f && v == rintf(v);
     }
+    __syncwarp();
     if (!__all_sync(0xffffffffu, all) && (threadIdx.x & 31) == 0) atomicAnd(ok, 0);
 }
 
@@ -2765,60 +2777,6 @@ __global__ void k_x_lowp(const float* __restrict__ X, int64_t n, int d, int prec
     if (lane == 0) sc[r] = s;
     for (int t = lane; t < d; t += 32)
         x8[r * d + t] = (uint8_t)__nv_cvt_float_to_fp8(x[t] / s, __NV_SATFINITE, __NV_E4M3);
-}
-
-__device__ __forceinline__ float lowp_elem(int prec, const uint16_t* xb, const uint8_t* x8, int64_t off) {
-    if (prec == 1) return __bfloat162float(__ushort_as_bfloat16(xb[off]));
-    __half_raw h = __nv_cvt_fp8_to_halfraw((__nv_fp8_storage_t)x8[off], __NV_E4M3);
-    return __half2float(__half(h));
-}
-
-// Distance of query row qs (shared) to row id in the given precision (0 FP32,
-// 1 BF16, 2 FP8 with row scale); one warp, result in every lane.
-__device__ __forceinline__ float lowp_dist(int prec, const float* __restrict__ qs, const float* __restrict__ X,
-                                           const uint16_t* __restrict__ xb, const uint8_t* __restrict__ x8,
-                                           const float* __restrict__ sc, int32_t id, int d, int ip, int lane) {
-    float acc = 0.f;
-    const float s = prec == 2 ? sc[id] : 1.f;
-    for (int t = lane; t < d; t += 32) {
-        const float xv = prec == 0 ? __ldg(X + (int64_t)id * d + t) : lowp_elem(prec, xb, x8, (int64_t)id * d + t) * s;
-        if (ip) acc = fmaf(qs[t], xv, acc);
-        else { const float e = qs[t] - xv; acc = fmaf(e, e, acc); }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    return ip ? -acc : acc;
-}
-
-// Widened first re-rank: the R_w candidates (topr) by low-precision
-// distance, the best Rf of them (by (distance, id)) written as keys to out.
-__global__ void __launch_bounds__(256) k_rerank_lowp(const float* __restrict__ Q, int d, int ip, int prec,
-                                                     const uint16_t* __restrict__ xb, const uint8_t* __restrict__ x8,
-                                                     const float* __restrict__ sc, const uint64_t* __restrict__ topr,
-                                                     int Rmax, const int32_t* __restrict__ rerank_q, int Rfix,
-                                                     int Rmin, int Rf, uint64_t* __restrict__ out) {
-    extern __shared__ uint64_t keys[];
-    __shared__ __align__(16) float qs[KSC_MAX_DIM];
-    const int64_t q = blockIdx.x;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int R = rerank_of(rerank_q, Rfix, Rmin, Rmax, q);
-    for (int t = threadIdx.x; t < d; t += blockDim.x) qs[t] = Q[q * d + t];
-    __syncthreads();
-    const uint64_t* cq = topr + q * Rmax;
-    for (int c = w; c < R; c += nw) {
-        const uint64_t kk = cq[c];
-        uint64_t o = KEY_NONE;
-        if (kk != KEY_NONE) {
-            const int32_t id = (int32_t)(kk & 0xffffffffu);
-            o = ((uint64_t)ordered_f32(lowp_dist(prec, qs, nullptr, xb, x8, sc, id, d, ip, lane)) << 32) | (uint32_t)id;
-        }
-        if (lane == 0) keys[c] = o;
-    }
-    const int S = pow2_ceil(R < 2 ? 2 : R);
-    for (int i = R + threadIdx.x; i < S; i += blockDim.x) keys[i] = KEY_NONE;
-    __syncthreads();
-    block_bitonic_sort(keys, S);
-    for (int i = threadIdx.x; i < Rf; i += blockDim.x) out[q * Rf + i] = i < R ? keys[i] : KEY_NONE;
 }
 
 // Diagnostic: distances of given (query, id) pairs in a precision.
@@ -2960,15 +2918,23 @@ static int dispatch_scan(int S, const ScanArgs& A, const ScanOut& O, const int64
 // Operand type of the list scores (a1): 16-bit tensor cores, FP32 CUDA
 // cores, or FP8 tensor cores.
 enum RankMode { RANK_TC16 = 0, RANK_FP32 = 1, RANK_FP8 = 2 };
+// Widest rows whose given scores come from the tensor cores everywhere; wider
+// ones only where the scores just preselect lists for the exact ranking.
+constexpr int TC_SCORES_D = 256;
 
 // List scores [nq x L] on the 16-bit or FP8 tensor cores or the FP32 CUDA
 // cores, with the per-query bound err [nq] on their distance from the exact
 // scores.
 static int list_scores(ksc_index* ix, const float* Q, int64_t nq, int mode, float* scores, float** err,
-                       cudaStream_t st) {
+                       cudaStream_t st, bool preselect = false) {
     KSC_TRY(ensure(ix->ws_err, sizeof(float) * nq, st));
     *err = (float*)ix->ws_err.p;
-    if (mode != RANK_FP32 && tc_rank_supported(ix))
+    // rows past TC_SCORES_D: the scores themselves stay FP32 (ksc_list_scores,
+    // the predictor's features); a ranking re-scores exactly whatever the
+    // scores' bound cannot exclude, so it takes the 16-bit tensor cores there
+    // too (10,000 x 784 against 256 lists: 365 us of FP32 scores and bounds
+    // before, 32 us now)
+    if (mode != RANK_FP32 && (ix->d <= TC_SCORES_D || (preselect && mode == RANK_TC16)))
         return mode == RANK_FP8 ? rank_scores_tc8(ix, Q, nq, scores, *err, st)
                                 : rank_scores_tc(ix, Q, nq, scores, *err, st);
     dim3 grid(blocks_for(ix->L, SC_T), blocks_for(nq, SC_T));
@@ -2998,7 +2964,7 @@ static int rank_lists(ksc_index* ix, const float* Q, int64_t nq, const int32_t* 
     KSC_TRY(ensure(ix->ws_scores, sizeof(float) * nq * ix->L, st));
     float* scores = (float*)ix->ws_scores.p;
     float* err = nullptr;
-    KSC_TRY(list_scores(ix, Q, nq, mode, scores, &err, st));
+    KSC_TRY(list_scores(ix, Q, nq, mode, scores, &err, st, !feat));
     return select_lists(ix, scores, err, Q, nq, nprobe_q, Pfix, Pmax, probes, score_out, st, feat);
 }
 
@@ -3050,19 +3016,14 @@ static int launch_luts(const LutArgs& A, uint32_t* rb, uint8_t* lut, int32_t* bi
     const size_t smem = sizeof(float) * (size_t)A.M * cb_ld(A.dsub);
     const int64_t warps = (A.nq * A.Pmax + LUT_WARPS - 1) / LUT_WARPS;  // a warp per item
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(warps, (int64_t)num_sms() * 8));
-    if (lut_ds2(A)) {
-        KSC_CUDA(cudaFuncSetAttribute(k_lut_range<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        KSC_CUDA(cudaFuncSetAttribute(k_lut_quant<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_lut_range<2><<<grid, LUT_WARPS * 32, smem, st>>>(A, rb);
-        KSC_LAUNCH_CHECK();
-        k_lut_quant<2><<<grid, LUT_WARPS * 32, smem, st>>>(A, rb, lut, bias, scale);
-    } else {
-        KSC_CUDA(cudaFuncSetAttribute(k_lut_range<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        KSC_CUDA(cudaFuncSetAttribute(k_lut_quant<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_lut_range<0><<<grid, LUT_WARPS * 32, smem, st>>>(A, rb);
-        KSC_LAUNCH_CHECK();
-        k_lut_quant<0><<<grid, LUT_WARPS * 32, smem, st>>>(A, rb, lut, bias, scale);
-    }
+    const int w = lut_width(A, false);
+    auto kr = w == 2 ? k_lut_range<2> : (w == 4 ? k_lut_range<4> : k_lut_range<0>);
+    auto kq = w == 2 ? k_lut_quant<2> : (w == 4 ? k_lut_quant<4> : k_lut_quant<0>);
+    KSC_CUDA(cudaFuncSetAttribute(kr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    KSC_CUDA(cudaFuncSetAttribute(kq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    kr<<<grid, LUT_WARPS * 32, smem, st>>>(A, rb);
+    KSC_LAUNCH_CHECK();
+    kq<<<grid, LUT_WARPS * 32, smem, st>>>(A, rb, lut, bias, scale);
     KSC_LAUNCH_CHECK();
     return KSC_OK;
 }
@@ -3098,11 +3059,9 @@ static int ensure_lowp(ksc_index* ix, int prec, cudaStream_t st) {
     return KSC_OK;
 }
 
-// The band of the exact re-rank, made on first use: U8 copies of the rows
-// when every coordinate is an integer in [0, 255] (checked once; exact, a
-// quarter of the FP32 bytes), else BF16 copies; and the rows' bounds (norm,
-// rounding error).
-static int ensure_band(ksc_index* ix, cudaStream_t st) {
+// U8 copies of the re-rank rows when every coordinate is an integer in [0,
+// 255] (checked once, x_u8_state).  Synchronises the stream on first use.
+static int ensure_u8(ksc_index* ix, cudaStream_t st) {
     const int64_t m = ix->n * (int64_t)rr_d(ix);
     if (ix->x_u8_state == 0) {
         KSC_TRY(ensure(ix->ws_flag, sizeof(int32_t), st));
@@ -3123,6 +3082,29 @@ static int ensure_band(ksc_index* ix, cudaStream_t st) {
         }
         ix->x_u8_state = (h && m > 0) ? 1 : -1;  // only once the copy exists
     }
+    return KSC_OK;
+}
+
+// Whether U8 copies of the re-rank rows are there, made now if they can be: not
+// while the stream is captured, nor (for good) once the device had no room.
+static bool u8_rows(ksc_index* ix, cudaStream_t st) {
+    if (ix->x_u8_state == 0) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
+        if (ensure_u8(ix, st) != KSC_OK) {
+            cudaGetLastError();
+            ix->x_u8_state = -1;
+        }
+    }
+    return ix->x_u8_state == 1;
+}
+
+// The band of the exact re-rank, made on first use: U8 copies of the rows
+// when every coordinate is an integer in [0, 255] (checked once; exact, a
+// quarter of the FP32 bytes), else BF16 copies; and the rows' bounds (norm,
+// rounding error).
+static int ensure_band(ksc_index* ix, cudaStream_t st) {
+    KSC_TRY(ensure_u8(ix, st));
     const bool u8 = ix->x_u8_state == 1;
     if (!u8) KSC_TRY(ensure_lowp(ix, 1, st));
     if (!ix->X_band) {
@@ -3222,13 +3204,9 @@ static int rerank_stage(ksc_index* ix, const float* Qr, const Plan& pl, const ui
         KSC_TRY(ensure_lowp(ix, pl.prec, st));
         KSC_TRY(ensure(ix->ws_topr2, sizeof(uint64_t) * nq * pl.Rf, st));
         uint64_t* topr2 = (uint64_t*)ix->ws_topr2.p;
-        const size_t smem = sizeof(uint64_t) * pow2_ceil(pl.Rmax < 2 ? 2 : pl.Rmax);
-        KSC_CUDA(cudaFuncSetAttribute(k_rerank_lowp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_rerank_lowp<<<(unsigned)nq, 256, smem, st>>>(Qr, dr, ix->metric == KSC_IP, pl.prec,
-                                                       (const uint16_t*)ix->X_bf16, (const uint8_t*)ix->X_fp8,
-                                                       ix->X_scale, topr, pl.Rmax, pl.rerank_q, pl.Rfix, pl.k, pl.Rf,
-                                                       topr2);
-        KSC_LAUNCH_CHECK();
+        KSC_TRY(launch_rerank_lowp(Qr, nq, dr, ix->metric == KSC_IP, pl.prec, (const uint16_t*)ix->X_bf16,
+                                   (const uint8_t*)ix->X_fp8, ix->X_scale, topr, pl.Rmax, pl.rerank_q, pl.Rfix, pl.k,
+                                   pl.Rf, topr2, st));
         ix->launches++;
         rr_keys = topr2;
         rr_R = pl.Rf;
@@ -3247,6 +3225,11 @@ static int rerank_stage(ksc_index* ix, const float* Qr, const Plan& pl, const ui
             band && ix->x_u8_state == 1 ? (const uint8_t*)ix->X_u8 : nullptr, band ? ix->X_band : nullptr);
         ix->launches++;
         KSC_LAUNCH_CHECK();
+    } else if (pl.band && pl.prec == 0 && rr_R > pl.k && ix->metric != KSC_IP && nq >= 2 * (int64_t)num_sms() &&
+               rerank_u8_supported(dr) && u8_rows(ix, st)) {
+        KSC_TRY(launch_rerank_u8(Qr, nq, Xr, (const uint8_t*)ix->X_u8, dr, rr_keys, rr_R, rr_q, rr_R, pl.k, ids, dists,
+                                 st));
+        ix->launches++;
     } else {
         const size_t smem = rerank_smem(rr_R, pl.k);
         // a CTA per query; 1024 threads (more rows in flight) when the batch is
@@ -3519,8 +3502,8 @@ static int search_from_probes(ksc_index* ix, const float* Q, const Plan& pl, con
         const size_t fsm = lut_fused_smem(M, ix->dsub, ix->d, Pb, pl.Pq_max);
         // one CTA per query at a time: worth it once every SM has queries to take
         if (fsm <= 160 * 1024 && nq >= 2 * (int64_t)num_sms()) {
-            const bool ds2 = lut_ds2(LA);
-            auto kf = ds2 ? k_lut_fused<2> : k_lut_fused<0>;
+            const int lw = lut_width(LA, true);
+            auto kf = lw == 2 ? k_lut_fused<2> : (lw == 4 ? k_lut_fused<4> : k_lut_fused<0>);
             KSC_CUDA(cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm));
             int per_sm = 0;
             KSC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kf, 256, fsm));

@@ -327,7 +327,7 @@ __global__ void __cluster_dims__(SP_CL, 1, 1) __launch_bounds__(SP_T) k_small_pr
 
 int launch_small_prep(const SmallPrep& S, cudaStream_t st) {
     const size_t smem = small_prep_smem(S);
-    auto kern = S.T.dsub == 2 ? k_small_prep<2> : k_small_prep<0>;
+    auto kern = S.T.dsub == 2 ? k_small_prep<2> : (S.T.dsub == 4 ? k_small_prep<4> : k_small_prep<0>);
     KSC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     kern<<<(unsigned)(S.T.nq * SP_CL), SP_T, smem, st>>>(S);
     KSC_LAUNCH_CHECK();
