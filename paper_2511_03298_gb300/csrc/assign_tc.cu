@@ -285,6 +285,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
             // all four stop together)
             q_best[quarter][row] = best;
             q_n[quarter][row] = over ? -1 : n;
+            __syncwarp();  // bar.sync is a warp-collective instruction
             asm volatile("bar.sync %0, %1;" ::"r"(1 + sub), "n"(32 * AT_Q) : "memory");  // the four warps of these rows
             if (quarter == 0 && lane == 0) s_stop[sub] = s_abort;
             if (quarter == 0 && in && ok) {
@@ -323,6 +324,7 @@ __global__ void __launch_bounds__(AT_THREADS, 1)
                 if (many || k == 0 || k > AT_ROWC) G.redo[atomicAdd(G.nredo, 1)] = (int32_t)r;
                 else if (k == 1) G.assign[r] = first;
             }
+            __syncwarp();
             asm volatile("bar.sync %0, %1;" ::"r"(1 + sub), "n"(32 * AT_Q) : "memory");  // before the lists are reused
             ok = s_stop[sub] == 0;
         }
