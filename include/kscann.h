@@ -150,9 +150,11 @@ typedef struct {
                                   over the best rerank_final of them */
     int32_t rerank_final;      /* precision 1/2: FP32 re-rank size; 0 -> max(k, R/2) */
     int32_t tile_blocks;       /* scan: 32-vector blocks per work item; 0 auto */
-    int32_t scan_tc;           /* 1: the scan on the tensor cores (one-hot codes x FP16 tables,
-                                  FP32 sums of integers: the same keys as the byte-permute scan;
-                                  M <= 128, not with hybrid); 0: byte permutes on the CUDA cores */
+    int32_t scan_tc;           /* 1: the filtered scan on the tensor cores (one-hot codes x the
+                                  tables' nibbles in FP8, FP32 sums of integers: the same keys as
+                                  the byte-permute scan; M <= 128, not with hybrid); 0: chosen by
+                                  the queries per list and the lists' lengths (byte permutes when
+                                  lanes_per_query is given) */
     int32_t rank_fp8;          /* 1: list scores from FP8-e4m3 operands (queries and centroids
                                   scaled per row by a power of two) on the tensor cores, FP32
                                   accumulate; the lists their error bound cannot exclude are

@@ -229,6 +229,7 @@ __device__ __forceinline__ float exact_list_score(const float* __restrict__ qs, 
 // supported), and one launch over a work list of items of at most nt queries
 // and TB blocks (whole 4-block units).
 int tcs_nt(int M);
+constexpr int TCS_MAX_TILE = 2048;  // largest TB (a buffered key holds its vector of the tile in 16 bits)
 int launch_scan_tc(const ScanArgs& A, const ScanOut& O, const int64_t* pair_off, const int64_t* item_off,
                    const uint32_t* pairs, int L, int TB, int nt, unsigned long long* next_item, int32_t* status,
                    cudaStream_t st);

@@ -24,6 +24,7 @@
 #include "rerank.cuh"
 #include "rerank_low.cuh"
 #include "scan.cuh"
+#include "scan_ops.cuh"
 #include "small.cuh"
 
 namespace ksc {
@@ -1367,172 +1368,6 @@ __global__ void k_fill_parts(ScanArgs A, int rs, const int32_t* __restrict__ spl
 
 // ------------------------------------------------------------------ a3: LUT16 scan
 
-// Eight lookups of one 16-entry u8 table t (4 registers, entry e in byte e)
-// for the eight 4-bit codes of w (code of vector n in bits 4n..4n+3):
-// lo = bytes T[c0..c3], hi = bytes T[c4..c7].  Two byte permutes fetch
-// T[c & 7] and T[8 + (c & 7)], a third picks per byte by bit 3 of c.  A byte
-// permute reads only the low 16 bits of its selector, so both halves come
-// from one masked word and a shift.
-__device__ __forceinline__ void lut16x8(uint32_t w, const uint4& t, uint32_t& lo, uint32_t& hi) {
-    const uint32_t s0 = w & 0x77777777u;                            // entry index within a half
-    const uint32_t s1 = s0 >> 16;
-    const uint32_t k0 = ((w >> 1) & 0x44444444u) | 0x32103210u;     // byte n of a (n) or of b (4 + n)
-    const uint32_t k1 = k0 >> 16;
-    lo = prmt(prmt(t.x, t.y, s0), prmt(t.z, t.w, s0), k0);
-    hi = prmt(prmt(t.x, t.y, s1), prmt(t.z, t.w, s1), k1);
-}
-
-// Add the 16 lookups of one (subspace, 16-byte code chunk) into the u16x2
-// lane sums acc[m] = (vector 2m, vector 2m+1).
-__device__ __forceinline__ void accum_chunk(const uint4& c, const uint4& t, uint32_t (&acc)[16]) {
-    const uint32_t w[4] = {c.x, c.y, c.z, c.w};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        uint32_t lo, hi;
-        lut16x8(w[k], t, lo, hi);
-        acc[4 * k + 0] += prmt(lo, 0u, 0x4140u);
-        acc[4 * k + 1] += prmt(lo, 0u, 0x4342u);
-        acc[4 * k + 2] += prmt(hi, 0u, 0x4140u);
-        acc[4 * k + 3] += prmt(hi, 0u, 0x4342u);
-    }
-}
-
-// Two subspaces at once: each lane sum takes both widened lookups in one
-// three-input add.
-__device__ __forceinline__ void accum_pair(const uint4& c0, const uint4& t0, const uint4& c1, const uint4& t1,
-                                           uint32_t (&acc)[16]) {
-    const uint32_t w0[4] = {c0.x, c0.y, c0.z, c0.w};
-    const uint32_t w1[4] = {c1.x, c1.y, c1.z, c1.w};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        uint32_t lo0, hi0, lo1, hi1;
-        lut16x8(w0[k], t0, lo0, hi0);
-        lut16x8(w1[k], t1, lo1, hi1);
-        acc[4 * k + 0] += prmt(lo0, 0u, 0x4140u) + prmt(lo1, 0u, 0x4140u);
-        acc[4 * k + 1] += prmt(lo0, 0u, 0x4342u) + prmt(lo1, 0u, 0x4342u);
-        acc[4 * k + 2] += prmt(hi0, 0u, 0x4140u) + prmt(hi1, 0u, 0x4140u);
-        acc[4 * k + 3] += prmt(hi0, 0u, 0x4342u) + prmt(hi1, 0u, 0x4342u);
-    }
-}
-
-// Reduce-scatter of the 16 u16x2 sums over the G lanes of a group: after it,
-// group lane g holds the full sums of vectors V*g .. V*g+V-1 (V = 32/G) in
-// out[0..V) (u16 values).
-// The same lookups with the widening done by byte dot products (dp4a with a
-// one-hot byte selector adds byte b of the looked-up word to a 32-bit sum):
-// acc[v] is the sum of vector v.  The dot products issue on the FMA pipe, so
-// the integer pipe keeps only the selector and permute work.
-__device__ __forceinline__ void widen_add4(uint32_t x, uint32_t* acc) {
-    acc[0] = __dp4a(x, 0x00000001u, acc[0]);
-    acc[1] = __dp4a(x, 0x00000100u, acc[1]);
-    acc[2] = __dp4a(x, 0x00010000u, acc[2]);
-    acc[3] = __dp4a(x, 0x01000000u, acc[3]);
-}
-
-__device__ __forceinline__ void accum_chunk32(const uint4& c, const uint4& t, uint32_t (&acc)[32]) {
-    const uint32_t w[4] = {c.x, c.y, c.z, c.w};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        uint32_t lo, hi;
-        lut16x8(w[k], t, lo, hi);
-        widen_add4(lo, acc + 8 * k);
-        widen_add4(hi, acc + 8 * k + 4);
-    }
-}
-
-__device__ __forceinline__ void accum_pair32(const uint4& c0, const uint4& t0, const uint4& c1, const uint4& t1,
-                                             uint32_t (&acc)[32]) {
-    accum_chunk32(c0, t0, acc);
-    accum_chunk32(c1, t1, acc);
-}
-
-// Selectors of one code word w (eight 4-bit codes, vector n in bits 4n..4n+3)
-// for lut16x8, computed once per word and shared by every query slot of a
-// warp: (s0, s1, k0, k1).
-__device__ __forceinline__ uint4 lut16_selectors(uint32_t w) {
-    const uint32_t s0 = w & 0x77777777u;
-    const uint32_t k0 = ((w >> 1) & 0x44444444u) | 0x32103210u;
-    return make_uint4(s0, s0 >> 16, k0, k0 >> 16);
-}
-
-// The lookups of one word from its selectors: lo = T[c0..c3], hi = T[c4..c7].
-__device__ __forceinline__ void lut16x8_sel(const uint4& s, const uint4& t, uint32_t& lo, uint32_t& hi) {
-    lo = prmt(prmt(t.x, t.y, s.x), prmt(t.z, t.w, s.x), s.z);
-    hi = prmt(prmt(t.x, t.y, s.y), prmt(t.z, t.w, s.y), s.w);
-}
-
-// Two subspaces j0, j1 from shared selectors (sel[k M + j]: word k of
-// subspace j): the looked-up bytes of the same vector from both subspaces
-// are interleaved by one byte permute, so one byte dot product adds two
-// lookups to the vector's 32-bit sum (acc[v], v the vector of the block).
-__device__ __forceinline__ void accum_pair_sel(const uint4* __restrict__ sel, int M, int j0, int j1, const uint4& t0,
-                                               const uint4& t1, uint32_t (&acc)[32]) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        uint32_t lo0, hi0, lo1, hi1;
-        lut16x8_sel(sel[k * M + j0], t0, lo0, hi0);
-        lut16x8_sel(sel[k * M + j1], t1, lo1, hi1);
-        uint32_t* a = acc + 8 * k;
-        uint32_t x = prmt(lo0, lo1, 0x5140u), y = prmt(lo0, lo1, 0x7362u);
-        a[0] = __dp4a(x, 0x00000101u, a[0]);
-        a[1] = __dp4a(x, 0x01010000u, a[1]);
-        a[2] = __dp4a(y, 0x00000101u, a[2]);
-        a[3] = __dp4a(y, 0x01010000u, a[3]);
-        x = prmt(hi0, hi1, 0x5140u);
-        y = prmt(hi0, hi1, 0x7362u);
-        a[4] = __dp4a(x, 0x00000101u, a[4]);
-        a[5] = __dp4a(x, 0x01010000u, a[5]);
-        a[6] = __dp4a(y, 0x00000101u, a[6]);
-        a[7] = __dp4a(y, 0x01010000u, a[7]);
-    }
-}
-
-__device__ __forceinline__ void accum_chunk_sel(const uint4* __restrict__ sel, int M, int j, const uint4& t,
-                                                uint32_t (&acc)[32]) {
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        uint32_t lo, hi;
-        lut16x8_sel(sel[k * M + j], t, lo, hi);
-        widen_add4(lo, acc + 8 * k);
-        widen_add4(hi, acc + 8 * k + 4);
-    }
-}
-
-template <int G>
-__device__ __forceinline__ void reduce_scatter(uint32_t (&acc)[16], int lane, uint32_t (&out)[32 / G]) {
-    constexpr int V = 32 / G;
-    int nreg = 16;
-#pragma unroll
-    for (int o = G / 2; o >= 1; o >>= 1) {
-        if (nreg == 1) break;
-        const int h = nreg >> 1;
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            if (i < h) {
-                uint32_t send = up ? acc[i] : acc[i + h];
-                uint32_t keep = up ? acc[i + h] : acc[i];
-                acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-            }
-        }
-        nreg = h;
-    }
-    if constexpr (V == 1) {
-        // G = 32: one register of two vectors left; split it over lane bit 0
-        const bool odd = lane & 1;
-        uint32_t send = odd ? (acc[0] & 0xffffu) : (acc[0] >> 16);
-        uint32_t keep = odd ? (acc[0] >> 16) : (acc[0] & 0xffffu);
-        out[0] = keep + __shfl_xor_sync(0xffffffffu, send, 1);
-    } else {
-#pragma unroll
-        for (int i = 0; i < V / 2; ++i) {
-            out[2 * i] = acc[i] & 0xffffu;
-            out[2 * i + 1] = acc[i] >> 16;
-        }
-    }
-}
-
-
 // Persistent, cluster-major scan with shared-memory staging of the codes.
 // A warp takes one item = (list p, group of QG = 32/G queries that probe p,
 // tile of at most TB blocks of p) and walks the tile in chunks of
@@ -1560,24 +1395,6 @@ template <int G>
 __host__ __device__ constexpr bool scan_shared_sel() { return G == 8; }
 template <int G>
 __host__ __device__ constexpr int scan_chunk_bytes() { return scan_shared_sel<G>() ? SCAN_CHUNK_BYTES_SEL : SCAN_CHUNK_BYTES; }
-constexpr uint32_t SCAN_WAIT_LIMIT = 1u << 22;
-
-
-// Poll an mbarrier phase at most SCAN_WAIT_LIMIT times; false if it never completed.
-__device__ __forceinline__ bool scan_wait(uint32_t bar, uint32_t parity) {
-    for (uint32_t i = 0; i < SCAN_WAIT_LIMIT; ++i) {
-        uint32_t ok;
-        asm volatile(
-            "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-            : "=r"(ok)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (ok) return true;
-    }
-    return false;
-}
-
-
 // The chunk stream of one warp: items it0, it0 + stride, ...; each item's
 // blocks [b0, b1) in chunks of cb blocks.
 struct ChunkCursor {
@@ -2843,7 +2660,8 @@ struct Plan {
     int prec, Rf;  // precision variant: first re-rank of R (= Rmax) in prec, then FP32 of the best Rf
     bool band;     // exact re-rank with the band of U8 / BF16 rows (k_rerank_w)
     int Pq_max;    // bound on the per-query nprobe (<= Pmax)
-    bool tc;       // scan on the tensor cores (k_scan_tc)
+    bool tc;       // filtered scan on the tensor cores (k_scan_tc)
+    bool tc_opt;   // asked for by the caller
     int nt;        // its queries per item
     bool small;    // the small-batch kernels (small.cu) around the scan,
     bool rank;     // which also rank the lists (no ranking has run)
@@ -3390,7 +3208,7 @@ constexpr int64_t SMALL_NEAR_KEYS = 32768;
 constexpr int64_t SMALL_MAX_RECS = 1 << 22;
 static void plan_small(const ksc_index* ix, Plan& pl, const ksc_search_opts* opts, bool distinct, bool can_rank) {
     const int64_t nq = pl.nq, P = pl.Pmax;
-    if (nq == 0 || nq >= 2 * (int64_t)num_sms() || pl.hybrid || pl.tc || (pl.G != 8 && pl.G != 16) || P > SP_MAX_P ||
+    if (nq == 0 || nq >= 2 * (int64_t)num_sms() || pl.hybrid || pl.tc_opt || (pl.G != 8 && pl.G != 16) || P > SP_MAX_P ||
         nq * P > 65536 || P * ix->max_list >= (1ll << 31))
         return;
     const int64_t maxb = (ix->max_list + 31) / 32;
@@ -3407,6 +3225,7 @@ static void plan_small(const ksc_index* ix, Plan& pl, const ksc_search_opts* opt
     const int64_t nrec = nq * (P + blocks / std::min(TB, TBa) + 1);
     if (nrec > SMALL_MAX_RECS) return;
     pl.small = true;
+    pl.tc = false;
     pl.all_near = near;
     if (near && !own_cap) pl.cap = (int)std::max<int64_t>(pl.cap, keys);
     pl.TB = TB;
@@ -3567,6 +3386,16 @@ static int search_from_probes(ksc_index* ix, const float* Q, const Plan& pl, con
     return rerank_stage(ix, Qr, pl, topr, ids, dists, st);
 }
 
+// The filtered scan takes the tensor cores from this many queries per list (nq P /
+// L) on lists of this many vectors: an item's cost is mostly the expansion of its
+// codes, whatever its queries, and the staging of their tables, whatever its
+// vectors.  Search with byte permutes / tensor cores in us, 1M x 64 subspaces in
+// 1024 lists, 7 probed: 224 / 277 at 7 queries per list, 318 / 324 at 14, 396 / 353
+// at 20, 490 / 404 at 28, 976 / 718 at 68; 200k x 48 in 512 lists: 146 / 150 at 16,
+// 203 / 189 at 32, 793 / 613 at 256; in 2048 lists (100 vectors each): 210 / 232 at
+// 16, 531 / 521 at 64.
+constexpr int64_t TC_MIN_SHARE = 20, TC_MIN_LIST = 256;
+
 // Tile lengths of the scan's warp items for an expected P probes per query.
 // Short tiles balance the persistent warps, long ones amortise an item's
 // set-up: about 220 items per SM for the filtered scan, and for the smaller
@@ -3590,9 +3419,14 @@ static void set_tiles(const ksc_index* ix, Plan& pl, int64_t nq, double P, const
     pl.TB = tile(blocks * (1.0 - near), 220.0);
     pl.TBa = tile(blocks * near, 60.0);
     if (opts && opts->tile_blocks > 0) pl.TB = pl.TBa = std::min(opts->tile_blocks, 1 << 20);
-    // tensor-core scan (the filtered part only): tiles of whole 128-vector
-    // products, 32 blocks unless given
-    if (pl.tc) pl.TB = (opts && opts->tile_blocks > 0) ? (std::min(opts->tile_blocks, 1 << 20) + 3) / 4 * 4 : 32;
+    // tensor-core scan of the filtered part: asked for, or by default where
+    // enough queries share a list; tiles of whole 128-vector products, 32 blocks
+    // unless given
+    pl.tc = pl.nt > 0 && !pl.hybrid &&
+            (pl.tc_opt || (!(opts && opts->lanes_per_query) && nq * P >= TC_MIN_SHARE * ix->L &&
+                           ix->n >= TC_MIN_LIST * ix->L));
+    if (pl.tc)
+        pl.TB = (opts && opts->tile_blocks > 0) ? (std::min(opts->tile_blocks, TCS_MAX_TILE) + 3) / 4 * 4 : 32;
 }
 
 static int make_plan(ksc_index* ix, int64_t nq, int k, int Pmax, int Rmax, const ksc_search_opts* opts, Plan& pl) {
@@ -3612,7 +3446,8 @@ static int make_plan(ksc_index* ix, int64_t nq, int k, int Pmax, int Rmax, const
     pl.rerank_q = nullptr;
     pl.G = choose_G(ix, nq, Pmax, opts ? opts->lanes_per_query : 0);
     pl.nt = tcs_nt(ix->M);
-    pl.tc = opts && opts->scan_tc && !opts->hybrid && pl.nt > 0;
+    pl.hybrid = opts && opts->hybrid;
+    pl.tc_opt = opts && opts->scan_tc;
     set_tiles(ix, pl, nq, Pmax, opts);
     int cap = (opts && opts->cand_cap > 0) ? opts->cand_cap : std::max(32 * Rmax, 8192);
     pl.cap = std::max(cap, Rmax);
@@ -3631,7 +3466,6 @@ static int make_plan(ksc_index* ix, int64_t nq, int k, int Pmax, int Rmax, const
         const int rf = (opts->rerank_final > 0) ? opts->rerank_final : std::max(k, Rmax / 2);
         pl.Rf = std::min(std::max(rf, k), Rmax);
     }
-    pl.hybrid = opts && opts->hybrid;
     pl.n_near = (opts && opts->n_near > 0) ? opts->n_near : 2;
     pl.efs = (opts && opts->efs > 0) ? opts->efs : 64;
     pl.tau = (opts && opts->tau >= 0 && opts->hybrid) ? opts->tau : 8;

@@ -178,8 +178,8 @@ def _hptr(a):
 def search_opts(lanes_per_query=0, hybrid=False, n_near=2, efs=64, tau=8, cand_cap=0, rank_fp32=False,
                 precision=0, rerank_final=0, tile_blocks=0, scan_tc=False, rank_fp8=False, rerank_band=0):
     """precision: 0 FP32 re-rank; 1 BF16 / 2 FP8 first re-rank of the widened
-    shortlist, then FP32 over the best rerank_final.  scan_tc: the scan on
-    the tensor cores (same keys).  rank_fp8: list scores from FP8 operands
+    shortlist, then FP32 over the best rerank_final.  scan_tc: the filtered
+    scan on the tensor cores (same keys) also where it is not the default.  rank_fp8: list scores from FP8 operands
     (same ranking).  rerank_band: 1 the exact re-rank reads U8 rows (exact,
     when every coordinate is an integer in [0, 255]) or BF16 rows first and
     FP32 rows only where its bound cannot exclude a candidate (same results),
