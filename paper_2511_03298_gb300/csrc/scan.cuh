@@ -158,12 +158,29 @@ __device__ __forceinline__ int32_t scalar_dist(const uint8_t* __restrict__ lutp,
     return D;
 }
 
-// A query whose candidate store overflowed, redone exactly by one CTA: every
-// key of every probed list is recomputed (scalar lookups) inside the radix
-// select.  The min(R, keys) smallest, sorted, into out; their number.  buf:
-// sel_cap keys (may be out), s_pref: one more than the query's probes.
-__device__ __forceinline__ int redo_select(const ScanArgs& A, int64_t q, int R, uint64_t* out, uint64_t* buf, int sel_cap,
-                                           uint32_t* hist, int32_t* s_pref) {
+// The keys of query q by position over all its probed lists, recomputed with
+// scalar lookups; s_pref: one more shared word than the query's probes.
+struct QueryKeys {
+    const ScanArgs& A;
+    int64_t q;
+    int P;
+    const int32_t* pref;
+    __device__ __forceinline__ uint64_t operator()(int i) const {
+        int lo = 0, hi = P - 1;
+        while (lo < hi) {
+            int mid = (lo + hi + 1) >> 1;
+            if (pref[mid] <= i) lo = mid; else hi = mid - 1;
+        }
+        const int64_t item = q * A.Pmax + lo;
+        const int p = A.probes[item];
+        const int m = i - pref[lo];
+        const int64_t blk = A.boff[p] + (m >> 5);
+        const int v = m & 31;
+        int32_t D = scalar_dist(A.lut + item * A.M * PQ_K, A.bias[item], A.codes + blk * A.M * 16, A.M, v);
+        return make_key(D, A.ids[blk * 32 + v]);
+    }
+};
+__device__ __forceinline__ QueryKeys query_keys(const ScanArgs& A, int64_t q, int32_t* s_pref) {
     const int P = nprobe_of(A, q);
     __syncthreads();  // s_pref of the previous query is no longer read
     if (threadIdx.x == 0) {
@@ -176,23 +193,50 @@ __device__ __forceinline__ int redo_select(const ScanArgs& A, int64_t q, int R, 
         s_pref[P] = acc;
     }
     __syncthreads();
-    const int N = s_pref[P];
-    auto load = [&](int i) -> uint64_t {
-        int lo = 0, hi = P - 1;
-        while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (s_pref[mid] <= i) lo = mid; else hi = mid - 1;
+    return QueryKeys{A, q, P, s_pref};
+}
+
+// The R best keys of a query whose store (`row`, cap keys, all written)
+// overflowed, in no particular order unless the last way is taken.  The row's
+// keys are some of the query's, so their R-th smallest bounds the R-th of all:
+// one pass over the recomputed keys gathers those at or below it in the row,
+// from which the R best are selected.  Only where these overflow the row as
+// well (or it holds R keys at most) the selection recomputes every key in each
+// of its nine passes.  3 queries of 9100 keys (8192 stored, 50 subspaces): 2600 us before,
+// 50 now.
+// hist: 256 shared words, 16-byte aligned; bb: 32; sel: sel_cap keys for the last
+// way (may be out).  All threads of the CTA; returns min(R, keys).
+__device__ __forceinline__ int redo_select(const ScanArgs& A, int64_t q, int R, uint64_t* row, int cap, uint64_t* out,
+                                           uint64_t* sel, int sel_cap, uint32_t* hist, uint64_t* bb, int32_t* s_pref) {
+    __shared__ int s_kept;
+    const QueryKeys key = query_keys(A, q, s_pref);
+    const int N = s_pref[key.P];
+    if (R < cap) {
+        auto stored = [&](int i) -> uint64_t { return row[i]; };
+        const uint64_t bound = block_topk(stored, cap, R, [](int, uint64_t) {}, hist, bb);
+        if (threadIdx.x == 0) s_kept = 0;
+        __syncthreads();  // (and the row has been read)
+        for (int i = threadIdx.x; i < N; i += blockDim.x) {
+            const uint64_t k = key(i);
+            if (k > bound) continue;
+            const int at = atomicAdd(&s_kept, 1);
+            if (at < cap) row[at] = k;
         }
-        const int64_t item = q * A.Pmax + lo;
-        const int p = A.probes[item];
-        const int m = i - s_pref[lo];
-        const int64_t blk = A.boff[p] + (m >> 5);
-        const int v = m & 31;
-        int32_t D = scalar_dist(A.lut + item * A.M * PQ_K, A.bias[item], A.codes + blk * A.M * 16, A.M, v);
-        return make_key(D, A.ids[blk * 32 + v]);
-    };
+        __syncthreads();
+        const int n = s_kept;  // at least R: the bound and the R - 1 stored keys below it are among them
+        if (n == R) {
+            for (int i = threadIdx.x; i < n; i += blockDim.x) out[i] = row[i];
+            __syncthreads();
+            return R;
+        }
+        if (n <= cap) {
+            block_topk(stored, n, R, [&](int i, uint64_t k) { out[i] = k; }, hist, bb);
+            __syncthreads();
+            return R;
+        }
+    }
     const int K = min(R, N);
-    block_select_smallest(load, N, K, out, buf, sel_cap, hist);
+    block_select_smallest([&](int i) -> uint64_t { return key(i); }, N, K, out, sel, sel_cap, hist);
     return K;
 }
 

@@ -2202,17 +2202,19 @@ __global__ void __launch_bounds__(NT) k_select_cta(ScanArgs A, int Rmax, const i
 }
 
 // The queries on the redo list.  A persistent grid walks it (usually empty).
-__global__ void __launch_bounds__(256) k_select_redo(ScanArgs A, int Rmax, int sel_cap, uint64_t* __restrict__ topr,
-                                                     int32_t* __restrict__ ncand, const int32_t* __restrict__ redo) {
+__global__ void __launch_bounds__(1024) k_select_redo(ScanArgs A, int Rmax, int sel_cap, uint64_t* cand, int cap,
+                                                      uint64_t* __restrict__ topr, int32_t* __restrict__ ncand,
+                                                      const int32_t* __restrict__ redo) {
     extern __shared__ uint64_t sbuf[];  // sel_cap keys
-    __shared__ uint32_t hist[256];
+    __shared__ __align__(16) uint32_t hist[256];
+    __shared__ uint64_t bb[32];
     __shared__ int32_t s_pref[MAX_NPROBE + 1];
     const int nredo = redo[0];
     for (int r0 = blockIdx.x; r0 < nredo; r0 += gridDim.x) {
         const int64_t q = redo[1 + r0];
         const int R = rerank_of(A.rerank_q, A.Rfix, A.Rmin, Rmax, q);
         uint64_t* out = topr + q * Rmax;
-        const int K = redo_select(A, q, R, out, sbuf, sel_cap, hist, s_pref);
+        const int K = redo_select(A, q, R, cand + q * cap, cap, out, sbuf, sel_cap, hist, bb, s_pref);
         for (int i = K + threadIdx.x; i < Rmax; i += blockDim.x) out[i] = KEY_NONE;
         if (threadIdx.x == 0 && ncand) ncand[q] = K;
     }
@@ -3069,7 +3071,7 @@ static int rerank_stage(ksc_index* ix, const float* Qr, const Plan& pl, const ui
 }
 
 // 5. the R best keys per query into topr (and, sorted, cand_out)
-static int select_stage(ksc_index* ix, const Plan& pl, const ScanArgs& A, const int32_t* cnt, const uint64_t* cand,
+static int select_stage(ksc_index* ix, const Plan& pl, const ScanArgs& A, const int32_t* cnt, uint64_t* cand,
                         uint64_t* topr, uint64_t* cand_out, int32_t* ncand_out, cudaStream_t st) {
     const int64_t nq = pl.nq;
     {
@@ -3087,12 +3089,11 @@ static int select_stage(ksc_index* ix, const Plan& pl, const ScanArgs& A, const 
             k_select_cta<256><<<(unsigned)nq, 256, 0, st>>>(A, pl.Rmax, cnt, cand, pl.cap, topr, ncand_out,
                                                              ix->status, ix->stats, redo);
         KSC_LAUNCH_CHECK();
-        // overflowed queries (usually none): radix select over recomputed keys,
-        // the R best plus their sort in a buffer of sel_cap keys
+        // overflowed queries (usually none): their keys recomputed
         const int sel_cap = sel_keys(pl.Rmax);
         const size_t smem = sel_cap * sizeof(uint64_t);
         KSC_CUDA(cudaFuncSetAttribute(k_select_redo, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_select_redo<<<num_sms() * 2, 256, smem, st>>>(A, pl.Rmax, sel_cap, topr, ncand_out, redo);
+        k_select_redo<<<num_sms(), 1024, smem, st>>>(A, pl.Rmax, sel_cap, cand, pl.cap, topr, ncand_out, redo);
         KSC_LAUNCH_CHECK();
         ix->launches += 2;
     }

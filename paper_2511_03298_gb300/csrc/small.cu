@@ -336,7 +336,7 @@ int launch_small_prep(const SmallPrep& S, cudaStream_t st) {
 
 template <int NT>
 __global__ void __launch_bounds__(NT) k_select_rerank(ScanArgs A, int Rmax, const int32_t* __restrict__ cnt,
-                                                      const uint64_t* __restrict__ cand, int cap, int nkeys,
+                                                      uint64_t* cand, int cap, int nkeys,
                                                       int sel_cap, const float* __restrict__ Q,
                                                       const float* __restrict__ X, int d, int ip, int k,
                                                       int64_t* __restrict__ out_ids, float* __restrict__ out_d,
@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(NT) k_select_rerank(ScanArgs A, int Rmax, cons
             atomicAdd(&stats[0], 1ull);
             atomicOr(status, KSC_STATUS_CAND_OVERFLOW);
         }
-        K = redo_select(A, q, R, sr_keys, sr_keys, sel_cap, hist, s_pref);
+        K = redo_select(A, q, R, cand + q * cap, cap, sr_keys, sr_keys, sel_cap, hist, bb, s_pref);
     } else {
         K = min(R, n);
         if (n <= K) {
@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(NT) k_select_rerank(ScanArgs A, int Rmax, cons
     cta_rerank<NT>(sr_keys, R, sr_keys + nkeys, qs, X, d, ip, k, out_ids + q * k, out_d + q * k);
 }
 
-int launch_select_rerank(const ScanArgs& A, int Rmax, const int32_t* cnt, const uint64_t* cand, int cap, int sel_cap,
+int launch_select_rerank(const ScanArgs& A, int Rmax, const int32_t* cnt, uint64_t* cand, int cap, int sel_cap,
                          const float* Q, const float* X, int d, int ip, int k, int64_t* ids, float* dists,
                          int32_t* status, unsigned long long* stats, cudaStream_t st) {
     const int nkeys = Rmax > sel_cap ? Rmax : sel_cap;

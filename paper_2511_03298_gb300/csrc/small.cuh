@@ -37,7 +37,7 @@ int launch_small_prep(const SmallPrep& S, cudaStream_t st);
 
 // One CTA per query: the R best keys of its store (redone exactly if it
 // overflowed) and their exact re-rank.
-int launch_select_rerank(const ScanArgs& A, int Rmax, const int32_t* cnt, const uint64_t* cand, int cap, int sel_cap,
+int launch_select_rerank(const ScanArgs& A, int Rmax, const int32_t* cnt, uint64_t* cand, int cap, int sel_cap,
                          const float* Q, const float* X, int d, int ip, int k, int64_t* ids, float* dists,
                          int32_t* status, unsigned long long* stats, cudaStream_t st);
 
