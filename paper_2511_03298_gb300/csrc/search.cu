@@ -858,7 +858,7 @@ __global__ void __launch_bounds__(LUT_WARPS * 32) k_lut_quant(LutArgs A, const u
 constexpr int LUT_TROW = 20;
 
 template <int DS>
-__global__ void __launch_bounds__(256) k_lut_fused(LutArgs A, int Pb, int Pm, uint8_t* __restrict__ lut,
+__global__ void __launch_bounds__(512) k_lut_fused(LutArgs A, int Pb, int Pm, uint8_t* __restrict__ lut,
                                                    int32_t* __restrict__ bias, float* __restrict__ scale) {
     extern __shared__ __align__(16) float fsm[];
     const int M = A.M;
@@ -3325,10 +3325,18 @@ static int search_from_probes(ksc_index* ix, const float* Q, const Plan& pl, con
             const int lw = lut_width(LA, true);
             auto kf = lw == 2 ? k_lut_fused<2> : (lw == 4 ? k_lut_fused<4> : k_lut_fused<0>);
             KSC_CUDA(cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm));
-            int per_sm = 0;
+            // 512 threads per CTA where the tables leave an SM few CTAs and so more
+            // warps run (60k x 784, M 196, nprobe 4: the search 1567 -> 1438 us; M 48
+            // with up to 256 probes per query: 800 -> 745)
+            int per_sm = 0, per_sm2 = 0, nt = 256;
             KSC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kf, 256, fsm));
+            KSC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm2, kf, 512, fsm));
+            if (2 * per_sm2 > per_sm) {
+                nt = 512;
+                per_sm = per_sm2;
+            }
             const int64_t grid = std::min<int64_t>(nq, (int64_t)num_sms() * (per_sm > 0 ? per_sm : 1));
-            kf<<<(unsigned)grid, 256, fsm, st>>>(LA, Pb, pl.Pq_max, lut, bias, scale);
+            kf<<<(unsigned)grid, nt, fsm, st>>>(LA, Pb, pl.Pq_max, lut, bias, scale);
             KSC_LAUNCH_CHECK();
             ix->launches++;
         } else {
