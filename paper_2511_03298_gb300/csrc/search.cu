@@ -1142,6 +1142,28 @@ __device__ uint64_t warp_topk_hi(const uint64_t* __restrict__ keys, int N, int K
     return warp_topk_tied(keys, N, need, lo, dst ? dst + out : nullptr, hist, bb);
 }
 
+// The K smallest (0 < K < n) of n unique keys (block_topk's rules), by a CTA of NT
+// threads: up to NT U keys are held in registers, read once, and emit may then
+// overwrite them; more (or U = 0) are read again in each pass.
+template <int NT, int U, class Emit>
+__device__ __forceinline__ uint64_t cta_topk(const uint64_t* keys, int n, int K, Emit emit, uint32_t* hist,
+                                             uint64_t* bb) {
+    if constexpr (U > 0) {
+        if (n <= NT * U) {
+            uint64_t kk[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) kk[u] = (int)threadIdx.x + u * NT < n ? keys[threadIdx.x + u * NT] : KEY_NONE;
+            auto each = [&](auto f) {
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (u * NT < n) f((int)threadIdx.x + u * NT < n, kk[u]);
+            };
+            return block_topk_each(each, K, emit, hist, bb);
+        }
+    }
+    return block_topk([&](int i) -> uint64_t { return keys[i]; }, n, K, emit, hist, bb);
+}
+
 // ------------------------------------------------------------------ threshold
 // Per query, after the scan of its nearest list(s) with no filter: the R-th
 // smallest of the keys found so far bounds the R-th smallest key of the whole
@@ -1152,7 +1174,13 @@ __device__ uint64_t warp_topk_hi(const uint64_t* __restrict__ keys, int N, int K
 // (gathered in `scratch`, a row of Rmax keys per query, then copied back),
 // unless it overflowed (the final select then redoes the query).
 constexpr int SW_WARPS = 8;        // queries per CTA of the warp selection kernels
-constexpr int SW_MAX_KEYS = 2048;  // expected keys per query up to which a warp selects
+constexpr int SW_MAX_KEYS = 2048;  // expected keys per query up to which a warp selects ...
+// ... in batches that fill the GPU; above SW_CTA_KEYS a CTA of 128 threads with its
+// keys in registers.  A warp reads its keys from L2 in each of three passes and
+// more, a CTA once, at the cost of some nine barriers: at R 400 (3001 queries) the
+// search takes 547 us by warps and 498 by CTAs, the hybrid search with 1560 near
+// keys 732 and 705, at R 200 (10,000 queries) 904 and 951.
+constexpr int SW_CTA_KEYS = 1024;
 
 __global__ void __launch_bounds__(SW_WARPS * 32) k_threshold(ScanArgs A, int Rmax, int32_t* __restrict__ cnt,
                                                              uint64_t* __restrict__ cand, int cap,
@@ -1191,8 +1219,9 @@ __global__ void __launch_bounds__(SW_WARPS * 32) k_threshold(ScanArgs A, int Rma
 }
 
 // The same with one CTA per query, for queries with many keys (NT threads:
-// 1024 when the batch is too small to fill the GPU with 256-thread CTAs).
-template <int NT>
+// 1024 when the batch is too small to fill the GPU with 256-thread CTAs; U keys
+// per thread in registers).
+template <int NT, int U>
 __global__ void __launch_bounds__(NT) k_threshold_cta(ScanArgs A, int Rmax, int32_t* __restrict__ cnt,
                                                        uint64_t* __restrict__ cand, int cap,
                                                        uint64_t* __restrict__ scratch,
@@ -1216,14 +1245,14 @@ __global__ void __launch_bounds__(NT) k_threshold_cta(ScanArgs A, int Rmax, int3
         __syncthreads();
         t = s_m;
     } else if (n > R) {
-        uint64_t* sq = scratch + q * Rmax;
-        auto load = [&](int i) -> uint64_t { return cq[i]; };
+        uint64_t* sq = n <= NT * U ? cq : scratch + q * Rmax;
         auto emit = [&](int i, uint64_t k) {
             if (!ovf) sq[i] = k;
         };
-        t = block_topk(load, n, R, emit, hist, bb);
+        t = cta_topk<NT, U>(cq, n, R, emit, hist, bb);
         if (!ovf) {
-            for (int i = threadIdx.x; i < R; i += blockDim.x) cq[i] = sq[i];
+            if (sq != cq)
+                for (int i = threadIdx.x; i < R; i += blockDim.x) cq[i] = sq[i];
             if (threadIdx.x == 0) cnt[q] = R;
         }
     }
@@ -2163,7 +2192,7 @@ __global__ void __launch_bounds__(SW_WARPS * 32) k_select(ScanArgs A, int Rmax, 
 }
 
 // The same with one CTA per query, for queries with many candidates.
-template <int NT>
+template <int NT, int U>
 __global__ void __launch_bounds__(NT) k_select_cta(ScanArgs A, int Rmax, const int32_t* __restrict__ cnt,
                                                     const uint64_t* __restrict__ cand, int cap,
                                                     uint64_t* __restrict__ topr, int32_t* __restrict__ ncand,
@@ -2193,9 +2222,8 @@ __global__ void __launch_bounds__(NT) k_select_cta(ScanArgs A, int Rmax, const i
     if (n <= K) {
         for (int i = threadIdx.x; i < n; i += blockDim.x) out[i] = cq[i];
     } else {
-        auto load = [&](int i) -> uint64_t { return cq[i]; };
         auto emit = [&](int i, uint64_t k) { out[i] = k; };
-        block_topk(load, n, K, emit, hist, bb);
+        cta_topk<NT, U>(cq, n, K, emit, hist, bb);
     }
     for (int i = K + threadIdx.x; i < Rmax; i += blockDim.x) out[i] = KEY_NONE;
     if (threadIdx.x == 0 && ncand) ncand[q] = K;
@@ -3079,15 +3107,15 @@ static int select_stage(ksc_index* ix, const Plan& pl, const ScanArgs& A, const 
         int32_t* redo = (int32_t*)ix->ws_redo.p;
         KSC_CUDA(cudaMemsetAsync(redo, 0, sizeof(int32_t), st));
         // candidates per query: the R kept by the threshold plus a few R more
-        if (4 * pl.Rmax <= SW_MAX_KEYS && warp_per_query(nq))
+        if (4 * pl.Rmax <= SW_CTA_KEYS && warp_per_query(nq)) {
             k_select<<<(unsigned)((nq + SW_WARPS - 1) / SW_WARPS), SW_WARPS * 32, 0, st>>>(
                 A, pl.Rmax, cnt, cand, pl.cap, topr, ncand_out, ix->status, ix->stats, redo);
-        else if (nq < 2 * (int64_t)num_sms())  // few queries: more threads per query
-            k_select_cta<1024><<<(unsigned)nq, 1024, 0, st>>>(A, pl.Rmax, cnt, cand, pl.cap, topr, ncand_out,
-                                                               ix->status, ix->stats, redo);
-        else
-            k_select_cta<256><<<(unsigned)nq, 256, 0, st>>>(A, pl.Rmax, cnt, cand, pl.cap, topr, ncand_out,
-                                                             ix->status, ix->stats, redo);
+        } else {
+            const bool few = nq < 2 * (int64_t)num_sms(), narrow = 4 * pl.Rmax <= SW_MAX_KEYS && warp_per_query(nq);
+            auto kf = few ? k_select_cta<1024, 0> : narrow ? k_select_cta<128, 16> : k_select_cta<256, 0>;
+            kf<<<(unsigned)nq, few ? 1024 : narrow ? 128 : 256, 0, st>>>(A, pl.Rmax, cnt, cand, pl.cap, topr, ncand_out,
+                                                                        ix->status, ix->stats, redo);
+        }
         KSC_LAUNCH_CHECK();
         // overflowed queries (usually none): their keys recomputed
         const int sel_cap = sel_keys(pl.Rmax);
@@ -3160,7 +3188,7 @@ static int search_small(ksc_index* ix, const float* Q, const Plan& pl, const int
                      nullptr, false));
     ix->launches++;
     if (!pl.all_near) {
-        k_threshold_cta<1024><<<(unsigned)nq, 1024, 0, st>>>(A, pl.Rmax, cnt, cand, pl.cap, topr, thr);
+        k_threshold_cta<1024, 0><<<(unsigned)nq, 1024, 0, st>>>(A, pl.Rmax, cnt, cand, pl.cap, topr, thr);
         KSC_LAUNCH_CHECK();
         ix->launches++;
     }
@@ -3347,15 +3375,18 @@ static int search_from_probes(ksc_index* ix, const float* Q, const Plan& pl, con
     // 3. scan of the nearest lists with no filter, then the threshold
     mark(ix, 3, st);
     KSC_TRY(run_scan(pl, M, A, ScanOut{nullptr, cnt, cand, pl.cap}, wa, L, ix->status, st, tc_next, false));
-    // expected keys per query of the unfiltered scan: max(4 R, N / 16), N from
-    // the mean list length; a warp per query up to SW_MAX_KEYS, else a CTA
-    if (std::max(4.0 * pl.Rmax, (double)pl.Pmax * ix->n / L / 16.0) <= SW_MAX_KEYS && warp_per_query(nq))
+    // expected keys per query of the unfiltered scan from the mean list length:
+    // max(4 R, N / 16), or the hybrid search's near lists
+    const double near = pl.hybrid ? (double)rA * ix->n / L
+                                  : std::max(4.0 * pl.Rmax, (double)pl.Pmax * ix->n / L / 16.0);
+    if (near <= SW_CTA_KEYS && warp_per_query(nq)) {
         k_threshold<<<(unsigned)((nq + SW_WARPS - 1) / SW_WARPS), SW_WARPS * 32, 0, st>>>(A, pl.Rmax, cnt, cand,
                                                                                            pl.cap, topr, thr);
-    else if (nq < 2 * (int64_t)num_sms())  // few queries: more threads per query
-        k_threshold_cta<1024><<<(unsigned)nq, 1024, 0, st>>>(A, pl.Rmax, cnt, cand, pl.cap, topr, thr);
-    else
-        k_threshold_cta<256><<<(unsigned)nq, 256, 0, st>>>(A, pl.Rmax, cnt, cand, pl.cap, topr, thr);
+    } else {
+        const bool few = nq < 2 * (int64_t)num_sms(), narrow = near <= SW_MAX_KEYS && warp_per_query(nq);
+        auto kf = few ? k_threshold_cta<1024, 0> : narrow ? k_threshold_cta<128, 16> : k_threshold_cta<256, 0>;
+        kf<<<(unsigned)nq, few ? 1024 : narrow ? 128 : 256, 0, st>>>(A, pl.Rmax, cnt, cand, pl.cap, topr, thr);
+    }
     KSC_LAUNCH_CHECK();
     ix->launches += 2;
     // 4. scan of the other lists, keeping keys at or below the threshold;
