@@ -3232,13 +3232,17 @@ static int search_small(ksc_index* ix, const float* Q, const Plan& pl, const int
 // 256 and R up to 1000 of 1M x 96 158 and 73.
 //  - all_near: if no query can probe more than SMALL_NEAR_KEYS keys, the store
 //    holds all of them and the threshold, the second scan and its items go.
+//  - pairs of a query and a probed list: with many, the general path's shared
+//    lists win (299 queries at up to 144 probes of 758k x 96, 43,000 pairs: 288 us
+//    here, 265 there; 158 at up to 199, 31,000 pairs: 205 here, 234 there).
+constexpr int64_t SMALL_MAX_PAIRS = 40000;
 constexpr int64_t SMALL_RANK_BYTES = 64 << 20;
 constexpr int64_t SMALL_NEAR_KEYS = 32768;
 constexpr int64_t SMALL_MAX_RECS = 1 << 22;
 static void plan_small(const ksc_index* ix, Plan& pl, const ksc_search_opts* opts, bool distinct, bool can_rank) {
     const int64_t nq = pl.nq, P = pl.Pmax;
     if (nq == 0 || nq >= 2 * (int64_t)num_sms() || pl.hybrid || pl.tc_opt || (pl.G != 8 && pl.G != 16) || P > SP_MAX_P ||
-        nq * P > 65536 || P * ix->max_list >= (1ll << 31))
+        nq * P > SMALL_MAX_PAIRS || P * ix->max_list >= (1ll << 31))
         return;
     const int64_t maxb = (ix->max_list + 31) / 32;
     const int64_t blocks = distinct ? ix->h_top_blocks[P] : P * maxb;
