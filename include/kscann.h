@@ -160,7 +160,8 @@ typedef struct {
                                   accumulate; the lists their error bound cannot exclude are
                                   re-scored exactly, so the ranking is the same (rank_fp32 wins
                                   when both are set) */
-    int32_t rerank_band;       /* exact FP32 re-rank (precision 0, k <= 32, d <= 128): 1 first reads
+    int32_t rerank_band;       /* exact FP32 re-rank (precision 0; k <= 32 and d <= 128, or byte-valued
+                                  rows in larger batches at any k and d): 1 first reads
                                   low-precision copies of the candidate rows and bounds each FP32
                                   distance (the row's own rounding error plus FP32 evaluation
                                   error); only candidates whose lower bound is at most the k-th
