@@ -3357,13 +3357,14 @@ static int search_from_probes(ksc_index* ix, const float* Q, const Plan& pl, con
             const int lw = lut_width(LA, true);
             auto kf = lw == 2 ? k_lut_fused<2> : (lw == 4 ? k_lut_fused<4> : k_lut_fused<0>);
             KSC_CUDA(cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsm));
-            // 512 threads per CTA where the tables leave an SM few CTAs and so more
-            // warps run (60k x 784, M 196, nprobe 4: the search 1567 -> 1438 us; M 48
-            // with up to 256 probes per query: 800 -> 745)
+            // 512 threads per CTA where they cost no CTA, so the tables alone limit
+            // them (60k x 784, M 196, nprobe 4: the search 1567 -> 1438 us), or a query
+            // has many rows (M 48, up to 256 probes: 800 -> 745); with 4 CTAs of 256
+            // against 3 (M 64, nprobe 8) they were slower (904 -> 916)
             int per_sm = 0, per_sm2 = 0, nt = 256;
             KSC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kf, 256, fsm));
             KSC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm2, kf, 512, fsm));
-            if (2 * per_sm2 > per_sm) {
+            if (per_sm2 >= std::max(per_sm, 1) || (per_sm2 > 0 && (int64_t)pl.Pq_max * M >= 4096)) {
                 nt = 512;
                 per_sm = per_sm2;
             }
