@@ -38,8 +38,8 @@ namespace ksc {
 // instruction per 10 cycles and warp) a tile of 128 vectors x 34 queries took
 // 12000 cycles; short loops, one barrier per 4 chunks and 8 staging warps brought
 // it to 4000 to 5500.  An MMA of these shapes takes 80 cycles whatever its N (32
-// a tile).  The scan of 1M x 64 subspaces for 10k queries x 7 lists: 700 us with
-// byte permutes, 290 us here; the search 1290 -> 895 us.
+// a tile).  The scan of 1M x 64 subspaces for 10k queries x 8 lists: 707 us with
+// byte permutes, 327 us here; the search 1290 -> 899 us.
 // Every wait is bounded; a failed one stops all roles.
 constexpr int TS_NT = 64;      // queries per item at most
 constexpr int TS_EXP = 8, TS_EPI = 8, TS_STG = 8;  // expanding, epilogue, staging warps
