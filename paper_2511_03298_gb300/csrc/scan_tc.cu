@@ -610,6 +610,7 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                     mykc[col] = 0;
                     s_pick[warp - TS_W_EPI][__popc(ms & below)] = (uint8_t)lane;
                 }
+                __syncwarp();  // s_pick is read by other lanes (votes and reductions order no memory)
                 most = __reduce_max_sync(0xffffffffu, sel ? 0 : cnt);
                 const int32_t* idp = A.ids + (x.gb + x.b0) * 32;
 #pragma unroll 1
