@@ -707,6 +707,9 @@ static int lloyd(const float* X, const int64_t* sample_dev, int64_t ns, int d, i
     LL_CUDA(cudaMalloc(&Xs, sizeof(float) * ns * d));
     LL_CUDA(cudaMalloc(&cn, sizeof(float) * L));
     LL_CUDA(cudaMalloc(&a, sizeof(int32_t) * ns));
+    // an assignment on the tensor cores that gives up leaves rows undecided: they
+    // then hold a list of an earlier round (or list 0) until the check below
+    LL_CUDA(cudaMemsetAsync(a, 0, sizeof(int32_t) * ns, st));
     LL_CUDA(cudaMalloc(&sums, sizeof(double) * L * d));
     LL_CUDA(cudaMalloc(&cnt, sizeof(unsigned long long) * L));
     k_gather_rows<<<grid_for(ns * d), 256, 0, st>>>(X, sample_dev, ns, d, Xs);
@@ -737,6 +740,7 @@ static int lloyd(const float* X, const int64_t* sample_dev, int64_t ns, int d, i
         LL_CUDA(cudaGetLastError());
     }
     LL_CUDA(cudaStreamSynchronize(st));
+    if (T && rc == KSC_OK) rc = T->check(st);
     cleanup();
 #undef LL_CUDA
     return rc;
@@ -1054,6 +1058,7 @@ int ksc_build_index(const float* X_dev, int64_t n, int32_t d, int32_t nlist, int
                 if (r0) B_CUDA(cudaMemsetAsync(T.small, 0, sizeof(int32_t) * 2, st));
                 rc = assign_rows(T, ix->assign + r0, st);
             }
+            if (rc == KSC_OK) rc = T.check(st);  // before anything indexes with the lists
             if (rc) break;
         } else {
             k_assign<<<(unsigned)((n + AS_T - 1) / AS_T), 256, 0, st>>>(ix->X, n, d, ix->c_rank, ix->c_rank_sq, nlist,
@@ -1101,7 +1106,6 @@ int ksc_build_index(const float* X_dev, int64_t n, int32_t d, int32_t nlist, int
         B_CUDA(cudaGetLastError());
         B_CUDA(cudaMemcpyAsync(assign_host.data(), ix->assign, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, st));
         B_CUDA(cudaStreamSynchronize(st));
-        if (tc && (rc = T.check(st))) break;
         if ((rc = pack_lists(ix, codes_dev, assign_host.data(), st))) break;
         if ((rc = finish_common(ix, st))) break;
         if (opts && opts->build_graph) {
