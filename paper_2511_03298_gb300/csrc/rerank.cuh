@@ -153,7 +153,9 @@ __device__ __forceinline__ void cta_rerank(uint64_t* keys, int R, uint64_t* kbuf
         }
     }
     __syncthreads();
-    // an empty slot i becomes KEY_NONE - i: every key is then unique
+    // an empty slot i becomes KEY_NONE - i, which tells it from a candidate below
+    // (a list given twice by the caller's probes repeats its keys: places of
+    // equal keys go by position)
     for (int i = threadIdx.x; i < R; i += NT)
         if (keys[i] == KEY_NONE) keys[i] = KEY_NONE - (uint64_t)i;
     __syncthreads();
@@ -177,7 +179,10 @@ __device__ __forceinline__ void cta_rerank(uint64_t* keys, int R, uint64_t* kbuf
             const uint64_t v = i < R ? keys[i] : 0ull;
             int rank = 0;
 #pragma unroll 8
-            for (int j = o; j < R; j += parts) rank += keys[j] < v;
+            for (int j = o; j < R; j += parts) {
+                const uint64_t y = keys[j];
+                rank += y < v || (y == v && j < i);
+            }
             for (int s = parts >> 1; s > 0; s >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, s);
             if (i < R && o == 0 && rank < k) put(rank, v);
         }
@@ -197,7 +202,10 @@ __device__ __forceinline__ void cta_rerank(uint64_t* keys, int R, uint64_t* kbuf
             const uint64_t v = kbuf[i];
             int rank = 0;
 #pragma unroll 8
-            for (int j = 0; j < kr; ++j) rank += kbuf[j] < v;
+            for (int j = 0; j < kr; ++j) {
+                const uint64_t y = kbuf[j];
+                rank += y < v || (y == v && j < i);
+            }
             put(rank, v);
         }
     }
