@@ -44,6 +44,7 @@ struct ksc_index {
     float* X_scale = nullptr;      // [n] their per-row scales
     void* X_u8 = nullptr;          // [n x d] U8 rows when every coordinate is an integer in [0, 255] (exact)
     int x_u8_state = 0;            // 0 not checked, 1 X_u8 holds the rows exactly, -1 they do not fit bytes
+    int rank_tc_state = 0;         // rank_tc_narrow: 0 not checked, 1 narrow, -1 wide
     float2* X_band = nullptr;      // [n] per re-rank row: bounds of its norm and of its BF16 rounding error's norm (made on first use)
     // device status word, then [STATUS_NREC] the small-batch search's two item
     // counts, then [STATUS_STATS] the counters (stats: in the same allocation)
@@ -108,6 +109,10 @@ int free_index_memory(ksc_index* ix);
 // Tensor-core list scores (rank_tc.cu): approximate scores [nq x L] and a
 // per-query bound err [nq] on their error.
 int rank_scores_tc(ksc_index* ix, const float* Q, int64_t nq, float* scores, float* err, cudaStream_t st);
+// Whether the 16-bit scores suit the ranking of wide rows (once per index), for
+// at most RANK_TC_LISTS lists.
+constexpr int RANK_TC_LISTS = 1024;
+int rank_tc_narrow(ksc_index* ix, bool* narrow, cudaStream_t st);
 // The same from e4m3 operands with per-row power-of-two scales (FP8 option).
 int rank_scores_tc8(ksc_index* ix, const float* Q, int64_t nq, float* scores, float* err, cudaStream_t st);
 // Per-query error bound of the list scores (tensor-core or FP32 path).

@@ -28,6 +28,7 @@
 #include <vector>
 
 #include "index.cuh"
+#include "scan.cuh"
 #include "tc.cuh"
 
 namespace ksc {
@@ -404,6 +405,68 @@ static int err_params(ksc_index* ix, bool tensor_cores, float* rel, float* qmax,
     const float u2 = ix->tc_fp16 ? 9.77e-4f + 1e-6f : 0.0078125f + 6.2e-5f;  // 2u + u^2
     *rel = tensor_cores ? u2 + (float)ix->d * 4.8e-7f : (float)(ix->d + 8) * 1.2e-7f;
     *qmax = (tensor_cores && ix->tc_fp16) ? 6.0e4f : INFINITY;
+    return KSC_OK;
+}
+
+// Lists that the 16-bit scores' bound cannot tell from the 8 best, counted over
+// sampled centroids taken as queries: a CTA per sample.  rel: the relative
+// bound of the dot products; *total: their number over all samples.
+constexpr int RW_SAMPLES = 32, RW_BEST = 8, RW_T = 256;
+__global__ void __launch_bounds__(RW_T) k_rank_width(const float* __restrict__ C, const float* __restrict__ csq, int L,
+                                                     int d, int spherical, float rel, float cmax,
+                                                     int32_t* __restrict__ total) {
+    __shared__ __align__(16) float qs[KSC_MAX_DIM];
+    __shared__ float sc[RANK_TC_LISTS];
+    __shared__ float s_t;
+    const int s = (int)((int64_t)blockIdx.x * L / RW_SAMPLES);
+    const int lane = threadIdx.x & 31;
+    for (int t = threadIdx.x; t < d; t += RW_T) qs[t] = C[(int64_t)s * d + t];
+    if (threadIdx.x == 0) s_t = INFINITY;
+    __syncthreads();
+    for (int c = threadIdx.x >> 5; c < L; c += RW_T / 32) {
+        const float v = exact_list_score(qs, C + (int64_t)c * d, d, spherical, lane);
+        if (lane == 0) sc[c] = v;
+    }
+    __syncthreads();
+    for (int c = threadIdx.x; c < L; c += RW_T) {
+        int r = 0;
+        for (int j = 0; j < L; ++j) r += sc[j] < sc[c] || (sc[j] == sc[c] && j < c);
+        if (r == min(RW_BEST, L) - 1) s_t = sc[c];
+    }
+    __syncthreads();
+    const float dot = rel * sqrtf(csq[s]) * cmax, lim = s_t + 2.f * (spherical ? dot : 2.f * dot);
+    int n = 0;
+    for (int c = threadIdx.x; c < L; c += RW_T) n += sc[c] <= lim;
+    n = __reduce_add_sync(0xffffffffu, n);
+    if (lane == 0) atomicAdd(total, n);
+}
+
+// Whether the 16-bit scores of rows wider than the tensor cores' own range
+// (search.cu: TC_SCORES_D) tell most lists apart, from the centroids alone
+// (once per index; the bound grows with the norms, so centroids far from the
+// origin and close together defeat it).  Every list inside the bound is
+// re-scored exactly: 512 x 784, 10,000 queries: 583 us with FP32 scores, 353
+// with 16-bit ones where they leave 12 lists, 1197 where 96, 3170 where all.
+// At most RANK_TC_LISTS lists, so that the re-score buffer always holds them.
+int rank_tc_narrow(ksc_index* ix, bool* narrow, cudaStream_t st) {
+    if (ix->rank_tc_state == 0 && ix->L > RANK_TC_LISTS) ix->rank_tc_state = -1;
+    if (ix->rank_tc_state == 0) {
+        float rel, qmax;
+        KSC_TRY(err_params(ix, true, &rel, &qmax, st));  // max ||c||
+        const float u2 = ix->c_rank_max_norm < 16384.f ? 9.77e-4f + 1e-6f : 0.0078125f + 6.2e-5f;
+        rel = u2 + (float)ix->d * 4.8e-7f;
+        KSC_TRY(ensure(ix->ws_flag, sizeof(int32_t), st));
+        int32_t* total = (int32_t*)ix->ws_flag.p;
+        int32_t h = 0;
+        KSC_CUDA(cudaMemsetAsync(total, 0, sizeof(int32_t), st));
+        k_rank_width<<<RW_SAMPLES, RW_T, 0, st>>>(ix->c_rank, ix->c_rank_sq, ix->L, ix->d, ix->spherical, rel,
+                                                  ix->c_rank_max_norm, total);
+        KSC_LAUNCH_CHECK();
+        KSC_CUDA(cudaMemcpyAsync(&h, total, sizeof(h), cudaMemcpyDeviceToHost, st));
+        KSC_CUDA(cudaStreamSynchronize(st));
+        ix->rank_tc_state = h <= 4 * RW_BEST * RW_SAMPLES ? 1 : -1;
+    }
+    *narrow = ix->rank_tc_state > 0;
     return KSC_OK;
 }
 

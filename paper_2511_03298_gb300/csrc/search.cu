@@ -2780,9 +2780,12 @@ static int list_scores(ksc_index* ix, const float* Q, int64_t nq, int mode, floa
     // rows past TC_SCORES_D: the scores themselves stay FP32 (ksc_list_scores,
     // the predictor's features); a ranking re-scores exactly whatever the
     // scores' bound cannot exclude, so it takes the 16-bit tensor cores there
-    // too (10,000 x 784 against 256 lists: 365 us of FP32 scores and bounds
-    // before, 32 us now)
-    if (mode != RANK_FP32 && (ix->d <= TC_SCORES_D || (preselect && mode == RANK_TC16)))
+    // too where that bound excludes most lists and the rest always fit the
+    // re-score buffer (10,000 x 784 against 256 lists: 365 us of FP32 scores and
+    // bounds before, 32 us now)
+    bool wide_tc = false;
+    if (preselect && mode == RANK_TC16 && ix->d > TC_SCORES_D) KSC_TRY(rank_tc_narrow(ix, &wide_tc, st));
+    if (mode != RANK_FP32 && (ix->d <= TC_SCORES_D || wide_tc))
         return mode == RANK_FP8 ? rank_scores_tc8(ix, Q, nq, scores, *err, st)
                                 : rank_scores_tc(ix, Q, nq, scores, *err, st);
     dim3 grid(blocks_for(ix->L, SC_T), blocks_for(nq, SC_T));
@@ -2820,6 +2823,7 @@ static int select_lists(ksc_index* ix, const float* scores, const float* err, co
                         const int32_t* nprobe_q, int Pfix, int Pmax, int32_t* probes, float* score_out,
                         cudaStream_t st, float* feat) {
     // re-score buffer of the CTA kernel: 4 Pmax lists (a power of two, at least 1024, at most RS_CAP)
+    static_assert(RANK_TC_LISTS <= 1024, "wide rows' 16-bit scores rely on a buffer of every list");
     const int rs_cap = std::min(RS_CAP, std::max(1024, pow2_ceil(4 * Pmax)));
     const size_t smem = rs_cap * sizeof(uint64_t) + (ix->L <= RS_SMEM_L ? sizeof(float) * ix->L : 0);
     KSC_CUDA(cudaFuncSetAttribute(k_rank_select<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
