@@ -154,7 +154,8 @@ typedef struct {
                                   tables' nibbles in FP8, FP32 sums of integers: the same keys as
                                   the byte-permute scan; M <= 128, not with hybrid); 0: chosen by
                                   the queries per list and the lists' lengths (byte permutes when
-                                  lanes_per_query is given) */
+                                  lanes_per_query is given); 2: as 0, also with lanes_per_query
+                                  given */
     int32_t rank_fp8;          /* 1: list scores from FP8-e4m3 operands (queries and centroids
                                   scaled per row by a power of two) on the tensor cores, FP32
                                   accumulate; the lists their error bound cannot exclude are
@@ -267,10 +268,12 @@ int ksc_plan_buffers(ksc_plan* plan, float** Q_dev, int64_t** ids_dev, float** d
 
 void ksc_plan_free(ksc_plan* plan);
 
-/* Autotuner: times the scan's lanes-per-query (8/16/32) and tile length
+/* Autotuner: times the scan's lanes-per-query (4/8/16/32) and tile length
  * (auto, 8, 16, 32, 64 blocks) on the batch Q_dev [nq x d] with the given k,
- * nprobe, rerank and options, and writes the fastest into
- * opts_inout->lanes_per_query / tile_blocks; *best_ms_host (may be NULL)
+ * nprobe, rerank and options, and, where the batch takes the tensor cores by
+ * itself, that scan with each tile length; writes the fastest into
+ * opts_inout->lanes_per_query / tile_blocks (scan_tc 2 where it is the
+ * tensor cores); *best_ms_host (may be NULL)
  * receives its time per search.  Blocking. */
 int ksc_autotune(ksc_index* ix, const float* Q_dev, int64_t nq, int32_t k, int32_t nprobe, int32_t rerank,
                  ksc_search_opts* opts_inout, void* stream, float* best_ms_host);

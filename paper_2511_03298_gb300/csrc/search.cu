@@ -3444,6 +3444,7 @@ static int search_from_probes(ksc_index* ix, const float* Q, const Plan& pl, con
 // 203 / 189 at 32, 793 / 613 at 256; in 2048 lists (100 vectors each): 210 / 232 at
 // 16, 531 / 521 at 64.
 constexpr int64_t TC_MIN_SHARE = 20, TC_MIN_LIST = 256;
+constexpr int SCAN_TC_RULE = 2;  // ksc_search_opts.scan_tc: the rule also where lanes are given
 
 // Tile lengths of the scan's warp items for an expected P probes per query.
 // Short tiles balance the persistent warps, long ones amortise an item's
@@ -3472,8 +3473,8 @@ static void set_tiles(const ksc_index* ix, Plan& pl, int64_t nq, double P, const
     // enough queries share a list; tiles of whole 128-vector products, 32 blocks
     // unless given
     pl.tc = pl.nt > 0 && !pl.hybrid &&
-            (pl.tc_opt || (!(opts && opts->lanes_per_query) && nq * P >= TC_MIN_SHARE * ix->L &&
-                           ix->n >= TC_MIN_LIST * ix->L));
+            (pl.tc_opt || ((!(opts && opts->lanes_per_query) || opts->scan_tc == SCAN_TC_RULE) &&
+                           nq * P >= TC_MIN_SHARE * ix->L && ix->n >= TC_MIN_LIST * ix->L));
     if (pl.tc)
         pl.TB = (opts && opts->tile_blocks > 0) ? (std::min(opts->tile_blocks, TCS_MAX_TILE) + 3) / 4 * 4 : 32;
 }
@@ -3496,7 +3497,7 @@ static int make_plan(ksc_index* ix, int64_t nq, int k, int Pmax, int Rmax, const
     pl.G = choose_G(ix, nq, Pmax, opts ? opts->lanes_per_query : 0);
     pl.nt = tcs_nt(ix->M);
     pl.hybrid = opts && opts->hybrid;
-    pl.tc_opt = opts && opts->scan_tc;
+    pl.tc_opt = opts && opts->scan_tc && opts->scan_tc != SCAN_TC_RULE;
     set_tiles(ix, pl, nq, Pmax, opts);
     int cap = (opts && opts->cand_cap > 0) ? opts->cand_cap : std::max(32 * Rmax, 8192);
     pl.cap = std::max(cap, Rmax);
@@ -4412,12 +4413,22 @@ int ksc_autotune(ksc_index* ix, const float* Q_dev, int64_t nq, int32_t k, int32
     const int TBs[5] = {0, 8, 16, 32, 64};
     ksc_search_opts best = *opts;
     float best_ms = INFINITY;
-    int rc = KSC_OK;
-    for (int gi = 0; gi < 4 && rc == KSC_OK; ++gi) {
-        if (Gs[gi] == 4 ? ix->M > 128 : (ix->M + Gs[gi] - 1) / Gs[gi] > 16) continue;
+    // First what the batch takes by itself, where that is the tensor cores (lanes
+    // alone ask for byte permutes): its own lanes for the first part, and
+    // scan_tc 2, which leaves the scan to the rule.  (10,000 queries of 1M x 64
+    // subspaces at nprobe 7: 718 us, 976 at the best lanes.)
+    ksc_search_opts own = *opts;
+    own.lanes_per_query = own.tile_blocks = 0;
+    Plan pl;
+    int rc = make_plan(ix, nq, k, nprobe, rerank, &own, pl);
+    if (rc == KSC_OK) plan_small(ix, pl, &own, true, true);
+    own.lanes_per_query = pl.G;
+    own.scan_tc = SCAN_TC_RULE;
+    for (int gi = pl.tc && !pl.tc_opt ? -1 : 0; gi < 4 && rc == KSC_OK; ++gi) {
+        if (gi >= 0 && (Gs[gi] == 4 ? ix->M > 128 : (ix->M + Gs[gi] - 1) / Gs[gi] > 16)) continue;
         for (int ti = 0; ti < 5 && rc == KSC_OK; ++ti) {
-            ksc_search_opts o = *opts;
-            o.lanes_per_query = Gs[gi];
+            ksc_search_opts o = gi < 0 ? own : *opts;
+            if (gi >= 0) o.lanes_per_query = Gs[gi];
             o.tile_blocks = TBs[ti];
             float ms = 0.f, tot = 0.f;
             for (int rep = 0; rep < 4 && rc == KSC_OK; ++rep) {
@@ -4441,6 +4452,7 @@ int ksc_autotune(ksc_index* ix, const float* Q_dev, int64_t nq, int32_t k, int32
     if (rc != KSC_OK) return rc;
     opts->lanes_per_query = best.lanes_per_query;
     opts->tile_blocks = best.tile_blocks;
+    opts->scan_tc = best.scan_tc;
     if (best_ms_host) *best_ms_host = best_ms;
     return KSC_OK;
 }

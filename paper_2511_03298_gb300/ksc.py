@@ -179,8 +179,9 @@ def search_opts(lanes_per_query=0, hybrid=False, n_near=2, efs=64, tau=8, cand_c
                 precision=0, rerank_final=0, tile_blocks=0, scan_tc=False, rank_fp8=False, rerank_band=0):
     """precision: 0 FP32 re-rank; 1 BF16 / 2 FP8 first re-rank of the widened
     shortlist, then FP32 over the best rerank_final.  scan_tc: the filtered
-    scan on the tensor cores (same keys) also where it is not the default.  rank_fp8: list scores from FP8 operands
-    (same ranking).  rerank_band: 1 the exact re-rank reads U8 rows (exact,
+    scan on the tensor cores (same keys) also where it is not the default (2:
+    where it is the default, also with lanes_per_query given).  rank_fp8: list
+    scores from FP8 operands (same ranking).  rerank_band: 1 the exact re-rank reads U8 rows (exact,
     when every coordinate is an integer in [0, 255]) or BF16 rows first and
     FP32 rows only where its bound cannot exclude a candidate (same results),
     -1 FP32 rows of every candidate, 0 auto (the band for L2)."""
@@ -516,7 +517,8 @@ class Index:
         return Plan(h.value, self, nq, k)
 
     def autotune(self, Q, k, nprobe, rerank, opts=None, stream=None):
-        """Fastest scan lanes-per-query / tile length for this batch: (opts, ms)."""
+        """Fastest scan lanes-per-query / tile length for this batch, scan_tc 2 where
+        that is the tensor-core scan: (opts, ms)."""
         torch = _torch()
         o = opts if opts is not None else search_opts()
         ms = C.c_float(0)
