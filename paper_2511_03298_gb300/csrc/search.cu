@@ -2690,6 +2690,7 @@ struct Plan {
     int prec, Rf;  // precision variant: first re-rank of R (= Rmax) in prec, then FP32 of the best Rf
     bool band;     // exact re-rank with the band of U8 / BF16 rows (k_rerank_w)
     int Pq_max;    // bound on the per-query nprobe (<= Pmax)
+    double Pexp;   // expected nprobe
     bool tc;       // filtered scan on the tensor cores (k_scan_tc)
     bool tc_opt;   // asked for by the caller
     int nt;        // its queries per item
@@ -3239,14 +3240,29 @@ static int search_small(ksc_index* ix, const float* Q, const Plan& pl, const int
 //  - pairs of a query and a probed list: with many, the general path's shared
 //    lists win (299 queries at up to 144 probes of 758k x 96, 43,000 pairs: 288 us
 //    here, 265 there; 158 at up to 199, 31,000 pairs: 205 here, 234 there).
+//  - sharing: the general path reads a list's codes and builds its selectors once
+//    for several queries, the small one for each.  Where more than two queries
+//    share a list (one, past 256 queries), it is taken only up to SMALL_SHARED_NQ
+//    queries and SMALL_LOOKUPS table lookups, fewer the more queries there are
+//    (SMALL_NQ_LOOKUPS over their number).  Here / there in us, 1M x 64 subspaces in 1024
+//    lists: 303 queries at nprobe 16 259 / 212, at 4 162 / 169; 200 at 16 206 /
+//    188, at 8 158 / 170; 150 at 32 213 / 191, at 16 163 / 170; 64 at 256 382 /
+//    331, at 64 164 / 194; 303 on 10k x 64 in 64 lists at 16 174 / 144; 250 on 1M x
+//    48 in 4096 lists at 64 201 / 204, at 16 136 / 154; 303 there at 64 226 / 212.
 constexpr int64_t SMALL_MAX_PAIRS = 40000;
 constexpr int64_t SMALL_RANK_BYTES = 64 << 20;
 constexpr int64_t SMALL_NEAR_KEYS = 32768;
 constexpr int64_t SMALL_MAX_RECS = 1 << 22;
+constexpr int64_t SMALL_SHARED_NQ = 200;
+constexpr double SMALL_LOOKUPS = 450e6, SMALL_NQ_LOOKUPS = 36e9;
 static void plan_small(const ksc_index* ix, Plan& pl, const ksc_search_opts* opts, bool distinct, bool can_rank) {
     const int64_t nq = pl.nq, P = pl.Pmax;
     if (nq == 0 || nq >= 2 * (int64_t)num_sms() || pl.hybrid || pl.tc_opt || (pl.G != 8 && pl.G != 16) || P > SP_MAX_P ||
         nq * P > SMALL_MAX_PAIRS || P * ix->max_list >= (1ll << 31))
+        return;
+    const double share = (double)nq * pl.Pexp / ix->L, lookups = share * (double)ix->n * ix->M;
+    if (share > (nq > 256 ? 1.0 : 2.0) &&
+        (nq > SMALL_SHARED_NQ || lookups > SMALL_LOOKUPS || nq * lookups > SMALL_NQ_LOOKUPS))
         return;
     const int64_t maxb = (ix->max_list + 31) / 32;
     const int64_t blocks = distinct ? ix->h_top_blocks[P] : P * maxb;
@@ -3454,6 +3470,7 @@ constexpr int SCAN_TC_RULE = 2;  // ksc_search_opts.scan_tc: the rule also where
 // 4 to 32 blocks (on the 1M x 128 workload at nprobe 7: tiles of 14 and 6
 // blocks; filtered tiles of 12 to 17 blocks ran within 1% of each other).
 static void set_tiles(const ksc_index* ix, Plan& pl, int64_t nq, double P, const ksc_search_opts* opts) {
+    pl.Pexp = P;
     const int QG = 32 / pl.G;
     const double nbar = (double)ix->n / ix->L;
     const double blocks = std::ceil((double)nq * P / ix->L / QG) * ix->nblocks;
