@@ -57,20 +57,24 @@ __device__ __forceinline__ float rerank_rows8(const float4& qv, const float* __r
 }
 
 
-constexpr int RR_RANK_R = 512;  // candidates up to which the k best are found by counting ranks
+constexpr int RR_RANK_R = 512;  // keys up to which an order is found by counting ranks
 
-// Shared bytes of cta_rerank's keys: R of them and, past RR_RANK_R, k more.
-inline size_t rerank_smem(int R, int k) { return sizeof(uint64_t) * ((size_t)R + (R > RR_RANK_R ? k : 0)); }
+// Keys of cta_rerank's kbuf: the k best, to a power of two where they are sorted.
+__host__ __device__ inline int rerank_kbuf(int k) { return k > RR_RANK_R ? pow2_ceil(k) : k; }
+// Shared bytes of cta_rerank's keys: R of them and, past RR_RANK_R, its kbuf.
+inline size_t rerank_smem(int R, int k) {
+    return sizeof(uint64_t) * ((size_t)R + (R > RR_RANK_R ? rerank_kbuf(k) : 0));
+}
 
 // Exact distance of each of the R candidates keys[] (KEY_NONE: none) of one
 // query (qs, shared memory), by one CTA: L2 = sum (q_t - x_t)^2, IP = -<q, x>,
 // a warp per row, 16-byte loads when d is a multiple of 4; then the k best by
 // (distance, id) to out_ids / out_d (L2 distance ascending / IP similarity
-// descending).  keys[] is overwritten; kbuf: k keys when R > RR_RANK_R.
+// descending).  keys[] is overwritten; kbuf: rerank_kbuf(k) keys when R > RR_RANK_R.
 // Bound by the rows' latency: a warp keeps 8 rows (d <= 128) or 4 in flight;
 // up to 512 candidates are ordered by counting, for each, the smaller ones
 // (one pass of broadcast reads, no barriers), more are cut to the k best by
-// radix refinement first.
+// radix refinement first, and these sorted if they are more than 512 still.
 template <int NT>
 __device__ __forceinline__ void cta_rerank(uint64_t* keys, int R, uint64_t* kbuf, const float* qs,
                                            const float* __restrict__ X, int d, int ip, int k,
@@ -198,7 +202,15 @@ __device__ __forceinline__ void cta_rerank(uint64_t* keys, int R, uint64_t* kbuf
             for (int i = threadIdx.x; i < R; i += NT) kbuf[i] = keys[i];
         }
         __syncthreads();
-        for (int i = threadIdx.x; i < kr; i += NT) {
+        if (kr > RR_RANK_R) {
+            // counting costs kr^2 reads: more keys are sorted (10,000 queries, k = R
+            // 1000: the search 5547 us counted, 3010 sorted; 1000 queries 754 and 499)
+            const int S = pow2_ceil(kr);
+            for (int i = kr + threadIdx.x; i < S; i += NT) kbuf[i] = KEY_NONE;
+            __syncthreads();
+            block_bitonic_sort(kbuf, S);
+            for (int i = threadIdx.x; i < kr; i += NT) put(i, kbuf[i]);
+        } else for (int i = threadIdx.x; i < kr; i += NT) {
             const uint64_t v = kbuf[i];
             int rank = 0;
 #pragma unroll 8

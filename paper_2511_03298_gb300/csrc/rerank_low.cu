@@ -5,6 +5,8 @@
 // Both read a row with 8 lanes, 16 bytes (U8) or 8 / 4 bytes (BF16 / FP8) per
 // lane and step, 4 rows per lane group and 16 per warp in flight, and reduce 16
 // rows with 7 shuffles.
+#include <algorithm>
+
 #include "rerank.cuh"
 #include "rerank_low.cuh"
 #include "scan.cuh"
@@ -155,13 +157,13 @@ __global__ void __launch_bounds__(RL_T) k_rerank_u8(const float* __restrict__ Q,
                                                     const uint64_t* __restrict__ topr, int Rmax,
                                                     const int32_t* __restrict__ rerank_q, int Rfix, int k,
                                                     int64_t* __restrict__ out_ids, float* __restrict__ out_d) {
-    // Rmax keys, Rmax survivors' keys (first: bounds), k keys past RR_RANK_R
+    // Rmax keys (later the re-rank's kbuf: rerank_kbuf(k)), Rmax survivors' keys (first: bounds)
     extern __shared__ uint64_t keys[];
     __shared__ __align__(16) float qs[KSC_MAX_DIM];
     __shared__ __align__(16) uint32_t hist[256];
     __shared__ uint64_t bb[32];
     __shared__ int s_n;
-    uint64_t* live = keys + Rmax;
+    uint64_t* live = keys + max(Rmax, rerank_kbuf(k));
     float* dist = reinterpret_cast<float*>(live);  // [Rmax] the U8 pass's distances, read before live is written
     const int64_t q = blockIdx.x;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, j = lane & 7;
@@ -261,7 +263,7 @@ __global__ void __launch_bounds__(RL_T) k_rerank_u8(const float* __restrict__ Q,
 
 int launch_rerank_u8(const float* Q, int64_t nq, const float* X, const uint8_t* xu, int d, const uint64_t* topr,
                      int Rmax, const int32_t* rerank_q, int Rfix, int k, int64_t* ids, float* dists, cudaStream_t st) {
-    const size_t smem = sizeof(uint64_t) * 2 * (size_t)Rmax;
+    const size_t smem = sizeof(uint64_t) * ((size_t)std::max(Rmax, rerank_kbuf(k)) + Rmax);
     KSC_CUDA(cudaFuncSetAttribute(k_rerank_u8, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     k_rerank_u8<<<(unsigned)nq, RL_T, smem, st>>>(Q, X, xu, d, topr, Rmax, rerank_q, Rfix, k, ids, dists);
     KSC_LAUNCH_CHECK();

@@ -2255,7 +2255,7 @@ __global__ void __launch_bounds__(NT) k_rerank(const float* __restrict__ Q, cons
                                                 int ip, const uint64_t* __restrict__ topr, int Rmax,
                                                 const int32_t* __restrict__ rerank_q, int Rfix, int k,
                                                 int64_t* __restrict__ out_ids, float* __restrict__ out_d) {
-    extern __shared__ uint64_t keys[];  // Rmax keys, then KSC_MAX_K for the selection of more than RR_RANK_R
+    extern __shared__ uint64_t keys[];  // Rmax keys, then rerank_kbuf(k) for the selection of more than RR_RANK_R
     __shared__ __align__(16) float qs[KSC_MAX_DIM];
     const int64_t q = blockIdx.x;
     const int R = rerank_of(rerank_q, Rfix, k, Rmax, q);

@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(NT) k_select_rerank(ScanArgs A, int Rmax, cons
                                                       int64_t* __restrict__ out_ids, float* __restrict__ out_d,
                                                       int32_t* __restrict__ status,
                                                       unsigned long long* __restrict__ stats) {
-    extern __shared__ uint64_t sr_keys[];  // nkeys (at least Rmax; sel_cap when a store may overflow), then k
+    extern __shared__ uint64_t sr_keys[];  // nkeys (at least Rmax; sel_cap when a store may overflow), then rerank_kbuf(k)
     __shared__ __align__(16) uint32_t hist[256];
     __shared__ uint64_t bb[32];
     __shared__ __align__(16) float qs[KSC_MAX_DIM];
@@ -394,7 +394,7 @@ int launch_select_rerank(const ScanArgs& A, int Rmax, const int32_t* cnt, uint64
                          const float* Q, const float* X, int d, int ip, int k, int64_t* ids, float* dists,
                          int32_t* status, unsigned long long* stats, cudaStream_t st) {
     const int nkeys = Rmax > sel_cap ? Rmax : sel_cap;
-    const size_t smem = sizeof(uint64_t) * ((size_t)nkeys + (Rmax > RR_RANK_R ? k : 0));
+    const size_t smem = sizeof(uint64_t) * ((size_t)nkeys + (Rmax > RR_RANK_R ? rerank_kbuf(k) : 0));
     KSC_CUDA(cudaFuncSetAttribute(k_select_rerank<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     k_select_rerank<1024><<<(unsigned)A.nq, 1024, smem, st>>>(A, Rmax, cnt, cand, cap, nkeys, sel_cap, Q, X, d, ip, k,
                                                               ids, dists, status, stats);
