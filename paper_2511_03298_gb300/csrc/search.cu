@@ -4114,7 +4114,7 @@ int ksc_train_predictor(ksc_index* ix, const float* Qtrain_dev, int64_t nt, cons
     const int target = (opts && opts->target_hits > 0) ? opts->target_hits : 9;
     const int R_lab = (opts && opts->rerank_label > 0) ? opts->rerank_label : 200;
     const int epochs = (opts && opts->epochs > 0) ? opts->epochs : 8;
-    const int batch = (opts && opts->batch > 0) ? opts->batch : 256;
+    const int batch = (int)std::min<int64_t>((opts && opts->batch > 0) ? opts->batch : 256, nt);
     const float lr = (opts && opts->lr > 0.f) ? opts->lr : 1e-3f;
     uint64_t seed = (opts && opts->seed) ? opts->seed : 0x6d6c70ull;
     const bool regression = opts && opts->regression;
@@ -4591,7 +4591,7 @@ int ksc_train_pruner(ksc_index* ix, const float* Qtrain_dev, int64_t nt, const f
     cudaStream_t st = as_stream(stream);
     if (!ix->pr_have_stats) KSC_TRY(prune_stats(ix, 30, st));
     const int epochs = (opts && opts->epochs > 0) ? opts->epochs : 4;
-    const int batch = (opts && opts->batch > 0) ? opts->batch : 1024;
+    const int batch = (int)std::min<int64_t>((opts && opts->batch > 0) ? opts->batch : 1024, nt * P);
     const float lr = (opts && opts->lr > 0.f) ? opts->lr : 1e-3f;
     uint64_t seed = (opts && opts->seed) ? opts->seed : 0x707275ull;
     const int64_t chunk = 8192, rows = nt * P;
