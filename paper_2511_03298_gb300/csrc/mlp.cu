@@ -173,6 +173,24 @@ __device__ __forceinline__ void adam_update(const AdamArgs& A, int i, float gi) 
     A.w[i] -= A.lr * (mi / A.bc1) / (sqrtf(vi / A.bc2) + A.eps);
 }
 
+template <int F, int H>
+static size_t grad_smem() {
+    return sizeof(float) * (mlp_nparam<F, H>() + MLP_TILE * (F + 3 * H + MLP_O));
+}
+
+template <int F, int H>
+static int mlp_grad_t(const float* w, const float* x, const float* y, int64_t B, float* grad, float* loss,
+                      cudaStream_t st) {
+    KSC_CUDA(cudaMemsetAsync(grad, 0, sizeof(float) * mlp_nparam<F, H>(), st));
+    if (loss) KSC_CUDA(cudaMemsetAsync(loss, 0, sizeof(float), st));
+    KSC_CUDA(cudaFuncSetAttribute(k_mlp_grad<F, H>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)grad_smem<F, H>()));
+    k_mlp_grad<F, H><<<(unsigned)((B + MLP_TILE - 1) / MLP_TILE), 256, grad_smem<F, H>(), st>>>(w, x, y, B, grad,
+                                                                                              loss);
+    KSC_LAUNCH_CHECK();
+    return KSC_OK;
+}
+
 // ------------------------------------------------------------------ one training step over the whole chip
 // k_mlp_grad gives each 128 samples one CTA, so a 256-sample step runs on two
 // SMs and walks its dependent products there (213 us a step).  A step is
@@ -347,10 +365,36 @@ static AdamArgs adam_args(float* w, float* m, float* v, int t, float lr) {
     return AdamArgs{w, m, v, lr, b1, b2, 1e-8f, 1.f - powf(b1, (float)t), 1.f - powf(b2, (float)t)};
 }
 
+__global__ void k_adam(const float* __restrict__ g, int n, AdamArgs A) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) adam_update(A, i, g[i]);
+}
+
+// Samples of a step up to which it is spread as above: k_train_grads walks them
+// in its few CTAs (a pair of tiles, 256 samples, at a time), k_mlp_grad gives
+// every tile a CTA of its own.  Past it the step is gathered and taken by
+// k_mlp_grad and k_adam.  A step in us, spread / gathered: 64 x 64 x 64
+// weights 18 / 224 at 256 samples, 240 / 275 at 8192, 394 / 314 at 16,384; 16 x
+// 32 x 32 18 / 62 at 256, 73 / 74 at 2048, 137 / 88 at 4096.
+template <int F, int H>
+static constexpr int64_t train_spread() {
+    return F * H > 2048 ? 8192 : 2048;
+}
+
 template <int F, int H>
 static int train_step_t(float* w, float* m, float* v, const float* feats, const float* Y, const int64_t* idx,
                         int64_t nb, int64_t batch, float* act, float* loss, int t, float lr, cudaStream_t st) {
     static_assert(F % 4 == 0 && 256 % H == 0 && 256 % F == 0 && H * F % 256 == 0 && H * H % 256 == 0, "layer sizes");
+    if (batch > train_spread<F, H>()) {
+        constexpr int NP = mlp_nparam<F, H>();
+        float *xb = act, *yb = xb + batch * F, *g = yb + batch * MLP_O;
+        k_gather_rows<<<(unsigned)((nb * F + 255) / 256), 256, 0, st>>>(feats, idx, nb, F, xb);
+        k_gather_rows<<<(unsigned)((nb * MLP_O + 255) / 256), 256, 0, st>>>(Y, idx, nb, MLP_O, yb);
+        KSC_TRY((mlp_grad_t<F, H>(w, xb, yb, nb, g, loss, st)));
+        k_adam<<<(NP + 255) / 256, 256, 0, st>>>(g, NP, adam_args(w, m, v, t, lr));
+        KSC_LAUNCH_CHECK();
+        return KSC_OK;
+    }
     const TrainAct ta = train_act<F, H>(act, batch);
     k_train_rows<F, H><<<(unsigned)((nb + 256 / H - 1) / (256 / H)), 256, 0, st>>>(w, feats, Y, idx, nb, ta, loss);
     constexpr int MAXF = F > H ? F : H, MINF = F < H ? F : H;
@@ -361,8 +405,14 @@ static int train_step_t(float* w, float* m, float* v, const float* feats, const 
     return KSC_OK;
 }
 
-size_t mlp_train_act(int64_t batch) { return (size_t)batch * (MLP_F + 4 * MLP_H + MLP_O); }
-size_t prune_train_act(int64_t batch) { return (size_t)batch * (KSC_PRUNE_FEATURES + 4 * 32 + MLP_O); }
+template <int F, int H>
+static size_t train_act_t(int64_t batch) {
+    return batch > train_spread<F, H>() ? (size_t)batch * (F + MLP_O) + mlp_nparam<F, H>()
+                                        : (size_t)batch * (F + 4 * H + MLP_O);
+}
+
+size_t mlp_train_act(int64_t batch) { return train_act_t<MLP_F, MLP_H>(batch); }
+size_t prune_train_act(int64_t batch) { return train_act_t<KSC_PRUNE_FEATURES, 32>(batch); }
 
 int mlp_train_step(float* w, float* m, float* v, const float* feats, const float* Y, const int64_t* idx, int64_t nb,
                    int64_t batch, float* act, float* loss, int t, float lr, cudaStream_t st) {
@@ -602,24 +652,7 @@ __global__ void k_hits(const float* __restrict__ dists, int64_t nq, int k, const
     hits[q] = h;
 }
 
-template <int F, int H>
-static size_t grad_smem() {
-    return sizeof(float) * (mlp_nparam<F, H>() + MLP_TILE * (F + 3 * H + MLP_O));
-}
 static size_t infer_smem() { return sizeof(float) * (MLP_NPARAM + 3 * MLP_ITILE * MLP_LDI); }
-
-template <int F, int H>
-static int mlp_grad_t(const float* w, const float* x, const float* y, int64_t B, float* grad, float* loss,
-                      cudaStream_t st) {
-    KSC_CUDA(cudaMemsetAsync(grad, 0, sizeof(float) * mlp_nparam<F, H>(), st));
-    if (loss) KSC_CUDA(cudaMemsetAsync(loss, 0, sizeof(float), st));
-    KSC_CUDA(cudaFuncSetAttribute(k_mlp_grad<F, H>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)grad_smem<F, H>()));
-    k_mlp_grad<F, H><<<(unsigned)((B + MLP_TILE - 1) / MLP_TILE), 256, grad_smem<F, H>(), st>>>(w, x, y, B, grad,
-                                                                                              loss);
-    KSC_LAUNCH_CHECK();
-    return KSC_OK;
-}
 
 int mlp_grad(const float* w, const float* x, const float* y, int64_t B, float* grad, float* loss, cudaStream_t st) {
     return mlp_grad_t<MLP_F, MLP_H>(w, x, y, B, grad, loss, st);
