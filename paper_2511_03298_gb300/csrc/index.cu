@@ -687,6 +687,18 @@ static int assign_rows(AssignTc& T, int32_t* assign, cudaStream_t st) {
     return KSC_OK;
 }
 
+// Whether the tensor cores pay off for a build's assignments (iters rounds of
+// ns rows and one of n).  They score 256 centroids whatever L, from FP16 copies
+// of the rows, in four launches; the FP32 kernel scores 64 at a time from the
+// rows themselves.  Builds of 10 rounds in ms, FP32 / tensor cores: 20,000 x 128
+// in 64 lists 2.0 / 2.3, in 192 2.6 / 2.4, in 256 2.9 / 2.5; 20,000 x 64 in 256
+// (0.33 G multiply-adds a round) 2.1 / 2.1; 200,000 x 16 in 256 (0.32) 3.7 / 3.9;
+// 1M x 128 in 64 14.8 / 16.0, in 128 15.4 / 16.0, in 192 17.0 / 15.8; 20,000 x 512 in
+// 64 3.3 / 3.5, in 96 4.4 / 3.6.
+static bool assign_tc_pays(int64_t n, int64_t ns, int d, int L, int iters) {
+    return (L > 128 || (L > 64 && d >= 256)) && ((double)iters * ns + n) * L * d >= 0.35e9 * (iters + 1);
+}
+
 // Rows per pass of the final assignment (bounds the FP16 copy).
 constexpr int64_t ASSIGN_CHUNK = 1 << 20;
 
@@ -1042,8 +1054,9 @@ int ksc_build_index(const float* X_dev, int64_t n, int32_t d, int32_t nlist, int
         B_CUDA(cudaMalloc(&ix->c_rank_sq, sizeof(float) * nlist));
         // 1. coarse quantiser
         float xmax = 0.f;
-        if ((rc = max_abs(ix->X, n * d, &xmax, st))) break;
-        const bool tc = assign_tc_supported(xmax);
+        bool tc = assign_tc_pays(n, ns, d, nlist, iters);
+        if (tc && (rc = max_abs(ix->X, n * d, &xmax, st))) break;
+        tc = tc && assign_tc_supported(xmax);
         if (tc && (rc = T.init(std::max(ns, std::min(n, ASSIGN_CHUNK)), d, nlist, xmax, st))) break;
         if ((rc = lloyd(ix->X, perm_dev, ns, d, nlist, iters, ix->c_mean, tc ? &T : nullptr, xmax, st))) break;
         B_CUDA(cudaMemcpyAsync(ix->c_rank, ix->c_mean, sizeof(float) * nlist * d, cudaMemcpyDeviceToDevice, st));
