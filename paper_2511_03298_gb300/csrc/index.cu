@@ -1057,13 +1057,24 @@ int ksc_build_index(const float* X_dev, int64_t n, int32_t d, int32_t nlist, int
         bool tc = assign_tc_pays(n, ns, d, nlist, iters);
         if (tc && (rc = max_abs(ix->X, n * d, &xmax, st))) break;
         tc = tc && assign_tc_supported(xmax);
-        if (tc && (rc = T.init(std::max(ns, std::min(n, ASSIGN_CHUNK)), d, nlist, xmax, st))) break;
-        if ((rc = lloyd(ix->X, perm_dev, ns, d, nlist, iters, ix->c_mean, tc ? &T : nullptr, xmax, st))) break;
+        // list of every row, and then the operands: where the device has no room for
+        // them, or for the k-means beside them, the FP32 kernel needs neither
+        B_CUDA(cudaMalloc(&ix->assign, sizeof(int32_t) * n));
+        if (tc) {
+            rc = T.init(std::max(ns, std::min(n, ASSIGN_CHUNK)), d, nlist, xmax, st);
+            if (rc == KSC_OK) rc = lloyd(ix->X, perm_dev, ns, d, nlist, iters, ix->c_mean, &T, xmax, st);
+            if (rc == KSC_ETIMEOUT) break;
+            if (rc != KSC_OK) {
+                cudaGetLastError();
+                T.free();
+                tc = false;
+            }
+        }
+        if (!tc && (rc = lloyd(ix->X, perm_dev, ns, d, nlist, iters, ix->c_mean, nullptr, 0.f, st))) break;
         B_CUDA(cudaMemcpyAsync(ix->c_rank, ix->c_mean, sizeof(float) * nlist * d, cudaMemcpyDeviceToDevice, st));
         if (spherical) k_normalise_rows<<<(nlist + 255) / 256, 256, 0, st>>>(ix->c_rank, nlist, d);
         k_row_sqnorm<<<(nlist + 255) / 256, 256, 0, st>>>(ix->c_rank, nlist, d, ix->c_rank_sq);
         // 2. list of every vector by the ranking score
-        B_CUDA(cudaMalloc(&ix->assign, sizeof(int32_t) * n));
         if (tc) {
             rc = T.set_centroids(ix->c_rank, nullptr, nullptr, spherical, spherical ? 1.f : xmax, st);
             for (int64_t r0 = 0; r0 < n && rc == KSC_OK; r0 += ASSIGN_CHUNK) {
@@ -1073,6 +1084,7 @@ int ksc_build_index(const float* X_dev, int64_t n, int32_t d, int32_t nlist, int
             }
             if (rc == KSC_OK) rc = T.check(st);  // before anything indexes with the lists
             if (rc) break;
+            T.free();
         } else {
             k_assign<<<(unsigned)((n + AS_T - 1) / AS_T), 256, 0, st>>>(ix->X, n, d, ix->c_rank, ix->c_rank_sq, nlist,
                                                                         spherical, ix->assign, nullptr, nullptr, 0);
