@@ -2938,10 +2938,19 @@ static int ensure_u8(ksc_index* ix, cudaStream_t st) {
     return KSC_OK;
 }
 
-// Whether U8 copies of the re-rank rows are there, made now if they can be: not
-// while the stream is captured, nor (for good) once the device had no room.
-static bool u8_rows(ksc_index* ix, cudaStream_t st) {
+// Whether U8 copies of the re-rank rows are there for a re-rank of `rows`
+// candidates.  Making them (a pass over the rows, their check and copy, n d bytes
+// of memory, a synchronisation) costs about what re-ranking 19 candidates per
+// row of the index in bytes saves (60k x 784: 450 us; 10,000 queries of 200
+// candidates 848 -> 477 us), so they are made once the handle has re-ranked
+// U8_AFTER per row, at once for a plan: a program that searches an index a few
+// times does not pay for them.  Not while the stream is captured, nor (for
+// good) once the device had no room.
+constexpr int64_t U8_AFTER = 16;
+static bool u8_rows(ksc_index* ix, int64_t rows, cudaStream_t st) {
     if (ix->x_u8_state == 0) {
+        ix->u8_wanted += rows;
+        if (!ix->u8_now && ix->u8_wanted < U8_AFTER * ix->n) return false;
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
         if (ensure_u8(ix, st) != KSC_OK) {
@@ -3079,7 +3088,7 @@ static int rerank_stage(ksc_index* ix, const float* Qr, const Plan& pl, const ui
         ix->launches++;
         KSC_LAUNCH_CHECK();
     } else if (pl.band && pl.prec == 0 && rr_R > pl.k && ix->metric != KSC_IP && nq >= 2 * (int64_t)num_sms() &&
-               rerank_u8_supported(dr) && u8_rows(ix, st)) {
+               rerank_u8_supported(dr) && u8_rows(ix, nq * rr_R, st)) {
         KSC_TRY(launch_rerank_u8(Qr, nq, Xr, (const uint8_t*)ix->X_u8, dr, rr_keys, rr_R, rr_q, rr_R, pl.k, ids, dists,
                                  st));
         ix->launches++;
@@ -4311,7 +4320,9 @@ static int plan_capture(ksc_plan* pl, cudaStream_t st) {
     if (pl->graph) { cudaGraphDestroy(pl->graph); pl->graph = nullptr; }
     const bool prof = pl->ix->prof;
     pl->ix->prof = false;
+    pl->ix->u8_now = true;
     int rc = plan_search(pl, st);
+    pl->ix->u8_now = false;
     if (rc == KSC_OK) {
         cudaError_t e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) { set_error("warm-up failed: %s", cudaGetErrorString(e)); rc = KSC_ECUDA; }
