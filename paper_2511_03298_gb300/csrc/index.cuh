@@ -43,7 +43,7 @@ struct ksc_index {
     void* X_fp8 = nullptr;         // [n x d] FP8 e4m3 rows
     float* X_scale = nullptr;      // [n] their per-row scales
     void* X_u8 = nullptr;          // [n x d] U8 rows when every coordinate is an integer in [0, 255] (exact)
-    int x_u8_state = 0;            // 0 not checked, 1 X_u8 holds the rows exactly, -1 they do not fit bytes
+    int x_u8_state = 0;            // 0 not checked, 1 X_u8 holds the rows exactly, -1 they do not fit bytes, 2 they do, no copy yet
     int64_t u8_wanted = 0;         // candidate rows re-ranked so far that U8 rows would have served (u8_rows)
     bool u8_now = false;           // make the copies with the next search (a plan is being made)
     int rank_tc_state = 0;         // rank_tc_narrow: 0 not checked, 1 narrow, -1 wide

@@ -2927,13 +2927,14 @@ static int ensure_u8(ksc_index* ix, cudaStream_t st) {
         int32_t h = 0;
         KSC_CUDA(cudaMemcpyAsync(&h, ok, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
         KSC_CUDA(cudaStreamSynchronize(st));
-        if (h && m > 0 && !ix->X_u8) {
-            KSC_CUDA(cudaMalloc(&ix->X_u8, (size_t)m));
-            k_x_u8<<<(unsigned)std::min<int64_t>((m + 255) / 256, 8 * (int64_t)num_sms()), 256, 0, st>>>(
-                rr_X(ix), m, (uint8_t*)ix->X_u8);
-            KSC_LAUNCH_CHECK();
-        }
-        ix->x_u8_state = (h && m > 0) ? 1 : -1;  // only once the copy exists
+        ix->x_u8_state = (h && m > 0) ? 2 : -1;
+    }
+    if (ix->x_u8_state == 2) {
+        if (!ix->X_u8) KSC_CUDA(cudaMalloc(&ix->X_u8, (size_t)m));
+        k_x_u8<<<(unsigned)std::min<int64_t>((m + 255) / 256, 8 * (int64_t)num_sms()), 256, 0, st>>>(
+            rr_X(ix), m, (uint8_t*)ix->X_u8);
+        KSC_LAUNCH_CHECK();
+        ix->x_u8_state = 1;  // only once the copy exists
     }
     return KSC_OK;
 }
@@ -2944,18 +2945,18 @@ static int ensure_u8(ksc_index* ix, cudaStream_t st) {
 // row of the index in bytes saves (60k x 784: 450 us; 10,000 queries of 200
 // candidates 848 -> 477 us), so they are made once the handle has re-ranked
 // U8_AFTER per row, at once for a plan: a program that searches an index a few
-// times does not pay for them.  Not while the stream is captured, nor (for
-// good) once the device had no room.
+// times does not pay for them.  Not while the stream is captured; where the
+// device has no room, tried again after as many candidates more.
 constexpr int64_t U8_AFTER = 16;
 static bool u8_rows(ksc_index* ix, int64_t rows, cudaStream_t st) {
-    if (ix->x_u8_state == 0) {
+    if (ix->x_u8_state == 0 || ix->x_u8_state == 2) {
         ix->u8_wanted += rows;
         if (!ix->u8_now && ix->u8_wanted < U8_AFTER * ix->n) return false;
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
         if (ensure_u8(ix, st) != KSC_OK) {
             cudaGetLastError();
-            ix->x_u8_state = -1;
+            ix->u8_wanted = 0;
         }
     }
     return ix->x_u8_state == 1;

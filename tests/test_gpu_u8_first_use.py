@@ -1,7 +1,10 @@
 """When the exact re-rank's U8 copies are made: not by the first searches of an
 index, whose saving would not pay for them, but once a handle has re-ranked 16
 candidates per row, and by a plan's creation (told by the device memory taken:
-102 MB of copies); the results are those of the FP32 rows throughout."""
+102 MB of copies); the results are those of the FP32 rows throughout.  Where the
+device has no room for them the search goes on without, and they are made later."""
+import ctypes as C
+
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -60,3 +63,36 @@ def test_made_for_a_plan(env):
     st.synchronize()
     assert taken > 90 * MB
     assert torch.equal(got[0], ref[0]) and torch.equal(got[1], ref[1])
+
+
+def test_made_later_where_there_was_no_room(env):
+    torch, ksc, ix, Q = env
+    v = ix.view()
+    ref = v.search(Q, 10, 4, 400, opts=ksc.search_opts(rerank_band=-1))
+    v.search(Q, 10, 4, 400)
+    rt = C.CDLL("libcudart.so.13")
+    rt.cudaMalloc.argtypes, rt.cudaFree.argtypes = [C.POINTER(C.c_void_p), C.c_size_t], [C.c_void_p]
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    out = torch.empty((4096, 10), dtype=torch.int64, device="cuda"), torch.empty((4096, 10), device="cuda")
+    held = []
+    try:
+        for size in (8 << 30, 512 * MB, 16 * MB):
+            while torch.cuda.mem_get_info()[0] >= 60 * MB + size:
+                p = C.c_void_p()
+                if rt.cudaMalloc(C.byref(p), size):
+                    break
+                held.append(p)
+        for _ in range(2):  # the copies are due, and 102 MB are not to be had
+            v.search(Q, 10, 4, 400, out=out)
+            torch.cuda.synchronize()
+    finally:
+        for p in held:
+            assert rt.cudaFree(p) == 0
+    assert torch.equal(out[0], ref[0]) and torch.equal(out[1], ref[1])
+    made = 0
+    for _ in range(3):
+        got, taken = _taken(torch, lambda: v.search(Q, 10, 4, 400))
+        made += taken > 90 * MB
+        assert torch.equal(got[0], ref[0]) and torch.equal(got[1], ref[1])
+    assert made == 1
