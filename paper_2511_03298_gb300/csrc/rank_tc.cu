@@ -306,13 +306,19 @@ static int err_params(ksc_index* ix, bool tensor_cores, float* rel, float* qmax,
 int rank_scores_tc(ksc_index* ix, const float* Q, int64_t nq, float* scores, float* err, cudaStream_t st) {
     const int Kp = (ix->d + TC_KB - 1) / TC_KB * TC_KB;
     const int KB = Kp / TC_KB;
+    float rel, qmax;
     if (!ix->c_rank_bf16) {
-        // operand type: FP16 (11-bit significand) when the centroids fit it
-        std::vector<float> ch((size_t)ix->L * ix->d);
-        KSC_CUDA(cudaMemcpy(ch.data(), ix->c_rank, sizeof(float) * ch.size(), cudaMemcpyDeviceToHost));
-        float mx = 0.f;
-        for (float v : ch) mx = fmaxf(mx, fabsf(v));
-        ix->tc_fp16 = mx < 16384.f;
+        // operand type: FP16 (11-bit significand) when the centroids fit it, which
+        // the largest norm mostly shows (else from the coordinates, on the host)
+        KSC_TRY(err_params(ix, true, &rel, &qmax, st));
+        ix->tc_fp16 = ix->c_rank_max_norm < 16384.f;
+        if (!ix->tc_fp16) {
+            std::vector<float> ch((size_t)ix->L * ix->d);
+            KSC_CUDA(cudaMemcpy(ch.data(), ix->c_rank, sizeof(float) * ch.size(), cudaMemcpyDeviceToHost));
+            float mx = 0.f;
+            for (float v : ch) mx = fmaxf(mx, fabsf(v));
+            ix->tc_fp16 = mx < 16384.f;
+        }
         KSC_CUDA(cudaMalloc(&ix->c_rank_bf16, sizeof(uint16_t) * (size_t)ix->L * Kp));
         k_to_16<<<(unsigned)std::min<int64_t>(((int64_t)ix->L * Kp + 255) / 256, 4096), 256, 0, st>>>(
             ix->c_rank, ix->L, ix->d, Kp, ix->tc_fp16, (uint16_t*)ix->c_rank_bf16);
@@ -321,7 +327,6 @@ int rank_scores_tc(ksc_index* ix, const float* Q, int64_t nq, float* scores, flo
     }
     KSC_TRY(ensure(ix->ws_qbf16, sizeof(uint16_t) * (size_t)nq * Kp, st));
     uint16_t* qb = (uint16_t*)ix->ws_qbf16.p;
-    float rel, qmax;
     KSC_TRY(err_params(ix, true, &rel, &qmax, st));
     k_q16_err<<<(unsigned)((nq + 7) / 8), 256, 0, st>>>(Q, nq, ix->d, Kp, ix->tc_fp16, ix->c_rank_max_norm,
                                                          ix->spherical, rel, qmax, qb, err);

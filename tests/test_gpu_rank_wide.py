@@ -31,3 +31,21 @@ def test_wide_rows_ranked_exactly(d, L, offset):
     probes, scores = ix.rank_lists(torch.from_numpy(Q).cuda(), P)
     np.testing.assert_array_equal(probes.cpu().numpy(), want)
     np.testing.assert_array_equal(scores.cpu().numpy(), (np.take_along_axis(D, want, 1) / 256).astype(np.float32))
+
+
+@pytest.mark.parametrize("scale", [1, 1000, 4000, 8000])
+def test_operand_types(scale):
+    """Centroids whose norms, or coordinates, pass what the FP16 operands take."""
+    import torch
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2511_03298_gb300 import ksc
+    rng = np.random.default_rng(scale)
+    C = (scale * rng.integers(-3, 4, size=(300, 64))).astype(np.float32)
+    Q = (scale * rng.integers(-3, 4, size=(400, 64))).astype(np.float32)
+    ix = ksc.index_import(dict(X=C, c_rank=C, c_mean=C, codebook=np.zeros((16, 16, 4), np.float32),
+                               codes=np.zeros((300, 16), np.uint8), assign=np.arange(300, dtype=np.int32)))
+    q, c = Q.astype(np.float64) / scale, C.astype(np.float64) / scale
+    D = (q * q).sum(1)[:, None] + (c * c).sum(1)[None] - 2 * q @ c.T
+    probes, _ = ix.rank_lists(torch.from_numpy(Q).cuda(), 10)
+    np.testing.assert_array_equal(probes.cpu().numpy(), np.argsort(D, axis=1, kind="stable")[:, :10])
