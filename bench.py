@@ -31,8 +31,9 @@ GRID = (4, 5, 6, 7, 8, 9, 10, 12, 14, 16, 20, 24, 32, 48, 64, 96, 128)
 METRIC = "QPS at recall@10\u22650.90 (1M\u00d7128, 1 GB300) vs plain path; ADC-scan HBM GB/s vs peak"
 TARGET_RECALL = 0.90
 L2_FLUSH_BYTES = 256 << 20
-# DRAM bytes (read + write) of k_scan's two launches in one plain search at the
-# given nprobe, from ncu (profiles/k_scan_ivfpq_sift1m_nq10k_nprobe<P>.md)
+# DRAM bytes (read + write) of k_scan's two launches in one plain search by byte
+# permutes (--lanes 8) at the given nprobe, from ncu
+# (profiles/k_scan_ivfpq_sift1m_nq10k_nprobe<P>.md)
 SCAN_TRAFFIC_BYTES = {7: 186_770_944}
 # the same for the streaming leg of the 10M x 96 index at batch 256, nprobe 256
 # (profiles/k_scan_deep10m_b256_nprobe256.md)
@@ -461,9 +462,12 @@ def run_ours(args, rank, ws):
             if it >= args.warmup:
                 e2e_ms.append(e0.elapsed_time(e1))
     e2e = weak_value(CFG["nq"], ws, max_over_ranks(statistics.mean(e2e_ms), ws))
-    # roofline of the dominant kernel (the LUT16 scan), taken on the plain
-    # step of this run (same kernel; its DRAM traffic was captured with ncu on
-    # that step): lookups per search
+    # roofline of the dominant stage (the LUT16 scan), taken on the plain step of
+    # this run: lookups per search.  Unless lanes are asked for, its filtered part
+    # runs on the tensor cores; the DRAM traffic was captured with ncu on the
+    # byte-permute scan, and is given for that one only.
+    byte_permutes = bool(args.lanes) and not args.scan_tc
+    scan_traffic = SCAN_TRAFFIC_BYTES.get(nprobe) if args.lanes == 8 and byte_permutes and not args.tile_blocks else None
     probes, _ = ix.rank_lists(Qd, nprobe, want_scores=False)
     sizes = np.bincount(ix.export()["assign"], minlength=CFG["nlist"]) if rank == 0 else None
     out = None
@@ -519,30 +523,29 @@ def run_ours(args, rank, ws):
             stream["frac_of_read_stream"] = round(sbytes / (sms * 1e-3) / 1e9 / read_gbs, 4)
         except Exception as ex:  # reported, never fatal
             stream["read_stream_error"] = str(ex)[:200]
-        # the tensor-core scan on the plain step: its results against the
-        # byte-permute scan's and its two scan stages (L2 flushed before each search)
+        # the tensor-core scan and the byte-permute scan on the plain step: equal
+        # results, and the two scan stages of each (L2 flushed before each search)
         tcs = None
         if not args.scan_tc:
             try:
-                to = ksc.search_opts(scan_tc=True)
-                r0 = ix.search(Qd, k, nprobe, R, opts=ksc.search_opts(lanes_per_query=8))
-                r1 = ix.search(Qd, k, nprobe, R, opts=to)
+                ways = {"": ksc.search_opts(scan_tc=True), "byte_permute_": ksc.search_opts(lanes_per_query=8)}
+                r1, r0 = (ix.search(Qd, k, nprobe, R, opts=o) for o in ways.values())
                 same = bool(torch.equal(r0[0], r1[0]) and torch.equal(r0[1], r1[1]))
+                tcs = {"kernel": "k_scan_tc (ksc_search_opts.scan_tc)", "results_equal_byte_permutes": same}
                 ix.profile(True)
-                tn, tsc = [], []
-                for it in range(args.warmup + 5):
-                    flush.zero_()
-                    ix.search(Qd, k, nprobe, R, opts=to)
-                    pp, _ = ix.profile_read()
-                    if it >= args.warmup:
-                        tn.append(pp["near_scan"])
-                        tsc.append(pp["scan"])
+                for name, o in ways.items():
+                    tn, tsc = [], []
+                    for it in range(args.warmup + 5):
+                        flush.zero_()
+                        ix.search(Qd, k, nprobe, R, opts=o)
+                        pp, _ = ix.profile_read()
+                        if it >= args.warmup:
+                            tn.append(pp["near_scan"])
+                            tsc.append(pp["scan"])
+                    tcs[name + "near_scan_ms"] = round(statistics.median(tn), 4)
+                    tcs[name + "scan_ms"] = round(statistics.median(tsc), 4)
                 ix.profile(False)
-                tcs = {"kernel": "k_scan_tc (ksc_search_opts.scan_tc)", "results_equal_plain": same,
-                       "status": ix.last_status(), "near_scan_ms": round(statistics.median(tn), 4),
-                       "scan_ms": round(statistics.median(tsc), 4),
-                       "plain_near_scan_ms": round(plain_stage["near_scan"], 4),
-                       "plain_scan_ms": round(plain_stage["scan"], 4)}
+                tcs["status"] = ix.last_status()
             except Exception as ex:  # reported, never fatal to the benchmark line
                 ix.profile(False)
                 tcs = {"error": str(ex)[:200]}
@@ -627,10 +630,13 @@ def run_ours(args, rank, ws):
             "gpu_launches": launches,
             "search_stats": stats,
             "stage_ms": {s_: round(statistics.mean(v), 4) for s_, v in stage_ms.items()},
-            "roofline": {"bound": "alu", "kernel": "k_scan (LUT16 ADC scan)", "achieved": round(achieved_gl, 1),
+            "roofline": {"bound": "alu" if byte_permutes else "mma latency and issue (filtered part), alu (first part)",
+                         "kernel": "k_scan (LUT16 ADC scan)" if byte_permutes else
+                         "k_scan_tc (filtered part) and k_scan (first part) of the LUT16 ADC scan",
+                         "achieved": round(achieved_gl, 1),
                          "peak": round(peak_gl, 1), "unit": "Glookup/s", "frac": round(achieved_gl / peak_gl, 4),
-                         "peak_source": "measured: ksc_lut16_peak, the scan's shared-selector lookup sequence "
-                                        "with no global memory traffic",
+                         "peak_source": "measured: ksc_lut16_peak, the byte-permute scan's shared-selector lookup "
+                                        "sequence with no global memory traffic (the tensor-core scan is not bound by it)",
                          "peak_per_slot_sequence": round(peak_slot_gl, 1),
                          # the chip's integer-issue bound of that sequence: 64 integer-ALU
                          # lane-operations per clock per SM, 1.156 ALU operations per lookup
@@ -639,9 +645,9 @@ def run_ours(args, rank, ws):
                          "integer_issue_bound": round(64 * 152 * 2.07e9 / (18.5 / 16) / 1e9, 1),
                          "frac_of_integer_issue_bound": round(achieved_gl / (64 * 152 * 2.07e9 / (18.5 / 16) / 1e9), 4),
                          "lookups_per_launch": lookups,
-                         # DRAM read + write of the scan's two launches per search, from the
-                         # ncu capture of the plain step (profiles/k_scan_*.md)
-                         "traffic": None if sopts else SCAN_TRAFFIC_BYTES.get(nprobe),
+                         # DRAM read + write of the byte-permute scan's two launches per search,
+                         # from its ncu capture (profiles/k_scan_*.md)
+                         "traffic": scan_traffic,
                          "step": "plain nprobe %d search of this run" % nprobe,
                          "code_bytes_per_launch": code_bytes,
                          "effective_code_GBps": round(code_bytes / (scan_ms * 1e-3) / 1e9, 1),
@@ -649,8 +655,8 @@ def run_ours(args, rank, ws):
                          # the index's codes once; DRAM traffic above them is candidate keys
                          # and L2 misses of lists re-read by many queries
                          "unique_code_bytes": CFG["n"] * CFG["M"] // 2,
-                         "traffic_over_unique_code_bytes": None if sopts or SCAN_TRAFFIC_BYTES.get(nprobe) is None
-                         else round(SCAN_TRAFFIC_BYTES[nprobe] / (CFG["n"] * CFG["M"] / 2), 2)},
+                         "traffic_over_unique_code_bytes": None if scan_traffic is None
+                         else round(scan_traffic / (CFG["n"] * CFG["M"] / 2), 2)},
             # re-rank of the plain step: R gathered rows of d floats per query
             # (algorithmic bytes; an effective rate, some rows hit L2).  With
             # the band (the default for L2) every candidate is first read as
