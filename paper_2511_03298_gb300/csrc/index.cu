@@ -251,14 +251,6 @@ __device__ __forceinline__ PqRow<DS> pq_load(const float* __restrict__ p) {
     return r;
 }
 
-// (double)x.  This chip converts on its FP64 pipe (two lanes a clock and SM), so
-// a normal number's bits are widened with integer operations instead.
-__device__ __forceinline__ double widen_f32(float x) {
-    const uint32_t u = __float_as_uint(x), e = u & 0x7f800000u;
-    if (e == 0u || e == 0x7f800000u) return (double)x;  // zero, subnormal, infinity, NaN
-    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
-}
-
 template <int DS>
 __device__ __forceinline__ int pq_nearest(const PqRow<DS>& r, const float (&w)[PQ_K][DS]) {
     float best = INFINITY;
@@ -343,7 +335,7 @@ __global__ void __launch_bounds__(256) k_pq_step(const float* __restrict__ R, in
                 const int c = pq_nearest<DS>(x[u], w);
                 mc[c * M] += 1u;
 #pragma unroll
-                for (int t = 0; t < DS; ++t) ms[(c * DS + t) * M] += widen_f32(x[u].v[t]);
+                for (int t = 0; t < DS; ++t) ms[(c * DS + t) * M] += (double)x[u].v[t];
             }
         }
     }
