@@ -1,5 +1,5 @@
-// Lookup, widening and reduction steps of the byte-permute scans (search.cu,
-// scan_r.cu).
+// Lookup, widening and reduction steps of the byte-permute scans (search.cu); the
+// tensor-core scan (scan_tc.cu) splits its tables by the same lookups.
 #pragma once
 
 #include "scan.cuh"
@@ -54,9 +54,6 @@ __device__ __forceinline__ void accum_pair(const uint4& c0, const uint4& t0, con
     }
 }
 
-// Reduce-scatter of the 16 u16x2 sums over the G lanes of a group: after it,
-// group lane g holds the full sums of vectors V*g .. V*g+V-1 (V = 32/G) in
-// out[0..V) (u16 values).
 // The same lookups with the widening done by byte dot products (dp4a with a
 // one-hot byte selector adds byte b of the looked-up word to a 32-bit sum):
 // acc[v] is the sum of vector v.  The dot products issue on the FMA pipe, so
@@ -137,6 +134,9 @@ __device__ __forceinline__ void accum_chunk_sel(const uint4* __restrict__ sel, i
     }
 }
 
+// Reduce-scatter of the 16 u16x2 sums over the G lanes of a group: after it,
+// group lane g holds the full sums of vectors V*g .. V*g+V-1 (V = 32/G) in
+// out[0..V) (u16 values).
 template <int G>
 __device__ __forceinline__ void reduce_scatter(uint32_t (&acc)[16], int lane, uint32_t (&out)[32 / G]) {
     constexpr int V = 32 / G;
@@ -171,9 +171,7 @@ __device__ __forceinline__ void reduce_scatter(uint32_t (&acc)[16], int lane, ui
     }
 }
 
-
 constexpr uint32_t SCAN_WAIT_LIMIT = 1u << 22;
-
 
 // Poll an mbarrier phase at most SCAN_WAIT_LIMIT times; false if it never completed.
 __device__ __forceinline__ bool scan_wait(uint32_t bar, uint32_t parity) {
@@ -188,6 +186,5 @@ __device__ __forceinline__ bool scan_wait(uint32_t bar, uint32_t parity) {
     }
     return false;
 }
-
 
 }  // namespace ksc
