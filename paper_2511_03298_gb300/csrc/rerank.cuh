@@ -57,7 +57,10 @@ __device__ __forceinline__ float rerank_rows8(const float4& qv, const float* __r
 }
 
 
-constexpr int RR_RANK_R = 512;  // keys up to which an order is found by counting ranks
+// Keys up to which an order is found by counting ranks.  (1000 queries of 500k x
+// 64, k 10: at R 257 243 us counted, 207 cut by radix refinement first; at R 512 310
+// and 233; k = R = 400 286 counted, 246 sorted.)
+constexpr int RR_RANK_R = 256;
 
 // Keys of cta_rerank's kbuf: the k best, to a power of two where they are sorted.
 __host__ __device__ inline int rerank_kbuf(int k) { return k > RR_RANK_R ? pow2_ceil(k) : k; }
@@ -72,9 +75,9 @@ inline size_t rerank_smem(int R, int k) {
 // (distance, id) to out_ids / out_d (L2 distance ascending / IP similarity
 // descending).  keys[] is overwritten; kbuf: rerank_kbuf(k) keys when R > RR_RANK_R.
 // Bound by the rows' latency: a warp keeps 8 rows (d <= 128) or 4 in flight;
-// up to 512 candidates are ordered by counting, for each, the smaller ones
+// up to 256 candidates are ordered by counting, for each, the smaller ones
 // (one pass of broadcast reads, no barriers), more are cut to the k best by
-// radix refinement first, and these sorted if they are more than 512 still.
+// radix refinement first, and these sorted if they are more than 256 still.
 template <int NT>
 __device__ __forceinline__ void cta_rerank(uint64_t* keys, int R, uint64_t* kbuf, const float* qs,
                                            const float* __restrict__ X, int d, int ip, int k,

@@ -1,5 +1,5 @@
-"""The CTA re-ranks' order of more than 512 results (sorted in shared memory; up to
-512 counted): around 512 and a power of two, with as many candidates, more and
+"""The CTA re-ranks' order of more than 256 results (sorted in shared memory; up to
+256 counted): around 256, 512 and a power of two, with as many candidates, more and
 fewer than k, FP32 and exact U8 rows, L2 and inner products, small and larger
 batches.  Byte-valued data: distances are whole numbers, the order of (distance,
 id) is known."""
@@ -10,7 +10,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("nq", [5, 330])
-@pytest.mark.parametrize("k,R", [(512, 600), (513, 513), (513, 2000), (1000, 1000), (1024, 1024), (1024, 4096)])
+@pytest.mark.parametrize("k,R", [(10, 256), (10, 257), (256, 300), (257, 257), (300, 600), (512, 600), (513, 513), (513, 2000), (1000, 1000), (1024, 1024), (1024, 4096)])
 @pytest.mark.parametrize("metric,band", [("l2", 0), ("l2", -1), ("ip", 0)])
 def test_order(nq, k, R, metric, band):
     import torch
