@@ -1176,11 +1176,17 @@ __device__ __forceinline__ uint64_t cta_topk(const uint64_t* keys, int n, int K,
 constexpr int SW_WARPS = 8;        // queries per CTA of the warp selection kernels
 constexpr int SW_MAX_KEYS = 2048;  // expected keys per query up to which a warp selects ...
 // ... in batches that fill the GPU; above SW_CTA_KEYS a CTA of 128 threads with its
-// keys in registers.  A warp reads its keys from L2 in each of three passes and
-// more, a CTA once, at the cost of some nine barriers: at R 400 (3001 queries) the
-// search takes 547 us by warps and 498 by CTAs, the hybrid search with 1560 near
-// keys 732 and 705, at R 200 (10,000 queries) 904 and 951.
-constexpr int SW_CTA_KEYS = 1024;
+// keys in registers, in batches that do not give every SM SW_CTA_NQ warps.  A warp
+// reads its keys from L2 in each of three passes and more, a CTA once, at the cost
+// of some nine barriers: the search by warps / CTAs in us at R 400 (3001 queries)
+// 547 / 498, the hybrid search with 1560 near keys 732 / 705, at R 200 (10,000
+// queries) 904 / 951; at R 300 to 512 and nprobe 2 to 48 on three index shapes 3 to 12%
+// faster by CTAs with 1216 queries, 0 to 6% with 3000, 0 to 4% slower with 8000 (500k
+// x 64, R 400, nprobe 8: 678 / 707).
+constexpr int SW_CTA_KEYS = 1024, SW_CTA_NQ = 32;
+static bool select_by_warp(int64_t nq, double keys) {
+    return warp_per_query(nq) && keys <= SW_MAX_KEYS && (keys <= SW_CTA_KEYS || nq >= SW_CTA_NQ * (int64_t)num_sms());
+}
 
 __global__ void __launch_bounds__(SW_WARPS * 32) k_threshold(ScanArgs A, int Rmax, int32_t* __restrict__ cnt,
                                                              uint64_t* __restrict__ cand, int cap,
@@ -3122,7 +3128,7 @@ static int select_stage(ksc_index* ix, const Plan& pl, const ScanArgs& A, const 
         int32_t* redo = (int32_t*)ix->ws_redo.p;
         KSC_CUDA(cudaMemsetAsync(redo, 0, sizeof(int32_t), st));
         // candidates per query: the R kept by the threshold plus a few R more
-        if (4 * pl.Rmax <= SW_CTA_KEYS && warp_per_query(nq)) {
+        if (select_by_warp(nq, 4.0 * pl.Rmax)) {
             k_select<<<(unsigned)((nq + SW_WARPS - 1) / SW_WARPS), SW_WARPS * 32, 0, st>>>(
                 A, pl.Rmax, cnt, cand, pl.cap, topr, ncand_out, ix->status, ix->stats, redo);
         } else {
@@ -3414,7 +3420,7 @@ static int search_from_probes(ksc_index* ix, const float* Q, const Plan& pl, con
     // max(4 R, N / 16), or the hybrid search's near lists
     const double near = pl.hybrid ? (double)rA * ix->n / L
                                   : std::max(4.0 * pl.Rmax, (double)pl.Pmax * ix->n / L / 16.0);
-    if (near <= SW_CTA_KEYS && warp_per_query(nq)) {
+    if (select_by_warp(nq, near)) {
         k_threshold<<<(unsigned)((nq + SW_WARPS - 1) / SW_WARPS), SW_WARPS * 32, 0, st>>>(A, pl.Rmax, cnt, cand,
                                                                                            pl.cap, topr, thr);
     } else {
