@@ -3467,15 +3467,22 @@ static int search_from_probes(ksc_index* ix, const float* Q, const Plan& pl, con
     return rerank_stage(ix, Qr, pl, topr, ids, dists, st);
 }
 
-// The filtered scan takes the tensor cores from this many queries per list (nq P /
-// L) on lists of this many vectors: an item's cost is mostly the expansion of its
+// The filtered scan takes the tensor cores from this many queries per list of its
+// part (nq P / L times the part's share of the keys) on lists of this many
+// vectors: an item's cost is mostly the expansion of its
 // codes, whatever its queries, and the staging of their tables, whatever its
 // vectors.  Search with byte permutes / tensor cores in us, 1M x 64 subspaces in
 // 1024 lists, 7 probed: 224 / 277 at 7 queries per list, 318 / 324 at 14, 396 / 353
 // at 20, 490 / 404 at 28, 976 / 718 at 68; 200k x 48 in 512 lists: 146 / 150 at 16,
 // 203 / 189 at 32, 793 / 613 at 256; in 2048 lists (100 vectors each): 210 / 232 at
-// 16, 531 / 521 at 64.
-constexpr int64_t TC_MIN_SHARE = 20, TC_MIN_LIST = 256;
+// 16, 531 / 521 at 64 (queries per list of the whole search; at nprobe 7 the
+// filtered part has 0.8 of the keys, at nprobe 2 and R 257 of 390-vector lists none,
+// and 8000 queries took 433 / 444 us).
+// Above 96 subspaces an item holds 16 queries only, and takes as long as byte
+// permutes do: from this many vectors of the part's pairs on (128 subspaces, 400
+// queries at nprobe 4 of 100k in 64 lists, 2.0M: 185 / 202; 332 at nprobe 8 of 200k x 128 in
+// 128, 3.7M: 275 / 268; 2500 at nprobe 8 of 300k in 256, 21M: 1037 / 886).
+constexpr int64_t TC_MIN_SHARE = 16, TC_MIN_LIST = 256, TC_MIN_VECTORS_16 = 3'000'000;
 constexpr int SCAN_TC_RULE = 2;  // ksc_search_opts.scan_tc: the rule also where lanes are given
 
 // Tile lengths of the scan's warp items for an expected P probes per query.
@@ -3505,9 +3512,11 @@ static void set_tiles(const ksc_index* ix, Plan& pl, int64_t nq, double P, const
     // tensor-core scan of the filtered part: asked for, or by default where
     // enough queries share a list; tiles of whole 128-vector products, 32 blocks
     // unless given
+    const double tc_pairs = (double)nq * P * (1.0 - near);
     pl.tc = pl.nt > 0 && !pl.hybrid &&
             (pl.tc_opt || ((!(opts && opts->lanes_per_query) || opts->scan_tc == SCAN_TC_RULE) &&
-                           nq * P >= TC_MIN_SHARE * ix->L && ix->n >= TC_MIN_LIST * ix->L));
+                           tc_pairs >= (double)TC_MIN_SHARE * ix->L && ix->n >= TC_MIN_LIST * ix->L &&
+                           (pl.nt >= 32 || tc_pairs * nbar >= (double)TC_MIN_VECTORS_16)));
     if (pl.tc)
         pl.TB = (opts && opts->tile_blocks > 0) ? (std::min(opts->tile_blocks, TCS_MAX_TILE) + 3) / 4 * 4 : 32;
 }

@@ -48,3 +48,15 @@ def test_full_size_workload(ksc):
     X, Q = synth.base(2), synth.queries(2)
     g = ksc.build_index(torch.from_numpy(X).cuda(), 1024, 64, perm=synth.build_perm(2, len(X)))
     _compare(ksc, g, torch.from_numpy(Q).cuda(), 7, 200)
+
+
+@pytest.mark.parametrize("M,ds", [(1, 4), (9, 1), (50, 2), (80, 1), (97, 1), (104, 1), (128, 1)])
+@pytest.mark.parametrize("nq,P", [(16, 5), (17, 5), (700, 5), (600, 2)])
+def test_subspaces_and_groups_asked_for(ksc, M, ds, nq, P):
+    """The largest subspace counts hold 16 queries an item, and small batches take
+    the tensor cores only when asked to."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(M + nq)
+    X = torch.randn(20_000, M * ds, generator=g, device="cuda")
+    ix = ksc.build_index(X, 40, M, iters=2)
+    _compare(ksc, ix, torch.randn(nq, M * ds, generator=g, device="cuda"), P, 60)
