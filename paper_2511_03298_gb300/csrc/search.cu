@@ -3248,9 +3248,9 @@ static int search_small(ksc_index* ix, const float* Q, const Plan& pl, const int
 //    128, one query: 5 us of k_small_prep against 20 us of the three ranking
 //    kernels; at 128 queries those 64 MB take about as long as the tensor
 //    cores' path).
-// One query of 1M x 128 at nprobe 7 from a plan: 97.6 us before, 45.2 now; 100
-// queries of 10k x 128 by direct calls 112.9 and 58.0; 16 queries at nprobe up to
-// 256 and R up to 1000 of 1M x 96 158 and 73.
+// One query of 1M x 128 at nprobe 7 from a plan: 97.6 us before, 49 now; 100
+// queries of 10k x 128 by direct calls 112.9 and 58; 16 queries at nprobe up to
+// 256 and R up to 1000 of 1M x 96 158 and 72.
 //  - all_near: if no query can probe more than SMALL_NEAR_KEYS keys, the store
 //    holds all of them and the threshold, the second scan and its items go.
 //  - pairs of a query and a probed list: with many, the general path's shared
@@ -3315,8 +3315,9 @@ static int search_from_probes(ksc_index* ix, const float* Q, const Plan& pl, con
     if (!Qr) Qr = Q;
     if (pl.small) return search_small(ix, Q, pl, probes, ids, dists, cand_out, ncand_out, st, Qr);
     // queries per work item: the unfiltered first part always runs the
-    // byte-permute scan (few queries share a list there: too few columns for
-    // the tensor cores); the rest the chosen scan
+    // byte-permute scan (the tensor-core scan keeps only filtered keys; with the
+    // part's one or two lists a query, few queries share a list there unless the
+    // index has few lists), the rest the chosen scan
     const int QGa = 32 / pl.G;
     const int QG = pl.tc ? pl.nt : QGa;
     // hybrid: the n_near nearest lists are the fully scanned ones (Sec. 4.4);
