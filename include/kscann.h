@@ -168,7 +168,9 @@ typedef struct {
                                   error); only candidates whose lower bound is at most the k-th
                                   smallest upper bound are read in FP32, so the results are those
                                   of the plain pass; -1 every candidate in FP32; 0 auto: the band
-                                  for L2 indexes.  The copies are made on first use: U8 rows
+                                  for L2 indexes.  The copies are made on first use (in auto, past
+                                  k 32 or d 128, once the handle has re-ranked 16 candidates
+                                  per row, or with a plan): U8 rows
                                   (n d bytes, exact) when every re-rank coordinate is an integer
                                   in [0, 255], else BF16 rows (n d 2 bytes), and two bounds per
                                   row (n 8 bytes).  That first use synchronises the stream once

@@ -1171,6 +1171,7 @@ extern "C" int ksc_index_view(ksc_index* ix, ksc_index** out) {
     }
     v->prof = false;
     v->launches = 0;
+    v->u8_wanted = 0;
     v->status = nullptr;
     v->stats = nullptr;
     cudaError_t e = cudaMalloc(&v->status, STATUS_BYTES);

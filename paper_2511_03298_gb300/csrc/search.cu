@@ -2694,7 +2694,8 @@ struct Plan {
     bool hybrid;
     int n_near, efs, tau;
     int prec, Rf;  // precision variant: first re-rank of R (= Rmax) in prec, then FP32 of the best Rf
-    bool band;     // exact re-rank with the band of U8 / BF16 rows (k_rerank_w)
+    bool band;     // exact re-rank with the band of U8 / BF16 rows (k_rerank_w, k_rerank_u8)
+    bool band_now; // asked for by the caller: its copies are made at once
     int Pq_max;    // bound on the per-query nprobe (<= Pmax)
     double Pexp;   // expected nprobe
     bool tc;       // filtered scan on the tensor cores (k_scan_tc)
@@ -2950,14 +2951,14 @@ static int ensure_u8(ksc_index* ix, cudaStream_t st) {
 // of memory, a synchronisation) costs about what re-ranking 19 candidates per
 // row of the index in bytes saves (60k x 784: 450 us; 10,000 queries of 200
 // candidates 848 -> 477 us), so they are made once the handle has re-ranked
-// U8_AFTER per row, at once for a plan: a program that searches an index a few
-// times does not pay for them.  Not while the stream is captured; where the
+// U8_AFTER per row, at once (`now`) for a plan and for a caller who asks for the
+// band: a program that searches an index a few times does not pay for them.  Not while the stream is captured; where the
 // device has no room, tried again after as many candidates more.
 constexpr int64_t U8_AFTER = 16;
-static bool u8_rows(ksc_index* ix, int64_t rows, cudaStream_t st) {
+static bool u8_rows(ksc_index* ix, int64_t rows, bool now, cudaStream_t st) {
     if (ix->x_u8_state == 0 || ix->x_u8_state == 2) {
         ix->u8_wanted += rows;
-        if (!ix->u8_now && ix->u8_wanted < U8_AFTER * ix->n) return false;
+        if (!now && !ix->u8_now && ix->u8_wanted < U8_AFTER * ix->n) return false;
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
         if (ensure_u8(ix, st) != KSC_OK) {
@@ -3095,7 +3096,7 @@ static int rerank_stage(ksc_index* ix, const float* Qr, const Plan& pl, const ui
         ix->launches++;
         KSC_LAUNCH_CHECK();
     } else if (pl.band && pl.prec == 0 && rr_R > pl.k && ix->metric != KSC_IP && nq >= 2 * (int64_t)num_sms() &&
-               rerank_u8_supported(dr) && u8_rows(ix, nq * rr_R, st)) {
+               rerank_u8_supported(dr) && u8_rows(ix, nq * rr_R, pl.band_now, st)) {
         KSC_TRY(launch_rerank_u8(Qr, nq, Xr, (const uint8_t*)ix->X_u8, dr, rr_keys, rr_R, rr_q, rr_R, pl.k, ids, dists,
                                  st));
         ix->launches++;
@@ -3553,6 +3554,7 @@ static int make_plan(ksc_index* ix, int64_t nq, int k, int Pmax, int Rmax, const
     // real-valued rows the BF16 band is wide against the gaps between the
     // best scores)
     pl.band = opts && opts->rerank_band != 0 ? opts->rerank_band > 0 : ix->metric != KSC_IP;
+    pl.band_now = opts && opts->rerank_band > 0;
     KSC_CHECK_ARG(pl.prec >= 0 && pl.prec <= 2, "precision must be 0 (FP32), 1 (BF16) or 2 (FP8)");
     pl.Rf = pl.Rmax;
     if (pl.prec > 0) {
@@ -4458,6 +4460,7 @@ int ksc_autotune(ksc_index* ix, const float* Q_dev, int64_t nq, int32_t k, int32
     const int TBs[5] = {0, 8, 16, 32, 64};
     ksc_search_opts best = *opts;
     float best_ms = INFINITY;
+    // (lanes alone, whatever an earlier call left in opts: byte permutes.)
     // First what the batch takes by itself, where that is the tensor cores (lanes
     // alone ask for byte permutes): its own lanes for the first part, and
     // scan_tc 2, which leaves the scan to the rule.  (10,000 queries of 1M x 64
@@ -4473,7 +4476,10 @@ int ksc_autotune(ksc_index* ix, const float* Q_dev, int64_t nq, int32_t k, int32
         if (gi >= 0 && (Gs[gi] == 4 ? ix->M > 128 : (ix->M + Gs[gi] - 1) / Gs[gi] > 16)) continue;
         for (int ti = 0; ti < 5 && rc == KSC_OK; ++ti) {
             ksc_search_opts o = gi < 0 ? own : *opts;
-            if (gi >= 0) o.lanes_per_query = Gs[gi];
+            if (gi >= 0) {
+                o.lanes_per_query = Gs[gi];
+                if (o.scan_tc == SCAN_TC_RULE) o.scan_tc = 0;
+            }
             o.tile_blocks = TBs[ti];
             float ms = 0.f, tot = 0.f;
             for (int rep = 0; rep < 4 && rc == KSC_OK; ++rep) {

@@ -47,6 +47,13 @@ def test_lanes_elsewhere(env, nq, ask):
     assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
 
 
+def test_tuned_options_tuned_again(env):
+    ksc, ix, Q = env
+    opts, _ = ix.autotune(Q, 10, 8, 200)
+    again, _ = ix.autotune(Q[:1000].contiguous(), 10, 3, 100, opts=opts)  # a batch that takes byte permutes
+    assert again.scan_tc == 0 and again.lanes_per_query in (4, 8, 16, 32)
+
+
 def test_bad_arguments_are_refused(env):
     ksc, ix, Q = env
     for k, P, R in ((0, 8, 200), (10, 0, 200), (10, 257, 200), (10, 8, 5000)):

@@ -1,6 +1,6 @@
 """When the exact re-rank's U8 copies are made: not by the first searches of an
 index, whose saving would not pay for them, but once a handle has re-ranked 16
-candidates per row, and by a plan's creation (told by the device memory taken:
+candidates per row, by a plan's creation and when the band is asked for (told by the device memory taken:
 102 MB of copies); the results are those of the FP32 rows throughout.  Where the
 device has no room for them the search goes on without, and they are made later."""
 import ctypes as C
@@ -61,6 +61,18 @@ def test_made_for_a_plan(env):
         plan, taken = _taken(torch, lambda: v.plan(400, 10, nprobe=4, rerank=100, stream=st))
         got = plan.execute(q, stream=st)
     st.synchronize()
+    assert taken > 90 * MB
+    assert torch.equal(got[0], ref[0]) and torch.equal(got[1], ref[1])
+
+
+@pytest.mark.parametrize("nq,R", [(400, 51), (304, 200)])
+def test_made_when_asked_for(env, nq, R):
+    torch, ksc, ix, Q = env
+    v = ix.view()
+    q = Q[:nq].contiguous()
+    ref = v.search(q, 10, 4, R, opts=ksc.search_opts(rerank_band=-1))
+    v.search(q, 10, 4, R)
+    got, taken = _taken(torch, lambda: v.search(q, 10, 4, R, opts=ksc.search_opts(rerank_band=1)))
     assert taken > 90 * MB
     assert torch.equal(got[0], ref[0]) and torch.equal(got[1], ref[1])
 
